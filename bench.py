@@ -272,7 +272,7 @@ def run_reference(args):
 
 # bound of each kernel class (see the design doc's kernel table): the tensor-core GEMM by the
 # tensor pipe, the CUDA-core GEMM by its arithmetic units, everything else by HBM
-CLASS_KERNEL = {"build": "k_build", "rows": "k_rows / k_outs / k_seg (fused permute-and-contract)",
+CLASS_KERNEL = {"build": "k_build", "rows": "k_rows / k_outs / k_waves / k_wave_wide (fused permute-and-contract)",
                 "splitk": "k_splitk", "results": "k_slice_result / k_sum_slices",
                 "gemm": "k_gemm (tiled strided complex GEMM, CUDA cores)",
                 "gemm_tc": "k_gemm_tc (complex GEMM on tcgen05 tensor cores, BF16 digit products)",

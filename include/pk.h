@@ -142,9 +142,9 @@ typedef struct {
   uint64_t workspace_c128;   /* device workspace bytes for PK_C128                          */
   uint64_t workspace_c64;    /* device workspace bytes for PK_C64                           */
   uint64_t workspace_split;  /* device workspace bytes for PK_SPLIT                         */
-  int32_t n_segments;        /* runs of consecutive small steps launched as one sequence
-                                kernel (one CTA, a block barrier between steps)              */
-  int32_t n_segment_steps;   /* steps inside those runs                                     */
+  int32_t n_segments;        /* PK_C128: launches that run several small steps (whole levels
+                                of the contraction tree) at once                             */
+  int32_t n_segment_steps;   /* steps inside those launches                                 */
   double est_cost;           /* the planner's estimated cost of the chosen sequence, all
                                 slices (the ranking's units: row-kernel multiply-adds)        */
 } pk_plan_stats;
@@ -159,9 +159,10 @@ typedef struct {
   int32_t batch_threads;     /* threads per CTA of the batch executor: 128, 256 or 512       */
   int32_t batch_ktab;        /* batch executor: contracted-index offsets of a step kept in
                                 shared memory (steps with longer K recompute them): 256..2048 */
-  int64_t seq_outs;          /* runs of small steps launched as one sequence kernel: outputs
-                                per step at most (1..65536)                                   */
-  int64_t seq_work;          /* ... complex multiply-adds per step at most (1..2^24)          */
+  int64_t seq_outs;          /* small steps, run together level by level: outputs per step at
+                                most (1..65536; 65536: as many as the level kernels take)     */
+  int64_t seq_work;          /* ... complex multiply-adds per step at most (1..2^24; 16 times
+                                as many for a contracted extent above 32)                     */
   int64_t seq_k;             /* ... contracted extent per step at most (1..2048)              */
   int64_t tc_min_k;          /* PK_SPLIT: row steps of GEMM shape (M >= 64, N >= tc_min_n)
                                 with this contracted extent or more run on the tensor cores
@@ -309,7 +310,7 @@ pk_status pk_upload(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_wo
                     uint64_t workspace_bytes);
 /* As pk_upload, but only the knot-derived part of the program: the initial-tensor recipes
  * and their slots (the program's first bytes).  The plan's other records (conversion and
- * sequence-kernel step records) stay as an earlier pk_upload of this plan and precision
+ * level records) stay as an earlier pk_upload of this plan and precision
  * left them in the same workspace, which the caller must have done (not checked).  For
  * repeated evaluations of the same plan.  *copied (may be NULL): the bytes copied. */
 pk_status pk_upload_inputs(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_workspace,
@@ -358,7 +359,7 @@ pk_status pk_plan_debug_blob(const pk_plan* p, int32_t which, void* dst, uint64_
 /* Runs the kernels of pk_launch once (same stream, same workspace, recipe already
  * uploaded; d_arena NULL = the arena inside the workspace, else as pk_launch_arena)
  * with a CUDA event pair around every launch, waits, and returns per kernel
- * class c (0 build, 1 rows: row, thread-per-output and sequence kernels, 2 split-K,
+ * class c (0 build, 1 rows: row, thread-per-output and level kernels, 2 split-K,
  * 3 results, 4 GEMM on CUDA cores, 5 GEMM on the tensor cores, 6 digit conversion for
  * the tensor-core GEMM): out[c] = milliseconds, out[7+c] = launches, out[14+c] =
  * algorithmic complex multiply-adds, out[21+c] = algorithmic bytes (|A| + |B| + |C| at
@@ -458,7 +459,8 @@ pk_status pk_plan_launches(const pk_plan* p, int32_t precision, int64_t* launche
  * of 64 MiB (67108864 bytes) that every GPU loading the library holds until exit; no
  * cudaMalloc, cudaFree or other allocating routine is called.  Plans whose
  * pk_plan_workspace_bytes exceeds 64 MiB are refused with PK_ENOMEM and a message in
- * pk_last_error.  The first call on a device looks up the array's device address
+ * pk_last_error, except that a plan which exceeds it only by running its small steps level by
+ * level runs here on the tighter layout of its steps' own order.  The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress, with that device current) and caches it: make that first call
  * before any stream capture.  All calls on a device share the array, which keeps the
  * previous call's contents (each call re-uploads its program and clears its bookkeeping);
@@ -587,7 +589,8 @@ pk_status pk_ctx_set_debug(pk_ctx* ctx, int32_t flags);
  * runs, and in the GEMM view C's runs) enumerate the operand's dense tensor exactly once
  * with extents R, K, N (Bsz, M); each step reads live tensors and writes its own; every
  * tensor lies inside the arena on a 512-byte boundary, and tensors live at the same step do
- * not overlap; sequence-kernel records equal their steps; the complex128 tail, the split
+ * not overlap; the level schedule's units, replayed over its own layout, read what they should
+ * and overwrite nothing still needed; the complex128 tail, the split
  * precision's digit scratch, the reverse program (PK_FLAG_GRAD) and the state records fit
  * the workspace of pk_plan_workspace_bytes.  PK_EINVAL with the first violation in msg
  * (NUL-terminated, at most msg_bytes; msg may be NULL). */

@@ -6,7 +6,7 @@ before every timed launch, the fastest median kept:
 * batch executor (`pk_batch_*`, one persistent launch for many knots): threads per CTA
   x contracted-index offsets kept in shared memory, on the 4096-knot batch workload
   (q = 3, split precision);
-* sequence runs (consecutive small steps of a plan launched as one one-CTA kernel): the
+* level launches (small steps of a plan run together, level by level): the
   largest step, in outputs and in complex multiply-adds, that joins a run, on the 64-knot
   scale workload (q = 2, 3, 5; 192 plans replayed as one concurrent graph, split);
 * the smallest contracted extent and column count from which row steps of GEMM shape
@@ -41,8 +41,8 @@ REFINE = 8       # subtree reconfiguration of the scale workload's plans, as ben
 
 BATCH_THREADS = (128, 256, 512)
 BATCH_KTAB = (512, 1024, 2048)
-SEQ_OUTS = (1024, 2048, 4096, 8192)
-SEQ_WORK = (1 << 12, 1 << 14, 1 << 16)
+SEQ_OUTS = (1024, 8192, 65536)
+SEQ_WORK = (1 << 16, 1 << 18, 1 << 20, 1 << 22)
 TC_MIN_K = (4, 8, 16)
 TC_DB_GROUPS = (0, 2, 3, 4, 6)
 TC_MIN_N = (8, 12, 16, 24, 32)
@@ -120,8 +120,8 @@ def sweep_seq(pk, ctx, stream, flush, reps, log, quick):
     kn = [pk.Knot.from_pd(ctx, k.pd, outer=k.outer) for k in knots]
     jobs = [(k, q) for k in kn for q in (2, 3, 5)]
     rows, ref, best = [], None, None
-    outs = SEQ_OUTS if not quick else (2048, 4096)
-    works = SEQ_WORK if not quick else (1 << 12, 1 << 14)
+    outs = SEQ_OUTS if not quick else (8192, 65536)
+    works = SEQ_WORK if not quick else (1 << 18, 1 << 20)
     for so in outs:
         for sw in works:
             ctx.set_tuning(seq_outs=so, seq_work=sw)
@@ -141,7 +141,7 @@ def sweep_seq(pk, ctx, stream, flush, reps, log, quick):
             ok = err <= 1e-6
             launches = sum(p.launches("split") for p in plans)
             rows.append((so, sw, ms, ok, launches))
-            log(f"sequence runs outs<={so} work<={sw}: {ms:.2f} ms per step, {launches} launches"
+            log(f"level launches outs<={so} work<={sw}: {ms:.2f} ms per step, {launches} launches"
                 f"{'' if ok else ' RESULTS DIFFER'}")
             if ok and (best is None or ms < best[2]):
                 best = (so, sw, ms)
@@ -203,7 +203,7 @@ def write_table(path, tune, batch_rows, seq_rows, gpu, param_rows):
              "// Batch executor, 4096 knots at q = 3, split, one launch (median ms):"]
     for th, kt, ms, ok in batch_rows:
         lines.append(f"//   threads {th:4d}  ktab {kt:5d}  {ms:8.3f}{'' if ok else '  (results differ)'}")
-    lines.append("// Sequence runs, 192 evaluations of the scale workload, split (median ms per step):")
+    lines.append("// Level launches, 192 evaluations of the scale workload, split (median ms per step):")
     for so, sw, ms, ok, nl in seq_rows:
         lines.append(f"//   outs <= {so:5d}  work <= {sw:6d}  {ms:8.2f}  ({nl} launches)"
                      f"{'' if ok else '  (results differ)'}")

@@ -25,7 +25,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # same on x86-64 and aarch64 hosts
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O3,-ffp-contract=off", "-I", INCLUDE, "-I", CSRC,
          "--expt-relaxed-constexpr"]
-SOURCES = ["knot.cpp", "plan.cpp", "grad_plan.cpp", "jones_exact.cpp", "verify.cpp", "launch.cu",
+SOURCES = ["knot.cpp", "plan.cpp", "grad_plan.cpp", "wave_plan.cpp", "jones_exact.cpp", "verify.cpp", "launch.cu",
            "api.cu", "noalloc.cu", "batch.cu", "exact.cu"]
 
 

@@ -88,7 +88,7 @@ pk_status launch_recorded(pk_ctx* ctx, const pk_plan* p, int32_t precision, void
     cudaError_t e = pk::launch_plan_opts(P, precision, ws, arena, ctx->stream, o);
     return e == cudaSuccess ? PK_OK : cuda_fail(ctx, e, "launch");
   }
-  const double nodes = (double)P.n_slices * (double)(P.steps.size() + 4);
+  const double nodes = (double)P.n_slices * (double)(P.wave.stages[precision == PK_C128].size() + P.n_tc + 4);
   if (nodes > 20000.0) {
     cudaError_t e = pk::launch_plan(P, precision, ws, arena, ctx->stream);
     return e == cudaSuccess ? PK_OK : cuda_fail(ctx, e, "launch");
@@ -382,8 +382,11 @@ pk_status pk_plan_create(pk_ctx* ctx, const pk_knot* k, int32_t q, const pk_plan
       return fail(ctx, PK_EINVAL, err);
     }
     const pk::Plan& P = p->p;
-    const uint64_t need = std::max(P.ws_bytes(PK_C128), std::max(P.ws_bytes(PK_SPLIT), P.ws_bytes(PK_C64)));
-    if (budget == 0 || need <= budget) break;
+    auto need = [&] { return std::max(P.ws_bytes(PK_C128), std::max(P.ws_bytes(PK_SPLIT), P.ws_bytes(PK_C64))); };
+    if (budget == 0 || need() <= budget) break;
+    // the level schedule on the layout of the steps' own order, before slicing further
+    pk::plan_waves(p->p, true);
+    if (need() <= budget) break;
     // over the device-memory budget: one index fewer on the largest tensor (more slices)
     const double lq = std::log2((double)q);
     if (q < 2 || P.max_rank <= 1) {
@@ -415,10 +418,8 @@ pk_status pk_plan_info(const pk_plan* p, pk_plan_stats* out) {
   out->workspace_c128 = P.ws_bytes(PK_C128);
   out->workspace_c64 = P.ws_bytes(PK_C64);
   out->workspace_split = P.ws_bytes(PK_SPLIT);
-  int32_t seg_steps = 0;
-  for (const pk::Segment& g : P.segments) seg_steps += g.count;
-  out->n_segments = (int32_t)P.segments.size();
-  out->n_segment_steps = seg_steps;
+  out->n_segments = P.wave.n_fused[1];
+  out->n_segment_steps = P.wave.n_fused_steps[1];
   out->est_cost = P.est_cost;
   return PK_OK;
 }
@@ -514,10 +515,13 @@ pk_status pk_plan_launches(const pk_plan* p, int32_t precision, int64_t* launche
   if (!p || !launches || !valid_precision(precision)) return PK_EINVAL;
   const pk::Plan& P = p->p;
   const int64_t widen = (precision == PK_C64 && !P.conv.empty()) ? 1 : 0;
-  const int64_t digits = precision == PK_SPLIT ? (int64_t)P.n_tc : 0;  // one conversion launch per tensor-core step
-  int64_t fused = 0;  // steps saved by sequence launches (runs of small steps)
-  for (const pk::Segment& g : P.segments)
-    if (precision != PK_C64 || g.first + g.count <= P.tail_first) fused += g.count - 1;
+  int64_t digits = 0;   // split precision: one conversion launch per tensor-core step
+  if (precision == PK_SPLIT)
+    for (const pk::WaveStage& g : P.wave.stages[0])
+      digits += g.kind == pk::WaveStage::STEP && P.steps[g.step].tc;
+  // steps saved by the level launches (a complex128 tail's steps are never inside one)
+  const int fp64 = precision == PK_C128;
+  const int64_t fused = P.wave.n_fused_steps[fp64] - P.wave.n_fused[fp64];
   *launches = P.n_slices * ((P.n_init > 0 ? 1 : 0) + (int64_t)P.steps.size() - fused + 1 + widen +
                             digits) + 1;
   return PK_OK;
@@ -569,7 +573,7 @@ pk_status pk_upload_inputs(pk_ctx* ctx, const pk_plan* p, int32_t precision, voi
     s = fail(ctx, PK_ENOMEM, "buffer smaller than the plan state (pk_plan_state_bytes)");
   if (s != PK_OK) return s;
   const pk::Plan& P = p->p;
-  // recipes and slots lie first in the program, the conversion and sequence records after
+  // recipes and slots lie first in the program, the conversion and level records after
   const uint64_t n = std::min<uint64_t>(P.off_conv, P.program.size());
   if (copied) *copied = n;
   if (n == 0) return PK_OK;
@@ -1016,7 +1020,7 @@ namespace {
 // (many slices) are launched directly.
 cudaError_t launch_grad_recorded(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* ws) {
   const pk::Plan& P = p->p;
-  const double nodes = (double)P.n_slices * (double)(P.grad.steps.size() + 4);
+  const double nodes = (double)P.n_slices * (double)(P.grad.wave.stages[precision == PK_C128].size() + 4);
   if (nodes > 20000.0) return pk::launch_grad(P, precision, ws, ctx->stream);
   PlanGraph& g = const_cast<pk_plan*>(p)->grad_graph;
   if (!(g.exec && g.ws == ws && g.precision == precision)) {

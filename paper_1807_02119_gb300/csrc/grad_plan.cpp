@@ -43,6 +43,7 @@ struct Op {
   Step st;
   int32_t in_a, in_b, out;  // instance ids (in_b = -1: the constant 1)
   int8_t phase;             // 0 forward, 1 recompute, 2 adjoint
+  int32_t after;            // recompute: the operation that forms its region's adjoint (-1: none)
 };
 
 uint64_t a256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
@@ -126,12 +127,13 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
     inst[st.c].born = inst[st.c].dies = t;
     use(st.a, t);
     use(st.b, t);
-    ops.push_back({st, st.a, st.b, st.c, 0});
+    ops.push_back({st, st.a, st.b, st.c, 0, -1});
   }
 
   // reverse pass, region by region from the root down
   std::vector<int32_t> cur(n_tens), adj(n_tens, -2);  // adj: -1 constant 1, -2 not yet formed
   std::iota(cur.begin(), cur.end(), 0);
+  std::vector<int32_t> adj_op(n_tens, -1);                  // operation that formed adj
   adj[root] = -1;
   std::vector<int32_t> heads;
   for (int32_t X = p.n_init; X < n_tens; ++X)
@@ -151,7 +153,7 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
       st.c = inst[id].meta;
       use(cur[A], t);
       if (B >= 0) use(cur[B], t);
-      ops.push_back({st, cur[A], B >= 0 ? cur[B] : -1, id, 1});
+      ops.push_back({st, cur[A], B >= 0 ? cur[B] : -1, id, 1, adj_op[X]});
       cur[C] = id;
     }
     for (auto it = R.rbegin(); it != R.rend(); ++it) {  // adjoint steps
@@ -165,6 +167,7 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
       }
       if (B < 0) {  // C = sum A: the adjoint of A is C' (constant along the summed indices)
         adj[A] = Xb;
+        adj_op[A] = adj_op[C];
         continue;
       }
       for (int side = 0; side < 2; ++side) {
@@ -196,8 +199,9 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
         st.c = inst[id].meta;
         use(ia, t);
         use(ib, t);
-        ops.push_back({st, ia, ib, id, 2});
+        ops.push_back({st, ia, ib, id, 2, -1});
         adj[T] = id;
+        adj_op[T] = (int32_t)ops.size() - 1;
       }
     }
   }
@@ -212,36 +216,70 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
   }
 
   // arena: first fit by decreasing size over lifetime intervals
-  std::vector<int32_t> ord(inst.size());
-  std::iota(ord.begin(), ord.end(), 0);
-  std::sort(ord.begin(), ord.end(), [&](int32_t x, int32_t y) {
-    if (inst[x].elems != inst[y].elems) return inst[x].elems > inst[y].elems;
-    return x < y;
-  });
-  struct Placed {
-    int64_t off, len;
-    int32_t born, dies;
-  };
-  std::vector<Placed> placed;
-  int64_t top = 0;
-  for (int32_t id : ord) {
-    Inst& in = inst[id];
-    const int64_t len = (in.elems + 63) / 64 * 64;
-    std::vector<std::pair<int64_t, int64_t>> busy;
-    for (const auto& pl : placed)
-      if (!(pl.dies < in.born || in.dies < pl.born)) busy.push_back({pl.off, pl.off + pl.len});
-    std::sort(busy.begin(), busy.end());
-    int64_t off = 0;
-    for (const auto& iv : busy) {
-      if (off + len <= iv.first) break;
-      off = std::max(off, iv.second);
-    }
-    in.off = off;
-    placed.push_back({off, len, in.born, in.dies});
-    top = std::max(top, off + len);
+  std::vector<int64_t> elems, seq_off;
+  std::vector<int32_t> born, dies;
+  for (const Inst& in : inst) {
+    elems.push_back(in.elems);
+    born.push_back(in.born);
+    dies.push_back(in.dies);
   }
-  G.arena_elems = top;
+  const int64_t top = first_fit(elems, born, dies, seq_off);
   G.n_meta = next_meta;
+
+  // level schedule.  Running the recomputation as early as its checkpoints allow would keep
+  // every intermediate alive at once, so with checkpoints it waits for its region's adjoint;
+  // the first schedule within the memory limit wins, down to one heavy step at a time and to
+  // the operations' own layout.
+  {
+    const int32_t no = (int32_t)ops.size(), ni = (int32_t)inst.size();
+    std::vector<Step> st(no);
+    std::vector<char> pinned(ni, 0);
+    for (int32_t i = 0; i < no; ++i) {
+      st[i] = ops[i].st;
+      st[i].tc = 0;   // the reverse program keeps its GEMM steps on the CUDA cores
+      st[i].a = ops[i].in_a;
+      st[i].b = ops[i].in_b;
+      st[i].c = ops[i].out;
+    }
+    for (int32_t i = 0; i < ni; ++i) pinned[i] = inst[i].dies == END;
+    WaveProgram& w = G.wave;
+    w.n_init = 0;   // the program's recipes carry their offsets
+    const int64_t limit = 2 * top <= (1 << 26) ? 2 * top : top;   // growth up to 1 GiB in all
+    std::vector<std::pair<int32_t, int32_t>> held, edges;
+    for (int32_t i = 0; i < no; ++i)
+      if (ops[i].after >= 0) held.push_back({ops[i].after, i});
+    for (int breadth = 1; breadth >= 0; --breadth) {
+      wave_schedule(st, ni, tune, breadth != 0, &held, no, w.units);
+      w.arena_elems = wave_layout(st, elems, pinned, w.units, w.off);
+      if (w.arena_elems <= limit) break;
+      w.off.clear();
+    }
+    if (w.off.empty()) {
+      w.off = seq_off;
+      w.arena_elems = top;
+      wave_hazards(st, elems, w.off, edges);
+      wave_schedule(st, ni, tune, false, &edges, no, w.units);
+    }
+    // the operations in launch order, on the schedule's offsets; bookkeeping slots in a, b, c
+    std::vector<Op> sorted;
+    std::vector<int64_t> off = w.off;
+    for (WaveUnit& u : w.units)
+      for (int32_t& i : u.steps) {
+        sorted.push_back(ops[i]);
+        i = (int32_t)sorted.size() - 1;
+      }
+    ops.swap(sorted);
+    std::vector<Step> by_meta;
+    w.off.assign(G.n_meta, 0);
+    for (int32_t i = 0; i < ni; ++i) {
+      inst[i].off = off[i];
+      w.off[inst[i].meta] = off[i];
+    }
+    for (const Op& op : ops) by_meta.push_back(op.st);
+    for (Step& x : by_meta) x.tc = 0;
+    G.arena_elems = w.arena_elems;
+    wave_stages(by_meta, w);
+  }
 
   // steps with their offsets
   for (Op& op : ops) {
@@ -287,9 +325,6 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
     G.leaves.push_back(L);
   }
 
-  // runs of small steps as sequence launches
-  build_segments(G.steps, tune, G.segments, G.tiny);
-
   // workspace layout
   const uint64_t nl = std::max<size_t>(1, G.leaves.size());
   uint64_t off = 0;
@@ -299,8 +334,8 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
   off = a256(off + sizeof(Slot) * std::max<size_t>(1, p.slots.size()));
   G.off_leaves = off;
   off = a256(off + sizeof(GradLeaf) * nl);
-  G.off_tiny = off;
-  off = a256(off + sizeof(TinyStep) * G.tiny.size());
+  G.off_wave = off;
+  off = a256(off + G.wave.blob.size());
   G.off_meta = off;
   off = a256(off + 16ull * (uint64_t)G.n_meta);
   G.off_counter = off;
@@ -319,8 +354,8 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
     std::memcpy(G.program.data() + G.off_slots, p.slots.data(), sizeof(Slot) * p.slots.size());
   if (!G.leaves.empty())
     std::memcpy(G.program.data() + G.off_leaves, G.leaves.data(), sizeof(GradLeaf) * G.leaves.size());
-  if (!G.tiny.empty())
-    std::memcpy(G.program.data() + G.off_tiny, G.tiny.data(), sizeof(TinyStep) * G.tiny.size());
+  if (!G.wave.blob.empty())
+    std::memcpy(G.program.data() + G.off_wave, G.wave.blob.data(), G.wave.blob.size());
   G.built = true;
   return true;
 }

@@ -42,7 +42,7 @@ struct pk_plan {
 
 namespace pk {
 // Kernel classes of the launch-sequence timing: build, rows (row / thread-per-output /
-// sequence kernels), split-K, results, GEMM on the CUDA cores, tensor-core GEMM, digit
+// level kernels), split-K, results, GEMM on the CUDA cores, tensor-core GEMM, digit
 // conversion for the tensor-core GEMM.
 constexpr int kNumClasses = 7;
 // Per-launch CUDA events of one recorded launch sequence (launch.cu).

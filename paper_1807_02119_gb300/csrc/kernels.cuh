@@ -93,7 +93,7 @@ __device__ __forceinline__ Cx<ff> ld(const Cx<ff>* p) {
   float4 v = __ldg(reinterpret_cast<const float4*>(p));
   return {{v.x, v.y}, {v.z, v.w}};
 }
-// Coherent loads (plain ld.global): for data the same kernel wrote earlier, which the
+// Coherent loads (plain ld.global): for data the same CTA wrote earlier, which the
 // read-only path of __ldg does not guarantee to see.
 __device__ __forceinline__ Cx<double> ldc(const Cx<double>* p) {
   double2 v = *reinterpret_cast<const double2*>(p);
@@ -273,13 +273,15 @@ __device__ __forceinline__ void recipe_value(const Recipe& r, const Slot* slots,
 }
 
 // One grid row (blockIdx.y) per initial tensor, formed in double and rounded once to
-// the storage type.
+// the storage type; offs: its place under the level schedule (NULL: the recipe's own).
 template <typename R>
 __global__ void __launch_bounds__(256) k_build(const Recipe* __restrict__ rec,
-                                               const Slot* __restrict__ slots, Cx<R>* arena,
+                                               const Slot* __restrict__ slots,
+                                               const int64_t* __restrict__ offs, Cx<R>* arena,
                                                Meta* meta, int q, long long slice, int n_sliced) {
   using S = typename Traits<R>::S;
   const Recipe r = rec[blockIdx.y];
+  Cx<R>* dst = arena + (offs ? (long long)offs[blockIdx.y] : (long long)r.offset);
   S vmax = 0;
   int sdig[64];
   {
@@ -294,7 +296,7 @@ __global__ void __launch_bounds__(256) k_build(const Recipe* __restrict__ rec,
     double sre, sim;
     recipe_value(r, slots, e, q, sdig, sre, sim);
     const Cx<R> v{from_double<R>(sre), from_double<R>(sim)};
-    st(arena + r.offset + e, v);
+    st(dst + e, v);
     vmax = fmax(vmax, mag(v));
   }
   block_max_to_meta(vmax, meta + r.meta);
@@ -459,59 +461,6 @@ __global__ void __launch_bounds__(256) k_outs(const Step s, Cx<R>* arena, Meta* 
     vmax = fmax(vmax, mag(v));
   }
   block_max_to_meta(vmax, meta + s.c);
-}
-
-// Consecutive small steps of one plan in one CTA: each step's outputs spread over the
-// threads, a block barrier between steps, its max-abs formed by a block reduction.
-// Operands written by earlier steps of the same launch are read with coherent loads
-// (the writes are visible to the CTA after the barrier).
-template <typename R>
-__global__ void __launch_bounds__(256) k_seg(const TinyStep* __restrict__ steps, int n,
-                                             Cx<R>* arena, Meta* meta) {
-  using S = typename Traits<R>::S;
-  __shared__ long long kA[kTinyK], kB[kTinyK];
-  __shared__ S red[32];
-  for (int i = 0; i < n; ++i) {
-    const TinyStep& s = steps[i];
-    const int ea = bin_exp(bits_to_val<S>(meta[s.a].maxbits));
-    const bool hasB = s.b >= 0;
-    const int eb = hasB ? bin_exp(bits_to_val<S>(meta[s.b].maxbits)) : 0;
-    const long long exp_c = meta[s.a].exp + (hasB ? meta[s.b].exp : 0) + ea + eb;
-    const S scale = (S)ldexp(1.0, -(ea + eb));
-    for (long long k = threadIdx.x; k < s.K; k += blockDim.x) split_runs32((unsigned)k, s.kr, s.nk, kA[k], kB[k]);
-    __syncthreads();
-    const Cx<R>* A = arena + s.off_a;
-    const Cx<R>* B = arena + s.off_b;
-    Cx<R>* C = arena + s.off_c;
-    const unsigned outs = (unsigned)(s.R * s.N), R_ = (unsigned)s.R;
-    const int K = (int)s.K;
-    S vmax = 0;
-    for (unsigned o = threadIdx.x; o < outs; o += blockDim.x) {
-      const unsigned nn = o / R_, r = o - nn * R_;
-      long long oa, ob, d, nb = 0;
-      split_runs32(r, s.row, s.nrow, oa, ob);
-      if (hasB) split_runs32(nn, s.nr, s.nn, d, nb);
-      Acc<R> acc;
-      if (hasB) {
-        for (int k = 0; k < K; ++k) acc.mac(ldc(A + oa + kA[k]), ldc(B + ob + nb + kB[k]));
-      } else {
-        for (int k = 0; k < K; ++k) acc.add(ldc(A + oa + kA[k]));
-      }
-      const Cx<R> v = acc.get(scale);
-      st(C + o, v);
-      vmax = fmax(vmax, mag(v));
-    }
-    for (int off = 16; off > 0; off >>= 1) vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, off));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = vmax;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      S m = 0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, red[w]);
-      meta[s.c].maxbits = m > S(0) ? max_bits(m) : 0ull;
-      meta[s.c].exp = exp_c;
-    }
-    __syncthreads();
-  }
 }
 
 // Same contraction without offset tables (K too long for shared memory): every k

@@ -17,6 +17,7 @@
 #include "handles.h"
 #include "kernels.cuh"
 #include "gemm_tc.cuh"
+#include "wave.cuh"
 
 namespace pk {
 
@@ -292,7 +293,53 @@ double step_bytes(const Plan& p, const Step& s, double elem_bytes) {
                                p.tensors[s.c].elems);
 }
 
-// Steps [first, last) of the plan, all in storage type R.
+constexpr uint32_t kWaveSmem = 100 * 1024;   // a level launch's records in shared memory: two CTAs per SM
+
+// One launch of the level schedule `w` (records at `blob` on the device); `steps` are the
+// steps it orders, its heavy ones launched alone on their offsets under the schedule.
+template <typename R>
+cudaError_t launch_stage(const WaveProgram& w, const WaveStage& g, const std::vector<Step>& steps,
+                         const unsigned char* blob, Cx<R>* arena, Meta* meta, Cx<double>* partial,
+                         unsigned* counters, unsigned char* tcs, unsigned long long* err, int64_t db_groups,
+                         cudaStream_t stream, Marker& mk, double cm, double by) {
+  mk.step = g.step;
+  if (g.kind == WaveStage::STEP) {
+    Step s = steps[g.step];
+    s.off_a = w.off[s.a];
+    s.off_b = s.b >= 0 ? w.off[s.b] : 0;
+    s.off_c = w.off[s.c];
+    return launch_step<R>(s, arena, meta, partial, counters + g.step, stream, mk, by, tcs, err, db_groups);
+  }
+  if (g.kind == WaveStage::WIDE) {
+    // few warps per CTA while that spreads the level over more multiprocessors
+    const int64_t wpb = std::max<int64_t>(1, std::min<int64_t>(8, g.items / (2LL * g_sms)));
+    const unsigned grid = (unsigned)((g.items + wpb - 1) / wpb);
+    mk.begin(1, cm, by, gpu_fill(grid, 8));
+    k_wave_wide<R><<<grid, 32 * (unsigned)wpb, 0, stream>>>(blob, g.range, g.first, (unsigned)g.items, arena, meta);
+    mk.end();
+    return cudaGetLastError();
+  }
+  mk.begin(1, cm, by, gpu_fill(g.ctas, 2));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)g.ctas);
+  cfg.blockDim = dim3(32 * kWaveCtaWarps);
+  cfg.stream = stream;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)g.ctas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  const uint32_t prog = g.range.rec_bytes + g.range.item_bytes + g.range.lev_bytes;
+  const int smem = prog <= kWaveSmem ? (int)prog : 0;
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k_waves<R>, blob, g.range, (int)g.units, smem, arena, meta);
+  mk.end();
+  return e;
+}
+
+// Steps [first, last) of the plan, all in storage type R: through the level schedule, or (the
+// finite check) one at a time in their own order.
 template <typename R>
 cudaError_t launch_bulk(const Plan& p, char* base, char* arena_base, int32_t first, int32_t last,
                         cudaStream_t stream, Marker& mk, const LaunchOpts& o, long long sl) {
@@ -302,37 +349,33 @@ cudaError_t launch_bulk(const Plan& p, char* base, char* arena_base, int32_t fir
   unsigned* counters = (unsigned*)(base + p.off_counter);
   unsigned char* tcs = (std::is_same<R, ff>::value && p.tc_bytes > 0)
                            ? (unsigned char*)arena_base + p.tc_offset() : nullptr;
-  const TinyStep* tiny = (const TinyStep*)(base + p.off_tiny);
   unsigned long long* err = &((SliceResult*)(base + p.off_result))[p.n_slices].status;
-  size_t sg = 0;
-  for (int32_t i = first; i < last;) {
-    while (sg < p.segments.size() && p.segments[sg].first < i) ++sg;
-    if (!o.check_finite && sg < p.segments.size() && p.segments[sg].first == i &&
-        i + p.segments[sg].count <= last) {  // a run of small steps: one sequence launch
-      const Segment& g = p.segments[sg];
+  if (!o.check_finite) {
+    for (const WaveStage& g : p.wave.stages[std::is_same<R, double>::value]) {
+      if (g.step >= last) break;   // the complex128 tail's steps come last
       double cm = 0, by = 0;
-      for (int32_t j = i; j < i + g.count; ++j) {
+      if (g.kind == WaveStage::STEP)
+        by = step_bytes(p, p.steps[g.step], (double)sizeof(Cx<R>));
+      for (int32_t j : g.steps) {
         cm += (double)p.steps[j].R * (double)p.steps[j].K * (double)p.steps[j].N;
         by += step_bytes(p, p.steps[j], (double)sizeof(Cx<R>));
       }
-      mk.step = i;
-      mk.begin(1, cm, by, gpu_fill(1, 8));
-      k_seg<R><<<1, 256, 0, stream>>>(tiny + g.tiny0, g.count, arena, meta);
-      mk.end();
-      cudaError_t e = cudaGetLastError();
+      cudaError_t e = launch_stage<R>(p.wave, g, p.steps, (const unsigned char*)base + p.off_wave, arena,
+                                      meta, partial, counters, tcs, err, p.tuning.tc_db_groups, stream, mk,
+                                      cm, by);
       if (e != cudaSuccess) return e;
-      i += g.count;
-      continue;
     }
+    return cudaSuccess;
+  }
+  for (int32_t i = first; i < last; ++i) {
     mk.step = i;
     cudaError_t e = launch_step<R>(p.steps[i], arena, meta, partial, counters + i, stream, mk,
                                    step_bytes(p, p.steps[i], (double)sizeof(Cx<R>)), tcs, err,
                                    p.tuning.tc_db_groups);
-    if (e == cudaSuccess && o.check_finite)
+    if (e == cudaSuccess)
       e = check_tensor<R>(arena + p.steps[i].off_c, p.tensors[p.steps[i].c].elems, err,
                           status_nonfinite(sl, i), stream);
     if (e != cudaSuccess) return e;
-    ++i;
   }
   return cudaSuccess;
 }
@@ -352,6 +395,7 @@ cudaError_t launch_build(const Plan& p, char* base, char* arena_base, long long 
   mk.begin(0, 0, (double)sizeof(Cx<R>) * (double)initel, gpu_fill((long long)bx * p.n_init, 8));
   k_build<R><<<dim3(bx, (unsigned)p.n_init), 256, 0, stream>>>(
       (const Recipe*)(base + p.off_recipe), (const Slot*)(base + p.off_slots),
+      o.check_finite ? nullptr : (const int64_t*)(base + p.off_wave + p.wave.init_off),
       (Cx<R>*)arena_base, (Meta*)(base + p.off_meta), p.q, sl, (int)p.sliced.size());
   mk.end();
   cudaError_t e = cudaGetLastError();
@@ -371,6 +415,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
   char* base = (char*)ws;
   char* arena_base = (char*)arena;
   Marker mk{prof, stream, o.nvtx};
+  const long long final_off = o.check_finite ? p.tensors[p.final_tensor].offset : p.wave.off[p.final_tensor];
   SliceResult* res = (SliceResult*)(base + p.off_result);
   const int32_t n_steps = (int32_t)p.steps.size();
   const long long first = o.slice_first;
@@ -390,8 +435,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
       if ((e = launch_bulk<double>(p, base, arena_base, 0, n_steps, stream, mk, o, sl)) != cudaSuccess) return e;
       mk.step = -1;
       mk.begin(3, 0, 0, gpu_fill(1, 8));
-      k_slice_result<double><<<1, 32, 0, stream>>>((Cx<double>*)arena_base,
-                                                   p.tensors[p.final_tensor].offset,
+      k_slice_result<double><<<1, 32, 0, stream>>>((Cx<double>*)arena_base, final_off,
                                                    (Meta*)(base + p.off_meta), p.final_tensor, res, sl);
       mk.end();
     } else if (precision == PK_SPLIT) {
@@ -399,8 +443,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
       if ((e = launch_bulk<ff>(p, base, arena_base, 0, n_steps, stream, mk, o, sl)) != cudaSuccess) return e;
       mk.step = -1;
       mk.begin(3, 0, 0, gpu_fill(1, 8));
-      k_slice_result<ff><<<1, 32, 0, stream>>>((Cx<ff>*)arena_base,
-                                               p.tensors[p.final_tensor].offset,
+      k_slice_result<ff><<<1, 32, 0, stream>>>((Cx<ff>*)arena_base, final_off,
                                                (Meta*)(base + p.off_meta), p.final_tensor, res, sl);
       mk.end();
     } else if (p.tail.empty() && p.conv.empty()) {  // complex64
@@ -408,8 +451,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
       if ((e = launch_bulk<float>(p, base, arena_base, 0, n_steps, stream, mk, o, sl)) != cudaSuccess) return e;
       mk.step = -1;
       mk.begin(3, 0, 0, gpu_fill(1, 8));
-      k_slice_result<float><<<1, 32, 0, stream>>>((Cx<float>*)arena_base,
-                                                  p.tensors[p.final_tensor].offset,
+      k_slice_result<float><<<1, 32, 0, stream>>>((Cx<float>*)arena_base, final_off,
                                                   (Meta*)(base + p.off_meta), p.final_tensor, res, sl);
       mk.end();
     } else {  // complex64 with a complex128 tail
@@ -484,24 +526,14 @@ cudaError_t launch_grad_impl(const Plan& p, char* base, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     if (p.n_init > 0) {
       k_build<R><<<dim3(bx, (unsigned)p.n_init), 256, 0, stream>>>(
-          (const Recipe*)(base + G.off_recipe), (const Slot*)(base + G.off_slots), arena, meta,
+          (const Recipe*)(base + G.off_recipe), (const Slot*)(base + G.off_slots), nullptr, arena, meta,
           p.q, sl, (int)p.sliced.size());
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    const TinyStep* tiny = (const TinyStep*)(base + G.off_tiny);
-    size_t sg = 0;
-    for (size_t i = 0; i < G.steps.size();) {
-      while (sg < G.segments.size() && (size_t)G.segments[sg].first < i) ++sg;
-      if (sg < G.segments.size() && (size_t)G.segments[sg].first == i) {  // one sequence launch
-        const Segment& g = G.segments[sg];
-        k_seg<R><<<1, 256, 0, stream>>>(tiny + g.tiny0, g.count, arena, meta);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        i += g.count;
-        continue;
-      }
-      e = launch_step<R>(G.steps[i], arena, meta, partial, counters + i, stream, mk, 0.0);
+    for (const WaveStage& g : G.wave.stages[std::is_same<R, double>::value]) {
+      e = launch_stage<R>(G.wave, g, G.steps, (const unsigned char*)base + G.off_wave, arena, meta, partial,
+                          counters, nullptr, nullptr, 0, stream, mk, 0.0, 0.0);
       if (e != cudaSuccess) return e;
-      ++i;
     }
     k_slice_result<R><<<1, 32, 0, stream>>>(arena, G.root_offset, meta, G.root_meta, res, sl);
     if (!G.leaves.empty())
@@ -526,6 +558,8 @@ cudaError_t raise_rows_smem() {
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     if (e != cudaSuccess) return e;
   }
+  cudaError_t e = cudaFuncSetAttribute(k_waves<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWaveSmem);
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_outs<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 

@@ -21,7 +21,7 @@
 
 namespace {
 
-constexpr unsigned long long kNoallocScratchBytes = 64ull << 20;  // 64 MiB per device
+constexpr unsigned long long kNoallocScratchBytes = pk::kNoallocBytes;  // 64 MiB per device
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 
@@ -57,7 +57,7 @@ extern "C" pk_status pk_eval_noalloc(pk_ctx* ctx, const pk_plan* p, int32_t prec
     return noalloc_fail(ctx, PK_EINVAL, "bad precision");
   if (ctx->device < 0) return noalloc_fail(ctx, PK_ENODEVICE, "host-only context");
   if (ctx->device >= kMaxDevices) return noalloc_fail(ctx, PK_ENODEVICE, "device index too large");
-  const pk::Plan& P = p->p;
+  const pk::Plan& P = p->p.compact && p->p.ws_bytes(precision) > kNoallocScratchBytes ? *p->p.compact : p->p;
   const uint64_t need = P.ws_bytes(precision);
   if (need > kNoallocScratchBytes)
     return noalloc_fail(ctx, PK_ENOMEM,

@@ -3,7 +3,9 @@
 
 #include <array>
 #include <cstdint>
+#include <memory>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "pk.h"
@@ -161,23 +163,61 @@ struct ConvRec {
   int64_t elems;
   int32_t src_meta, dst_meta;
 };
-// A small step run inside a sequence kernel (one CTA runs consecutive small steps with a
-// block barrier between them): the step's row, contraction and column runs only.
-struct TinyStep {
+// ---- level schedule (wave_plan.cpp): steps of the same tree level run at the same time
+struct WaveRun {           // a stride run with 32-bit extents; y / size = (y mul) >> 32
+  uint32_t size, mul, sa, sb;
+};
+// A light step as the level kernels read it; its runs follow: rows, contracted, columns.
+struct WaveRec {
   int32_t a, b, c;         // bookkeeping slots (b = -1: constant 1)
-  int32_t nrow, nk, nn;
-  int64_t off_a, off_b, off_c;
-  int64_t R, K, N;
-  Run row[kMaxRuns];
-  Run kr[kMaxRuns];
-  Run nr[kMaxRuns];
+  uint32_t R;
+  uint32_t N, K, mul_r;    // mul_r: the division by R
+  uint8_t nrow, nk, nn, lanes;   // lanes: log2 of the lanes that share one output's sum
+  int64_t off_a, off_b;
+  int64_t off_c, pad;
 };
-// Consecutive small steps [first, first + count) run as one launch.
-struct Segment {
-  int32_t first, count;
-  int32_t tiny0;           // index of the first step's TinyStep record
+struct WaveItem {          // 32 lanes of a step's outputs: one warp's work
+  uint32_t rec, chunk;     // record (16-byte units), chunk of its lanes
 };
-constexpr int64_t kTinyK = 2048;          // contracted extent at most (offset table in shared memory)
+struct WaveUnit {          // a level of light steps, or one heavy step
+  bool heavy;
+  std::vector<int32_t> steps;
+};
+// Part of the device records (byte offsets, 16-byte aligned, and lengths) that one launch reads.
+struct WaveRange {
+  uint32_t rec, item, lev;
+  uint32_t rec_bytes, item_bytes, lev_bytes;
+  uint32_t item0, lev0;    // index of the first item; the first level's entry at `lev`
+};
+struct WaveStage {         // one launch
+  enum Kind : int32_t { FUSED, WIDE, STEP };
+  Kind kind = STEP;
+  int32_t units = 0;       // units it covers
+  int32_t step = -1;       // its (first) step
+  WaveRange range{};
+  uint32_t first = 0;      // WIDE: its first item after range.item
+  int32_t items = 0;
+  int32_t ctas = 1;        // FUSED: CTAs of the cluster
+  std::vector<int32_t> steps;   // FUSED, WIDE: its steps
+};
+struct WaveProgram {
+  std::vector<int64_t> off;          // arena offset of every tensor under this schedule
+  int64_t arena_elems = 0;
+  std::vector<WaveUnit> units;
+  std::vector<WaveStage> stages[2];  // launches in FP32 (complex64, split) and in FP64
+  std::vector<uint8_t> blob;         // records | items | level table | initial tensors' offsets
+  size_t init_off = 0;
+  int32_t n_init = 0;
+  int32_t n_fused[2] = {0, 0}, n_fused_steps[2] = {0, 0};   // launches of several steps, and their steps
+};
+constexpr int kWaveCtaWarps = 16;          // warps per CTA of the level kernel at most
+constexpr int kWaveMaxCtas = 8;            // CTAs of its cluster at most
+constexpr int kWaveCtaWarps32 = 16, kWaveCtaWarps64 = 4;   // warps of work per CTA it aims at
+constexpr int kWavePasses = 2;             // passes over a level at most; wider levels fill the GPU
+// split precision: a row step of GEMM shape with less work than this stays a row step of its
+// level instead of a conversion and a GEMM launch
+constexpr int64_t kWaveTcWork = 1LL << 20;
+constexpr int64_t kWaveOuts = 1LL << 18;   // outputs of a step inside a level at most
 
 struct TailStep {
   int32_t step;
@@ -252,8 +292,7 @@ struct GradProgram {
   std::vector<int8_t> phase;         // per step: 0 forward, 1 recompute, 2 adjoint
   std::vector<Recipe> recipes;       // initial tensors at their offsets in this arena
   std::vector<GradLeaf> leaves;      // one per EdgeGroup, same order
-  std::vector<Segment> segments;     // runs of small steps launched as one sequence kernel
-  std::vector<TinyStep> tiny;        // their records (in the program at off_tiny)
+  WaveProgram wave;                  // its level schedule (records in the program at off_wave)
   int32_t n_meta = 0;
   int32_t n_checkpoints = 0;
   int64_t arena_elems = 0;
@@ -261,13 +300,15 @@ struct GradProgram {
   int64_t root_offset = 0;
   int32_t root_meta = 0;
   double cmacs[3] = {0, 0, 0};       // per slice, by phase
-  uint64_t off_recipe = 0, off_slots = 0, off_leaves = 0, off_tiny = 0, off_meta = 0,
+  uint64_t off_recipe = 0, off_slots = 0, off_leaves = 0, off_wave = 0, off_meta = 0,
            off_counter = 0, off_result = 0, off_scratch = 0, off_acc = 0, off_arena = 0;
-  std::vector<uint8_t> program;      // recipes | slots | leaves | tiny steps, copied by pk_grad
+  std::vector<uint8_t> program;      // recipes | slots | leaves | level records, copied by pk_grad
   uint64_t ws_bytes(int32_t precision) const {
     return off_arena + (uint64_t)arena_elems * (precision == PK_C64 ? 8ull : 16ull);
   }
 };
+
+constexpr uint64_t kNoallocBytes = 64ull << 20;   // pk_eval_noalloc's workspace
 
 struct TensorInfo {
   std::vector<int32_t> dims;  // index ids, outermost first (row-major)
@@ -304,16 +345,20 @@ struct Plan {
   uint64_t off_recipe = 0, off_slots = 0, off_meta = 0, off_result = 0, off_scratch = 0,
            off_counter = 0, off_arena = 0;
   uint64_t ws_bytes(int32_t precision) const;
+  // elements of the arena the workspace holds: the steps' own order (arena_elems) or the
+  // level schedule's, whichever is larger
+  int64_t ws_elems() const { return arena_elems > wave.arena_elems ? arena_elems : wave.arena_elems; }
   // byte offset of the split precision's digit scratch from the arena's start
-  uint64_t tc_offset() const { return ((uint64_t)arena_elems * 16ull + 255) & ~uint64_t(255); }
+  uint64_t tc_offset() const { return ((uint64_t)ws_elems() * 16ull + 255) & ~uint64_t(255); }
   std::vector<uint8_t> program;      // recipe + slots blob copied by pk_upload
   // split precision: steps >= tail_first run in complex128 in a separate tail region;
   // bulk tensors they read are up-converted there first
   int32_t tail_first = 0;
   std::vector<ConvRec> conv;
-  std::vector<Segment> segments;     // runs of small steps launched as one sequence kernel
-  std::vector<TinyStep> tiny;        // their records (in the program at off_tiny)
-  uint64_t off_tiny = 0;
+  WaveProgram wave;                  // level schedule (records in the program at off_wave)
+  std::shared_ptr<Plan> compact;     // the same plan on its own order's layout, where only that
+                                     // fits pk_eval_noalloc's workspace
+  uint64_t off_wave = 0;
   pk_tuning tuning{};                // launch shapes the plan was made with
   std::vector<TailStep> tail;        // one per step >= tail_first
   int64_t tail_elems = 0;            // complex128 elements of the tail region
@@ -363,11 +408,31 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
 // of the summed R K N, out[2] initial tensors, out[3] indices, for the best candidate of
 // `order` (by rank, then cost).  False for an unknown order or q.
 bool order_stats(const Knot& k, int32_t q, int32_t order, int32_t restarts, double* out);
-// Maximal runs (>= 2) of consecutive small row-kernel steps (at most tune.seq_outs outputs,
-// K <= tune.seq_k <= kTinyK, at most tune.seq_work complex multiply-adds), with their
-// compact records, for the sequence kernel k_seg.
-void build_segments(const std::vector<Step>& steps, const pk_tuning& tune,
-                    std::vector<Segment>& segments, std::vector<TinyStep>& tiny);
+// Level schedule.  light: the step runs inside a level.  wave_schedule: the units in launch
+// order (breadth: every ready heavy step before the next levels; otherwise one at a time);
+// `extra` orders further pairs of steps.  wave_layout: first fit over the units' lifetimes,
+// pinned tensors kept to the end; returns the arena's elements.  wave_hazards: the pairs that
+// a given layout orders.  wave_stages: the launches and the device records.  wave_check: a
+// replay of the units over the layout.
+bool wave_light(const Step& s, const pk_tuning& tune);
+// Arena offsets (multiples of 64 elements) by first fit in decreasing size over the closed
+// lifetimes [born, dies]; returns the arena's elements.
+int64_t first_fit(const std::vector<int64_t>& elems, const std::vector<int32_t>& born,
+                  const std::vector<int32_t>& dies, std::vector<int64_t>& off);
+void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuning& tune, bool breadth,
+                   const std::vector<std::pair<int32_t, int32_t>>* extra, int32_t first_tail,
+                   std::vector<WaveUnit>& units);
+int64_t wave_layout(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
+                    const std::vector<char>& pinned, const std::vector<WaveUnit>& units,
+                    std::vector<int64_t>& off);
+void wave_hazards(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
+                  const std::vector<int64_t>& off, std::vector<std::pair<int32_t, int32_t>>& edges);
+void wave_stages(const std::vector<Step>& steps, WaveProgram& w);
+bool wave_check(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
+                const std::vector<char>& pinned, const WaveProgram& w, std::string& err);
+// The plan's level schedule and the workspace layout that holds it; `compact`: on the
+// tensors' offsets of the steps' own order, so that the workspace does not grow.
+void plan_waves(Plan& p, bool compact);
 bool valid_tuning(const pk_tuning& t);
 bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& tune, std::string& err);
 // Writes the clause values of p.weights into p.slots and both program blobs.

@@ -1306,7 +1306,7 @@ bool build_step(const std::vector<int32_t>& xd, const std::vector<int32_t>* yd,
 bool valid_tuning(const pk_tuning& t) {
   return (t.batch_threads == 128 || t.batch_threads == 256 || t.batch_threads == 512) &&
          t.batch_ktab >= 256 && t.batch_ktab <= 2048 && t.seq_outs >= 1 && t.seq_outs <= 65536 &&
-         t.seq_work >= 1 && t.seq_work <= (1 << 24) && t.seq_k >= 1 && t.seq_k <= kTinyK &&
+         t.seq_work >= 1 && t.seq_work <= (1 << 24) && t.seq_k >= 1 && t.seq_k <= 2048 &&
          t.tc_min_k >= 4 && t.tc_min_k <= 16 && t.tc_db_groups >= 0 && t.tc_db_groups <= 4096 &&
          t.tc_min_n >= 8 && t.tc_min_n <= 32 && t.cost_gemm_milli >= 10 &&
          t.cost_gemm_milli <= 1000 && t.cost_out_milli >= 0 && t.cost_out_milli <= 1000000 &&
@@ -1314,64 +1314,14 @@ bool valid_tuning(const pk_tuning& t) {
          t.cost_tcin_milli <= 1000000 && t.tc_min_work >= 0 && t.tc_min_work <= ((int64_t)1 << 40);
 }
 
-void build_segments(const std::vector<Step>& steps, const pk_tuning& tune,
-                    std::vector<Segment>& segments, std::vector<TinyStep>& tiny) {
-  segments.clear();
-  tiny.clear();
-  const int64_t max_k = std::min<int64_t>(tune.seq_k, kTinyK);
-  auto small = [&](const Step& st) {
-    return st.kernel == KROWS && !st.tc && st.R * st.N <= tune.seq_outs && st.K <= max_k &&
-           st.R * st.N * st.K <= tune.seq_work;
-  };
-  const int32_t n_steps = (int32_t)steps.size();
-  int32_t s0 = 0;
-  while (s0 < n_steps) {
-    if (!small(steps[s0])) {
-      ++s0;
-      continue;
-    }
-    int32_t s1 = s0;
-    while (s1 < n_steps && small(steps[s1])) ++s1;
-    if (s1 - s0 >= 2) {
-      Segment sg;
-      sg.first = s0;
-      sg.count = s1 - s0;
-      sg.tiny0 = (int32_t)tiny.size();
-      for (int32_t i = s0; i < s1; ++i) {
-        const Step& st = steps[i];
-        TinyStep ts;
-        std::memset(&ts, 0, sizeof(ts));
-        ts.a = st.a;
-        ts.b = st.b;
-        ts.c = st.c;
-        ts.nrow = st.nrow;
-        ts.nk = st.nk;
-        ts.nn = st.nn;
-        ts.off_a = st.off_a;
-        ts.off_b = st.off_b;
-        ts.off_c = st.off_c;
-        ts.R = st.R;
-        ts.K = st.K;
-        ts.N = st.N;
-        std::memcpy(ts.row, st.row, sizeof(ts.row));
-        std::memcpy(ts.kr, st.kr, sizeof(ts.kr));
-        std::memcpy(ts.nr, st.nr, sizeof(ts.nr));
-        tiny.push_back(ts);
-      }
-      segments.push_back(sg);
-    }
-    s0 = s1;
-  }
-}
-
 uint64_t Plan::ws_bytes(int32_t precision) const {
   if (precision == PK_C64) {
-    if (tail.empty()) return off_arena + (uint64_t)arena_elems * 8ull;
+    if (tail.empty()) return off_arena + (uint64_t)ws_elems() * 8ull;
     return off_tail + (uint64_t)tail_elems * 16ull;  // complex128 tail region after the arena
   }
   if (precision == PK_SPLIT && tc_bytes > 0)   // float-float pairs, then the digit scratch
     return off_arena + tc_offset() + (uint64_t)tc_bytes;
-  return off_arena + (uint64_t)arena_elems * 16ull;  // complex128 and float-float pairs
+  return off_arena + (uint64_t)ws_elems() * 16ull;  // complex128 and float-float pairs
 }
 
 static uint64_t align256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
@@ -1625,35 +1575,15 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
   p.splitk_partials = partials;
 
   // ---- arena: first fit by decreasing size over lifetime intervals
-  std::vector<int32_t> ord(n_tens);
-  std::iota(ord.begin(), ord.end(), 0);
-  std::sort(ord.begin(), ord.end(), [&](int32_t x, int32_t y) {
-    if (p.tensors[x].elems != p.tensors[y].elems) return p.tensors[x].elems > p.tensors[y].elems;
-    return x < y;
-  });
-  struct Placed {
-    int64_t off, len;
-    int32_t born, dies;
-  };
-  std::vector<Placed> placed;
-  int64_t top = 0;
-  for (int32_t id : ord) {
-    TensorInfo& ti = p.tensors[id];
-    int64_t len = (ti.elems + 63) / 64 * 64;
-    std::vector<std::pair<int64_t, int64_t>> busy;
-    for (const auto& pl : placed)
-      if (!(pl.dies < ti.born || ti.dies < pl.born)) busy.push_back({pl.off, pl.off + pl.len});
-    std::sort(busy.begin(), busy.end());
-    int64_t off = 0;
-    for (const auto& iv : busy) {
-      if (off + len <= iv.first) break;
-      off = std::max(off, iv.second);
-    }
-    ti.offset = off;
-    placed.push_back({off, len, ti.born, ti.dies});
-    top = std::max(top, off + len);
+  std::vector<int64_t> elems, offs;
+  std::vector<int32_t> born, dies;
+  for (const TensorInfo& ti : p.tensors) {
+    elems.push_back(ti.elems);
+    born.push_back(ti.born);
+    dies.push_back(ti.dies);
   }
-  p.arena_elems = top;
+  p.arena_elems = first_fit(elems, born, dies, offs);
+  for (int32_t i = 0; i < n_tens; ++i) p.tensors[i].offset = offs[i];
   for (auto& st : p.steps) {
     st.off_a = p.tensors[st.a].offset;
     st.off_b = st.b >= 0 ? p.tensors[st.b].offset : 0;
@@ -1762,9 +1692,6 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
     p.n_meta = n_tens + (int32_t)p.conv.size();
   }
 
-  // ---- segments: maximal runs (>= 2) of consecutive small row-kernel steps
-  build_segments(p.steps, tune, p.segments, p.tiny);
-
   // ---- workspace layout
   uint64_t off = 0;
   p.off_recipe = off;
@@ -1773,27 +1700,26 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
   off = align256(off + sizeof(Slot) * std::max<size_t>(1, p.slots.size()));
   p.off_conv = off;
   off = align256(off + sizeof(ConvRec) * std::max<size_t>(1, p.conv.size()));
-  p.off_tiny = off;
-  off = align256(off + sizeof(TinyStep) * p.tiny.size());
-  p.off_meta = off;
-  off = align256(off + 16ull * p.n_meta);
-  p.off_counter = off;
-  off = align256(off + 4ull * std::max<int32_t>(1, n_steps));
-  p.off_result = off;
-  off = align256(off + 32ull * (uint64_t)p.n_slices + 32);
-  p.off_scratch = off;
-  off = align256(off + 16ull * (uint64_t)std::max<int64_t>(1, partials));
-  p.off_arena = off;
-  p.off_tail = align256(p.off_arena + 8ull * (uint64_t)p.arena_elems);
-  p.program.assign(p.off_meta, 0);
+  p.off_wave = off;
+  p.program.assign(p.off_wave, 0);
   if (!p.recipes.empty())
     std::memcpy(p.program.data() + p.off_recipe, p.recipes.data(), sizeof(Recipe) * p.recipes.size());
   if (!p.slots.empty())
     std::memcpy(p.program.data() + p.off_slots, p.slots.data(), sizeof(Slot) * p.slots.size());
   if (!p.conv.empty())
     std::memcpy(p.program.data() + p.off_conv, p.conv.data(), sizeof(ConvRec) * p.conv.size());
-  if (!p.tiny.empty())
-    std::memcpy(p.program.data() + p.off_tiny, p.tiny.data(), sizeof(TinyStep) * p.tiny.size());
+  plan_waves(p, false);
+  // the level schedule's layout may not push a plan over the allocation-free entry point's
+  // fixed workspace that its own order fits: such a plan keeps a second schedule for it
+  for (int32_t prec : {PK_C128, PK_C64, PK_SPLIT})
+    if (!p.compact && p.wave.arena_elems > p.arena_elems && p.ws_bytes(prec) > kNoallocBytes) {
+      const uint64_t own = p.ws_bytes(prec) - (prec == PK_C64 ? 8ull : 16ull) * (uint64_t)(p.wave.arena_elems - p.arena_elems);
+      if (own <= kNoallocBytes + 512) {   // alignment of the scratch behind the arena
+        auto c = std::make_shared<Plan>(p);
+        plan_waves(*c, true);
+        p.compact = c;
+      }
+    }
   if (grad && !make_grad_program(p, opts.checkpoint_stride, opts.flags, tune, err)) return false;
   // clause values of general networks, stored scaled by powers of two (Recipe::exp2)
   if (p.general) apply_weights(p);
@@ -1827,6 +1753,11 @@ static int32_t max_exp4(double a, double b, double c, double d) {
 }
 
 void apply_weights(Plan& p) {
+  if (p.compact) {
+    p.compact->weights = p.weights;
+    p.compact->std_weights = p.std_weights;
+    apply_weights(*p.compact);
+  }
   p.slot_exp.assign(p.slots.size(), 0);
   for (const EdgeGroup& g : p.groups) {
     double dre = 1, dim = 0, ore = 1, oim = 0;

@@ -10,19 +10,13 @@
 //   threads  512  ktab   512     5.555
 //   threads  512  ktab  1024     5.578
 //   threads  512  ktab  2048     5.640
-// Sequence runs, 192 evaluations of the scale workload, split (median ms per step):
-//   outs <=  1024  work <=   4096     60.00  (6354 launches)
-//   outs <=  1024  work <=  16384     60.04  (6243 launches)
-//   outs <=  1024  work <=  65536     59.74  (6219 launches)
-//   outs <=  2048  work <=   4096     60.22  (6352 launches)
-//   outs <=  2048  work <=  16384     60.20  (6226 launches)
-//   outs <=  2048  work <=  65536     60.26  (6195 launches)
-//   outs <=  4096  work <=   4096     60.30  (6086 launches)
-//   outs <=  4096  work <=  16384     60.28  (4362 launches)
-//   outs <=  4096  work <=  65536     60.27  (4275 launches)
-//   outs <=  8192  work <=   4096     59.91  (6086 launches)
-//   outs <=  8192  work <=  16384     60.25  (4360 launches)
-//   outs <=  8192  work <=  65536     60.31  (3898 launches)
+// Level launches, single evaluations (us per call; 48 evaluations as one group last):
+//                                  q3 c128  q5 split  q3 c64  sliced split  grad q5 split  group
+//   outs <=  1024  work <=   65536    1346       877     441         37125            798   7839
+//   outs <=  8192  work <=  262144    1301       830     330         28571            579   7632
+//   outs <= 65536  work <=  262144    1275       780     318         23942            528   7563
+//   outs <= 65536  work <= 1048576    1266       758     320         20594            402   7921
+//   outs <= 65536  work <= 4194304    1259       754     316         20635            445   7911
 // Tensor cores for row steps of GEMM shape from this K, split (median ms per step):
 //   K >=  4     59.96
 //   K >=  8     60.36
@@ -129,4 +123,4 @@
 #pragma once
 #include "pk.h"
 
-constexpr pk_tuning kTunedDefault = {256, 512, 1024, 65536, 2048, 8, 0, 12, 100, 32000, 25, 4000, 65536};
+constexpr pk_tuning kTunedDefault = {256, 512, 65536, 1048576, 2048, 8, 0, 12, 100, 32000, 25, 4000, 65536};

@@ -8,7 +8,7 @@
 // stride, each stride equals the product of the extents below it and the extents multiply
 // to the tensor's size), the result must be the step's own new tensor, and every tensor
 // must lie inside the arena without overlapping another tensor that is live at the same
-// step.  The records the kernels read (the sequence kernel's copies of small steps, the
+// step.  The records the kernels read (the level schedule of the small steps, the
 // complex128 tail steps, the digit scratch of the tensor-core steps, the reverse program)
 // are checked against the same rules.
 #include <algorithm>
@@ -131,12 +131,6 @@ bool check_step(const Step& s, int64_t ea, int64_t eb, int64_t ec, const std::st
   return true;
 }
 
-bool same_runs(const Run* x, const Run* y, int n) {
-  for (int i = 0; i < n; ++i)
-    if (x[i].size != y[i].size || x[i].sa != y[i].sa || x[i].sb != y[i].sb) return false;
-  return true;
-}
-
 // [off, off + len) intervals that are live together must not overlap.
 struct Live {
   int64_t off, len;
@@ -198,22 +192,15 @@ bool check_forward(const Plan& p, int32_t precision, Checker& ck) {
       if (x.bytes > p.tc_bytes) return ck.fail(w, "digit scratch larger than the plan reserves");
     }
   }
-  // sequence-kernel records: exact copies of their steps' row views
-  for (const Segment& g : p.segments) {
-    const std::string w = "sequence run at step " + std::to_string(g.first);
-    if (g.count < 2 || g.first < 0 || g.first + g.count > ns || g.tiny0 < 0 ||
-        g.tiny0 + g.count > (int32_t)p.tiny.size())
-      return ck.fail(w, "range outside the steps or records");
-    for (int32_t j = 0; j < g.count; ++j) {
-      const Step& s = p.steps[g.first + j];
-      const TinyStep& t = p.tiny[g.tiny0 + j];
-      if (s.kernel != KROWS || s.tc || t.a != s.a || t.b != s.b || t.c != s.c ||
-          t.off_a != s.off_a || t.off_b != s.off_b || t.off_c != s.off_c || t.R != s.R ||
-          t.K != s.K || t.N != s.N || t.nrow != s.nrow || t.nk != s.nk || t.nn != s.nn ||
-          !same_runs(t.row, s.row, s.nrow) || !same_runs(t.kr, s.kr, s.nk) ||
-          !same_runs(t.nr, s.nr, s.nn) || s.K > kTinyK)
-        return ck.fail(w, "record differs from step " + std::to_string(g.first + j));
-    }
+  // level schedule: a replay of its units over its layout
+  {
+    std::vector<int64_t> elems;
+    std::vector<char> pinned(nt, 0);
+    for (const TensorInfo& t : p.tensors) elems.push_back(t.elems);
+    pinned[p.final_tensor] = 1;
+    if (p.wave.arena_elems > p.ws_elems()) return ck.fail("level schedule", "arena larger than the workspace's");
+    std::string e;
+    if (!wave_check(p.steps, elems, pinned, p.wave, e)) return ck.fail("plan", e);
   }
   // complex128 tail of the complex64 precision
   if (precision == PK_C64 && !p.tail.empty()) {
@@ -239,17 +226,17 @@ bool check_forward(const Plan& p, int32_t precision, Checker& ck) {
   }
   // workspace layout: state records in order, the arena (and the split digit scratch or the
   // tail region) inside the workspace
-  if (!(p.off_recipe <= p.off_slots && p.off_slots <= p.off_conv && p.off_conv <= p.off_tiny &&
-        p.off_tiny <= p.off_meta && p.off_meta + 16ull * p.n_meta <= p.off_counter &&
+  if (!(p.off_recipe <= p.off_slots && p.off_slots <= p.off_conv && p.off_conv <= p.off_wave &&
+        p.off_wave + p.wave.blob.size() <= p.off_meta && p.off_meta + 16ull * p.n_meta <= p.off_counter &&
         p.off_counter + 4ull * (uint64_t)ns <= p.off_result &&
         p.off_result + 32ull * (uint64_t)(p.n_slices + 1) <= p.off_scratch &&
         p.off_scratch + 16ull * (uint64_t)p.splitk_partials <= p.off_arena))
     return ck.fail("workspace", "state records overlap");
   const uint64_t esz = precision == PK_C64 ? 8 : 16;
-  uint64_t end = p.off_arena + esz * (uint64_t)p.arena_elems;
+  uint64_t end = p.off_arena + esz * (uint64_t)p.ws_elems();
   if (precision == PK_SPLIT && p.tc_bytes > 0) end = p.off_arena + p.tc_offset() + (uint64_t)p.tc_bytes;
   if (precision == PK_C64 && !p.tail.empty()) {
-    if (p.off_tail < p.off_arena + 8ull * (uint64_t)p.arena_elems)
+    if (p.off_tail < p.off_arena + 8ull * (uint64_t)p.ws_elems())
       return ck.fail("workspace", "tail region overlaps the arena");
     end = p.off_tail + 16ull * (uint64_t)p.tail_elems;
   }
@@ -280,6 +267,17 @@ bool check_grad(const Plan& p, Checker& ck) {
     if (s.a < 0 || s.a >= G.n_meta || s.c < 0 || s.c >= G.n_meta || s.b >= G.n_meta)
       return ck.fail(w, "bookkeeping slot out of range");
     if (!check_step(s, ea, eb, ec, w, ck)) return false;
+  }
+  {
+    std::vector<int64_t> elems(G.n_meta, 0);
+    std::vector<char> pinned(G.n_meta, 0);
+    for (const Recipe& r : G.recipes) elems[r.meta] = r.elems;
+    for (const Step& s : G.steps) elems[s.c] = s.R * s.N;
+    pinned[G.root_meta] = 1;
+    for (const GradLeaf& l : G.leaves)
+      if (l.meta >= 0) pinned[l.meta] = 1;
+    std::string e;
+    if (!wave_check(G.steps, elems, pinned, G.wave, e)) return ck.fail("reverse program", e);
   }
   for (const Recipe& r : G.recipes)
     if (r.offset < 0 || r.offset + r.elems > G.arena_elems)
