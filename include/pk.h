@@ -57,7 +57,9 @@ typedef enum {
 } pk_status;
 
 typedef enum {
-  PK_C128 = 0,       /* complex128 storage, FP64 arithmetic                               */
+  PK_C128 = 0,       /* complex128 storage, FP64 arithmetic; large GEMM-shaped steps on the
+                        tensor cores in exact 62-bit fixed point per row and column, with
+                        errors below FP64's own                                           */
   PK_C64 = 1,        /* complex64 storage, FP32 arithmetic; with pk_plan_opts.tail_steps
                         > 0 the final contractions run in complex128                      */
   PK_SPLIT = 2       /* split FP32: every real number is an unevaluated pair of floats
@@ -89,8 +91,8 @@ typedef enum {
  * the planner choose per step by its shape). */
 #define PK_FLAG_FORCE_GEMM 1 /* every two-operand step on the tiled GEMM kernel           */
 #define PK_FLAG_FORCE_ROWS 2 /* every step on the row kernel                               */
-#define PK_FLAG_NO_TC 8      /* PK_SPLIT: run GEMM-shaped steps on the CUDA cores (float-float
-                                SIMT kernel) instead of the tensor cores                     */
+#define PK_FLAG_NO_TC 8      /* PK_SPLIT, PK_C128: run GEMM-shaped steps on the CUDA cores
+                                (float-float or FP64 SIMT kernels) instead of the tensor cores */
 #define PK_FLAG_TC_DIGITS4 16 /* PK_SPLIT tensor-core steps: four BF16 digits per operand
                                 (10 digit-pair products, truncation near 2^-32 of a row's and
                                 column's largest entries) instead of five (15 products, 2^-40) */

@@ -515,7 +515,10 @@ pk_status pk_plan_launches(const pk_plan* p, int32_t precision, int64_t* launche
   if (!p || !launches || !valid_precision(precision)) return PK_EINVAL;
   const pk::Plan& P = p->p;
   const int64_t widen = (precision == PK_C64 && !P.conv.empty()) ? 1 : 0;
-  int64_t digits = 0;   // split precision: one conversion launch per tensor-core step
+  int64_t digits = 0;   // split and complex128: one conversion launch per tensor-core step
+  if (precision == PK_C128 && P.tc64_bytes > 0)
+    for (const pk::WaveStage& g : P.wave.stages[1])
+      digits += g.kind == pk::WaveStage::STEP && pk::tc64_step(P.steps[g.step]);
   if (precision == PK_SPLIT)
     for (const pk::WaveStage& g : P.wave.stages[0])
       digits += g.kind == pk::WaveStage::STEP && P.steps[g.step].tc;
@@ -1092,6 +1095,8 @@ pk_status pk_grad(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_work
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "reverse pass");
   const pk::SliceResult* r = (const pk::SliceResult*)(host + prog);
+  std::string werr;
+  if ((s = pk::status_error(r->status, werr)) != PK_OK) return fail(ctx, s, werr);
   pk::Scaled z;
   z.re = r->re;
   z.im = r->im;

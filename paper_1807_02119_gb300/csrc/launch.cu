@@ -18,6 +18,7 @@
 #include "kernels.cuh"
 #include "gemm_tc.cuh"
 #include "wave.cuh"
+#include "gemm_d64.cuh"
 
 namespace pk {
 
@@ -257,6 +258,22 @@ cudaError_t launch_tc(const Step& s, Cx<ff>* arena, Meta* meta, unsigned char* t
   return cudaGetLastError();
 }
 
+// complex128 on the tensor cores: the digits of both operands, then the GEMM.
+cudaError_t launch_tc64(const Step& s, Cx<double>* arena, Meta* meta, unsigned char* tcs,
+                        unsigned long long* err, cudaStream_t stream, Marker& mk, double cm, double by) {
+  const Tc64Scratch L = tc64_scratch(s.Bsz, s.M, s.N, s.K);
+  const long long nA = s.Bsz * L.tiles_m * (kTcMc / 8 / d64_groups(L.chunks, kTcMc / 8)),
+                  nB = s.Bsz * L.tiles_n * (kTc64Nc / 8 / d64_groups(L.chunks, kTc64Nc / 8));
+  mk.begin(6, 0.0, 16.0 * (double)(s.R * s.K + s.Bsz * s.K * s.N), gpu_fill(nA + nB, 8));
+  k_digits64<<<(unsigned)(nA + nB), d64::kConvThreads, 0, stream>>>(s, arena, tcs, nA);
+  mk.end();
+  const long long grid = std::min<long long>(L.tiles_m * L.tiles_n * s.Bsz, (long long)g_sms);
+  mk.begin(5, cm, by, gpu_fill(grid, 1));
+  k_gemm64<<<(unsigned)grid, d64::kThreads, d64::kSmem, stream>>>(s, arena, meta, tcs, err);
+  mk.end();
+  return cudaGetLastError();
+}
+
 template <typename R>
 cudaError_t launch_step(const Step& s, Cx<R>* arena, Meta* meta, Cx<double>* partial,
                         unsigned* counter, cudaStream_t stream, Marker& mk, double by,
@@ -270,6 +287,9 @@ cudaError_t launch_step(const Step& s, Cx<R>* arena, Meta* meta, Cx<double>* par
       return s.tc == 4
                  ? launch_tc<4>(s, arena, meta, tc_scratch, counter, err, stream, mk, cm, by, db_groups)
                  : launch_tc<5>(s, arena, meta, tc_scratch, counter, err, stream, mk, cm, by, db_groups);
+  }
+  if constexpr (std::is_same<R, double>::value) {
+    if (tc_scratch && err && tc64_step(s)) return launch_tc64(s, arena, meta, tc_scratch, err, stream, mk, cm, by);
   }
   if (s.kernel == KGEMM && gemm_tiles < (1LL << 31)) {
     mk.begin(4, cm, by, gpu_fill(gemm_tiles, 8));
@@ -347,8 +367,9 @@ cudaError_t launch_bulk(const Plan& p, char* base, char* arena_base, int32_t fir
   Meta* meta = (Meta*)(base + p.off_meta);
   Cx<double>* partial = (Cx<double>*)(base + p.off_scratch);
   unsigned* counters = (unsigned*)(base + p.off_counter);
-  unsigned char* tcs = (std::is_same<R, ff>::value && p.tc_bytes > 0)
-                           ? (unsigned char*)arena_base + p.tc_offset() : nullptr;
+  // digit scratch of the tensor-core steps
+  const bool digits = std::is_same<R, ff>::value ? p.tc_bytes > 0 : std::is_same<R, double>::value && p.tc64_bytes > 0;
+  unsigned char* tcs = digits ? (unsigned char*)arena_base + p.tc_offset() : nullptr;
   unsigned long long* err = &((SliceResult*)(base + p.off_result))[p.n_slices].status;
   if (!o.check_finite) {
     for (const WaveStage& g : p.wave.stages[std::is_same<R, double>::value]) {
@@ -512,6 +533,8 @@ cudaError_t launch_grad_impl(const Plan& p, char* base, cudaStream_t stream) {
   SliceResult* res = (SliceResult*)(base + G.off_result);
   Cx<double>* partial = (Cx<double>*)(base + G.off_scratch);
   unsigned* counters = (unsigned*)(base + G.off_counter);
+  unsigned char* tcs = std::is_same<R, double>::value && G.tc64_bytes > 0
+                           ? (unsigned char*)arena + G.tc_offset() : nullptr;
   const uint64_t nl = std::max<size_t>(1, G.leaves.size());
   Cx<double>* acc = (Cx<double>*)(base + G.off_acc);
   long long* acc_exp = (long long*)(base + G.off_acc + 16ull * (uint64_t)p.q * p.q * nl);
@@ -522,7 +545,8 @@ cudaError_t launch_grad_impl(const Plan& p, char* base, cudaStream_t stream) {
   cudaError_t e = cudaMemsetAsync(base + G.off_acc, 0, G.off_arena - G.off_acc, stream);
   if (e != cudaSuccess) return e;
   for (long long sl = 0; sl < p.n_slices; ++sl) {
-    e = cudaMemsetAsync(base + G.off_meta, 0, G.off_result - G.off_meta, stream);
+    // bookkeeping and tickets; the first slice also the results with the error word
+    e = cudaMemsetAsync(base + G.off_meta, 0, (sl == 0 ? G.off_scratch : G.off_result) - G.off_meta, stream);
     if (e != cudaSuccess) return e;
     if (p.n_init > 0) {
       k_build<R><<<dim3(bx, (unsigned)p.n_init), 256, 0, stream>>>(
@@ -532,7 +556,7 @@ cudaError_t launch_grad_impl(const Plan& p, char* base, cudaStream_t stream) {
     }
     for (const WaveStage& g : G.wave.stages[std::is_same<R, double>::value]) {
       e = launch_stage<R>(G.wave, g, G.steps, (const unsigned char*)base + G.off_wave, arena, meta, partial,
-                          counters, nullptr, nullptr, 0, stream, mk, 0.0, 0.0);
+                          counters, tcs, &res[p.n_slices].status, 0, stream, mk, 0.0, 0.0);
       if (e != cudaSuccess) return e;
     }
     k_slice_result<R><<<1, 32, 0, stream>>>(arena, G.root_offset, meta, G.root_meta, res, sl);
@@ -598,6 +622,7 @@ cudaError_t prepare_kernels() {
   if ((e = raise_rows_smem<ff>()) != cudaSuccess) return e;
   if ((e = prepare_tc<4>()) != cudaSuccess) return e;
   if ((e = prepare_tc<5>()) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_gemm64, cudaFuncAttributeMaxDynamicSharedMemorySize, d64::kSmem)) != cudaSuccess) return e;
   if (dev >= 0 && dev < 256) done[dev] = true;
   return cudaSuccess;
 }

@@ -180,7 +180,7 @@ struct WaveItem {          // 32 lanes of a step's outputs: one warp's work
   uint32_t rec, chunk;     // record (16-byte units), chunk of its lanes
 };
 struct WaveUnit {          // a level of light steps, or one heavy step
-  bool heavy;
+  bool heavy;                        // a launch of its own (in FP64 only, if the step is light)
   std::vector<int32_t> steps;
 };
 // Part of the device records (byte offsets, 16-byte aligned, and lengths) that one launch reads.
@@ -263,6 +263,39 @@ PK_HD inline TcScratch tc_scratch(long long Bsz, long long M, long long N, long 
   return x;
 }
 
+// GEMM steps of the complex128 precision on the tensor cores (gemm_d64.cuh): eight digits,
+// tiles of kTcMc x kTc64Nc complex, chunks of kTc64Kc complex k, one exponent per row and
+// column; the digits, exponents and C offsets lie after the arena as above.
+constexpr int kTc64Nc = 16, kTc64Kc = 8;
+constexpr long long kTc64AChunk = 8LL * kTcMc * (2 * kTc64Kc) * 2, kTc64BChunk = 8LL * (2 * kTc64Nc) * (2 * kTc64Kc) * 2;
+constexpr long long kTc64MaxK = 4096;   // offsets of the contracted index in shared memory
+struct Tc64Scratch {
+  long long tiles_m, tiles_n, chunks;
+  long long a_off, b_off, ea_off, eb_off, cr_off, cc_off, bytes;
+};
+PK_HD inline Tc64Scratch tc64_scratch(long long Bsz, long long M, long long N, long long K) {
+  Tc64Scratch x;
+  x.tiles_m = (M + kTcMc - 1) / kTcMc;
+  x.tiles_n = (N + kTc64Nc - 1) / kTc64Nc;
+  x.chunks = (K + kTc64Kc - 1) / kTc64Kc;
+  x.a_off = 0;
+  x.b_off = x.a_off + Bsz * x.tiles_m * x.chunks * kTc64AChunk;
+  x.ea_off = x.b_off + Bsz * x.tiles_n * x.chunks * kTc64BChunk;
+  x.eb_off = x.ea_off + ((Bsz * x.tiles_m * kTcMc * 4 + 255) & ~255LL);
+  x.cr_off = x.eb_off + ((Bsz * x.tiles_n * kTc64Nc * 4 + 255) & ~255LL);
+  x.cc_off = x.cr_off + ((Bsz * x.tiles_m * kTcMc * 8 + 255) & ~255LL);
+  x.bytes = x.cc_off + ((x.tiles_n * kTc64Nc * 8 + 255) & ~255LL);
+  return x;
+}
+// Whether complex128 runs the step there: GEMM-shaped, and enough work to pay for the
+// conversion and the second launch (about 10 us, in which FP64 does 1.5e6 multiply-adds).
+inline bool tc64_step(const Step& s) {
+  const long long work = s.R * s.K * s.N;
+  return s.b >= 0 && s.kernel != KSPLITK && s.M >= 64 && s.N >= 4 && s.K >= 4 && s.K <= kTc64MaxK &&
+         work >= (s.kernel == KGEMM ? 1LL << 19 : 1LL << 20) &&
+         tc64_scratch(s.Bsz, s.M, s.N, s.K).bytes <= (8LL << 30);
+}
+
 // Reverse pass: one record per clause tensor (merged edge group) of a gradient plan.
 // The adjoint dZ/dM of the group's matrix M (full shape q x q, or q for a loop vector)
 // is read from the arena with the strides below and added into an accumulator.
@@ -297,13 +330,16 @@ struct GradProgram {
   int32_t n_checkpoints = 0;
   int64_t arena_elems = 0;
   int64_t partials = 0;
+  int64_t tc64_bytes = 0;            // complex128: digit scratch of the largest tensor-core step
   int64_t root_offset = 0;
   int32_t root_meta = 0;
   double cmacs[3] = {0, 0, 0};       // per slice, by phase
   uint64_t off_recipe = 0, off_slots = 0, off_leaves = 0, off_wave = 0, off_meta = 0,
            off_counter = 0, off_result = 0, off_scratch = 0, off_acc = 0, off_arena = 0;
   std::vector<uint8_t> program;      // recipes | slots | leaves | level records, copied by pk_grad
+  uint64_t tc_offset() const { return ((uint64_t)arena_elems * 16ull + 255) & ~uint64_t(255); }
   uint64_t ws_bytes(int32_t precision) const {
+    if (precision == PK_C128 && tc64_bytes > 0) return off_arena + tc_offset() + (uint64_t)tc64_bytes;
     return off_arena + (uint64_t)arena_elems * (precision == PK_C64 ? 8ull : 16ull);
   }
 };
@@ -368,6 +404,9 @@ struct Plan {
   int64_t tc_bytes = 0;              // split precision: digit scratch of the largest
                                      // tensor-core step (after the arena)
   int32_t n_tc = 0;                  // tensor-core steps per slice
+  bool use_tc = true;                // made without PK_FLAG_NO_TC
+  int64_t tc64_bytes = 0;            // complex128: digit scratch of the largest tensor-core step
+                                     // (0: every step on the FP64 units)
   uint64_t off_conv = 0;             // byte offset of the ConvRec records (in the program)
   // general networks (PK_FLAG_GRAD or custom weights): every edge group is a tensor
   bool general = false;
@@ -419,19 +458,20 @@ bool wave_light(const Step& s, const pk_tuning& tune);
 // lifetimes [born, dies]; returns the arena's elements.
 int64_t first_fit(const std::vector<int64_t>& elems, const std::vector<int32_t>& born,
                   const std::vector<int32_t>& dies, std::vector<int64_t>& off);
-void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuning& tune, bool breadth,
-                   const std::vector<std::pair<int32_t, int32_t>>* extra, int32_t first_tail,
+void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuning& tune, bool tc64,
+                   bool breadth, const std::vector<std::pair<int32_t, int32_t>>* extra, int32_t first_tail,
                    std::vector<WaveUnit>& units);
 int64_t wave_layout(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
                     const std::vector<char>& pinned, const std::vector<WaveUnit>& units,
                     std::vector<int64_t>& off);
 void wave_hazards(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
                   const std::vector<int64_t>& off, std::vector<std::pair<int32_t, int32_t>>& edges);
-void wave_stages(const std::vector<Step>& steps, WaveProgram& w);
+void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, WaveProgram& w);
 bool wave_check(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
                 const std::vector<char>& pinned, const WaveProgram& w, std::string& err);
 // The plan's level schedule and the workspace layout that holds it; `compact`: on the
-// tensors' offsets of the steps' own order, so that the workspace does not grow.
+// tensors' offsets of the steps' own order and without the complex128 digit scratch, so that
+// the workspace does not grow.
 void plan_waves(Plan& p, bool compact);
 bool valid_tuning(const pk_tuning& t);
 bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& tune, std::string& err);

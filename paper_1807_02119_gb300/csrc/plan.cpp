@@ -1321,6 +1321,7 @@ uint64_t Plan::ws_bytes(int32_t precision) const {
   }
   if (precision == PK_SPLIT && tc_bytes > 0)   // float-float pairs, then the digit scratch
     return off_arena + tc_offset() + (uint64_t)tc_bytes;
+  if (precision == PK_C128 && tc64_bytes > 0) return off_arena + tc_offset() + (uint64_t)tc64_bytes;
   return off_arena + (uint64_t)ws_elems() * 16ull;  // complex128 and float-float pairs
 }
 
@@ -1376,6 +1377,7 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
     return false;
   }
   p.q = q;
+  p.use_tc = !(opts.flags & PK_FLAG_NO_TC);
   p.knot = k;
   const double lq = std::log2((double)q);
   double max_log2 = opts.max_log2_elems > 0 ? opts.max_log2_elems : 31.0;
@@ -1712,9 +1714,10 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
   // the level schedule's layout may not push a plan over the allocation-free entry point's
   // fixed workspace that its own order fits: such a plan keeps a second schedule for it
   for (int32_t prec : {PK_C128, PK_C64, PK_SPLIT})
-    if (!p.compact && p.wave.arena_elems > p.arena_elems && p.ws_bytes(prec) > kNoallocBytes) {
-      const uint64_t own = p.ws_bytes(prec) - (prec == PK_C64 ? 8ull : 16ull) * (uint64_t)(p.wave.arena_elems - p.arena_elems);
-      if (own <= kNoallocBytes + 512) {   // alignment of the scratch behind the arena
+    if (!p.compact && p.ws_bytes(prec) > kNoallocBytes) {
+      const uint64_t grown = 16ull * (uint64_t)std::max<int64_t>(0, p.wave.arena_elems - p.arena_elems) + 512 +
+                             (prec == PK_C128 ? (uint64_t)p.tc64_bytes : 0ull);
+      if (p.ws_bytes(prec) <= kNoallocBytes + grown) {
         auto c = std::make_shared<Plan>(p);
         plan_waves(*c, true);
         p.compact = c;

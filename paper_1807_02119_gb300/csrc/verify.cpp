@@ -235,6 +235,12 @@ bool check_forward(const Plan& p, int32_t precision, Checker& ck) {
   const uint64_t esz = precision == PK_C64 ? 8 : 16;
   uint64_t end = p.off_arena + esz * (uint64_t)p.ws_elems();
   if (precision == PK_SPLIT && p.tc_bytes > 0) end = p.off_arena + p.tc_offset() + (uint64_t)p.tc_bytes;
+  if (precision == PK_C128 && p.tc64_bytes > 0) {
+    end = p.off_arena + p.tc_offset() + (uint64_t)p.tc64_bytes;
+    for (const Step& s : p.steps)
+      if (tc64_step(s) && tc64_scratch(s.Bsz, s.M, s.N, s.K).bytes > p.tc64_bytes)
+        return ck.fail("workspace", "digit scratch larger than the plan reserves");
+  }
   if (precision == PK_C64 && !p.tail.empty()) {
     if (p.off_tail < p.off_arena + 8ull * (uint64_t)p.ws_elems())
       return ck.fail("workspace", "tail region overlaps the arena");

@@ -128,8 +128,8 @@ bool wave_light(const Step& s, const pk_tuning& tune) {
   return exact(s.row, s.nrow) && exact(s.kr, s.nk) && exact(s.nr, s.nn);
 }
 
-void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuning& tune, bool breadth,
-                   const std::vector<std::pair<int32_t, int32_t>>* extra, int32_t first_tail,
+void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuning& tune, bool tc64,
+                   bool breadth, const std::vector<std::pair<int32_t, int32_t>>* extra, int32_t first_tail,
                    std::vector<WaveUnit>& units) {
   const int32_t n = (int32_t)steps.size();
   units.clear();
@@ -152,7 +152,7 @@ void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuni
   std::vector<char> light(n);
   std::vector<int32_t> ready_l, ready_h;
   auto add = [&](int32_t i) { (light[i] ? ready_l : ready_h).push_back(i); };
-  for (int32_t i = 0; i < n; ++i) light[i] = i < first_tail && wave_light(steps[i], tune);
+  for (int32_t i = 0; i < n; ++i) light[i] = i < first_tail && wave_light(steps[i], tune) && !(tc64 && tc64_step(steps[i]));
   for (int32_t i = 0; i < n; ++i)
     if (need[i] == 0) add(i);
   auto finish = [&](int32_t i) {
@@ -286,7 +286,7 @@ bool wave_check(const std::vector<Step>& steps, const std::vector<int64_t>& elem
     size_t u = 0;
     for (const WaveStage& st : stages)
       for (int32_t i = 0; i < st.units; ++i, ++u)
-        if (u >= w.units.size() || w.units[u].heavy != (st.kind == WaveStage::STEP)) {
+        if (u >= w.units.size() || (!w.units[u].heavy && st.kind == WaveStage::STEP)) {
           err = "level schedule: stages do not cover the units";
           return false;
         }
@@ -298,7 +298,7 @@ bool wave_check(const std::vector<Step>& steps, const std::vector<int64_t>& elem
   return true;
 }
 
-void wave_stages(const std::vector<Step>& steps, WaveProgram& w) {
+void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, WaveProgram& w) {
   // records, items and level table of all levels in order
   std::vector<uint8_t> recs;
   std::vector<WaveItem> items;
@@ -307,7 +307,7 @@ void wave_stages(const std::vector<Step>& steps, WaveProgram& w) {
   for (size_t u = 0; u < nu; ++u) {
     lev[u] = (uint32_t)items.size();
     rec_at[u] = (uint32_t)recs.size();
-    if (w.units[u].heavy) continue;
+    if (w.units[u].heavy && !wave_light(steps[w.units[u].steps[0]], tune)) continue;
     for (int32_t i : w.units[u].steps) {
       const uint32_t at = push_record(steps[i], w.off, recs);
       const int64_t outs = steps[i].R * steps[i].N, lanes = outs << lanes_log2(outs, steps[i].K);
@@ -342,7 +342,7 @@ void wave_stages(const std::vector<Step>& steps, WaveProgram& w) {
       WaveStage st;
       st.step = w.units[u].steps[0];
       st.units = 1;
-      if (w.units[u].heavy) {
+      if (w.units[u].heavy && (fp64 || lev[u] == lev[u + 1])) {
         st.kind = WaveStage::STEP;
         out.push_back(st);
         ++u;
@@ -350,7 +350,7 @@ void wave_stages(const std::vector<Step>& steps, WaveProgram& w) {
       }
       int64_t most = lev[u + 1] - lev[u];
       size_t v = u + 1;
-      st.kind = most > fused_max ? WaveStage::WIDE : WaveStage::FUSED;
+      st.kind = most > fused_max || w.units[u].heavy ? WaveStage::WIDE : WaveStage::FUSED;
       if (st.kind == WaveStage::FUSED)
         for (; v < nu && !w.units[v].heavy && lev[v + 1] - lev[v] <= fused_max; ++v)
           most = std::max<int64_t>(most, lev[v + 1] - lev[v]);
@@ -388,6 +388,10 @@ void plan_waves(Plan& p, bool compact) {
   std::vector<char> pinned(n, 0);
   for (int32_t t = 0; t < n; ++t) elems[t] = p.tensors[t].elems;
   pinned[p.final_tensor] = 1;
+  const bool tc64 = p.use_tc && !compact;
+  p.tc64_bytes = 0;
+  for (const Step& s : p.steps)
+    if (tc64 && tc64_step(s)) p.tc64_bytes = std::max<int64_t>(p.tc64_bytes, tc64_scratch(s.Bsz, s.M, s.N, s.K).bytes);
   const int32_t tail = p.conv.empty() && p.tail.empty() ? ns : p.tail_first;
   // breadth first over the heavy steps has the fewest rounds; one heavy step at a time needs
   // about the memory of the steps' own order.  The widening records of a complex128 tail
@@ -399,7 +403,7 @@ void plan_waves(Plan& p, bool compact) {
   else if (limit <= (1 << 30) / 5 * 4)
     limit += limit / 4;
   for (int breadth = 1; breadth >= 0 && !compact && tail == ns; --breadth) {
-    wave_schedule(p.steps, n, p.tuning, breadth != 0, nullptr, ns, w.units);
+    wave_schedule(p.steps, n, p.tuning, tc64, breadth != 0, nullptr, ns, w.units);
     w.arena_elems = wave_layout(p.steps, elems, pinned, w.units, w.off);
     if (w.arena_elems <= limit) break;
     w.off.clear();
@@ -409,9 +413,9 @@ void plan_waves(Plan& p, bool compact) {
     w.arena_elems = p.arena_elems;
     std::vector<std::pair<int32_t, int32_t>> edges;
     wave_hazards(p.steps, elems, w.off, edges);
-    wave_schedule(p.steps, n, p.tuning, false, &edges, tail, w.units);
+    wave_schedule(p.steps, n, p.tuning, tc64, false, &edges, tail, w.units);
   }
-  wave_stages(p.steps, w);
+  wave_stages(p.steps, p.tuning, w);
   // workspace: [recipes | slots | conv | level records] uploaded, then the device's own state
   uint64_t off = p.off_wave;
   off = align256(off + w.blob.size());
