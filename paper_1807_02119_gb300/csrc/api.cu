@@ -71,6 +71,21 @@ pk_status check_ws(pk_ctx* ctx, const pk_plan* p, int32_t precision, void*& ws, 
   return check_ws_need(ctx, p->p.ws_bytes(precision), ws, bytes);
 }
 
+// What pk_upload copies for a precision, in pinned memory (kept with the plan): the program and
+// the precision's level records behind it.  NULL when the allocation fails.
+const uint8_t* pinned_image(const pk_plan* p, int32_t precision, uint64_t& n) {
+  const pk::Plan& P = p->p;
+  const std::vector<uint8_t>& blob = P.wave[precision].blob;
+  n = P.off_wave + blob.size();
+  uint8_t*& pin = const_cast<pk_plan*>(p)->pinned_program[precision];
+  if (!pin) {
+    if (cudaMallocHost((void**)&pin, n + 1) != cudaSuccess) return pin = nullptr;
+    std::memcpy(pin, P.program.data(), P.off_wave);
+    if (!blob.empty()) std::memcpy(pin + P.off_wave, blob.data(), blob.size());
+  }
+  return pin;
+}
+
 // Enqueues the plan's kernels on the context's stream.  The launch sequence is recorded
 // once into a CUDA graph on the context's private capture stream (for this state
 // buffer, arena and precision) and replayed afterwards; very long sequences (many
@@ -88,7 +103,7 @@ pk_status launch_recorded(pk_ctx* ctx, const pk_plan* p, int32_t precision, void
     cudaError_t e = pk::launch_plan_opts(P, precision, ws, arena, ctx->stream, o);
     return e == cudaSuccess ? PK_OK : cuda_fail(ctx, e, "launch");
   }
-  const double nodes = (double)P.n_slices * (double)(P.wave.stages[precision == PK_C128].size() + P.n_tc + 4);
+  const double nodes = (double)P.n_slices * (double)(P.wave[precision].stages[precision == PK_C128].size() + P.n_tc + 4);
   if (nodes > 20000.0) {
     cudaError_t e = pk::launch_plan(P, precision, ws, arena, ctx->stream);
     return e == cudaSuccess ? PK_OK : cuda_fail(ctx, e, "launch");
@@ -418,8 +433,8 @@ pk_status pk_plan_info(const pk_plan* p, pk_plan_stats* out) {
   out->workspace_c128 = P.ws_bytes(PK_C128);
   out->workspace_c64 = P.ws_bytes(PK_C64);
   out->workspace_split = P.ws_bytes(PK_SPLIT);
-  out->n_segments = P.wave.n_fused[1];
-  out->n_segment_steps = P.wave.n_fused_steps[1];
+  out->n_segments = P.wave[PK_C128].n_fused[1];
+  out->n_segment_steps = P.wave[PK_C128].n_fused_steps[1];
   out->est_cost = P.est_cost;
   return PK_OK;
 }
@@ -517,14 +532,14 @@ pk_status pk_plan_launches(const pk_plan* p, int32_t precision, int64_t* launche
   const int64_t widen = (precision == PK_C64 && !P.conv.empty()) ? 1 : 0;
   int64_t digits = 0;   // split and complex128: one conversion launch per tensor-core step
   if (precision == PK_C128 && P.tc64_bytes > 0)
-    for (const pk::WaveStage& g : P.wave.stages[1])
+    for (const pk::WaveStage& g : P.wave[PK_C128].stages[1])
       digits += g.kind == pk::WaveStage::STEP && pk::tc64_step(P.steps[g.step]);
   if (precision == PK_SPLIT)
-    for (const pk::WaveStage& g : P.wave.stages[0])
+    for (const pk::WaveStage& g : P.wave[PK_SPLIT].stages[0])
       digits += g.kind == pk::WaveStage::STEP && P.steps[g.step].tc;
   // steps saved by the level launches (a complex128 tail's steps are never inside one)
   const int fp64 = precision == PK_C128;
-  const int64_t fused = P.wave.n_fused_steps[fp64] - P.wave.n_fused[fp64];
+  const int64_t fused = P.wave[precision].n_fused_steps[fp64] - P.wave[precision].n_fused[fp64];
   *launches = P.n_slices * ((P.n_init > 0 ? 1 : 0) + (int64_t)P.steps.size() - fused + 1 + widen +
                             digits) + 1;
   return PK_OK;
@@ -532,7 +547,8 @@ pk_status pk_plan_launches(const pk_plan* p, int32_t precision, int64_t* launche
 
 void pk_plan_destroy(pk_plan* p) {
   if (!p) return;
-  if (p->pinned_program) cudaFreeHost(p->pinned_program);
+  for (uint8_t* pin : p->pinned_program)
+    if (pin) cudaFreeHost(pin);
   if (p->pinned_grad) cudaFreeHost(p->pinned_grad);
   if (p->graph.exec) cudaGraphExecDestroy(p->graph.exec);
   if (p->grad_graph.exec) cudaGraphExecDestroy(p->grad_graph.exec);
@@ -550,16 +566,10 @@ pk_status pk_upload(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_wo
   else if (workspace_bytes < p->p.off_arena)
     s = fail(ctx, PK_ENOMEM, "buffer smaller than the plan state (pk_plan_state_bytes)");
   if (s != PK_OK) return s;
-  const pk::Plan& P = p->p;
-  if (P.program.empty()) return PK_OK;
-  pk_plan* mp = const_cast<pk_plan*>(p);
-  if (!mp->pinned_program) {
-    if (cudaMallocHost((void**)&mp->pinned_program, P.program.size()) != cudaSuccess)
-      return fail(ctx, PK_ENOMEM, "pinned host allocation failed");
-    std::memcpy(mp->pinned_program, P.program.data(), P.program.size());
-  }
-  cudaError_t e = cudaMemcpyAsync(d_workspace, mp->pinned_program, P.program.size(),
-                                  cudaMemcpyHostToDevice, ctx->stream);
+  uint64_t n = 0;
+  const uint8_t* image = pinned_image(p, precision, n);
+  if (!image) return fail(ctx, PK_ENOMEM, "pinned host allocation failed");
+  cudaError_t e = cudaMemcpyAsync(d_workspace, image, n, cudaMemcpyHostToDevice, ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "upload");
   return PK_OK;
 }
@@ -580,14 +590,10 @@ pk_status pk_upload_inputs(pk_ctx* ctx, const pk_plan* p, int32_t precision, voi
   const uint64_t n = std::min<uint64_t>(P.off_conv, P.program.size());
   if (copied) *copied = n;
   if (n == 0) return PK_OK;
-  pk_plan* mp = const_cast<pk_plan*>(p);
-  if (!mp->pinned_program) {
-    if (cudaMallocHost((void**)&mp->pinned_program, P.program.size()) != cudaSuccess)
-      return fail(ctx, PK_ENOMEM, "pinned host allocation failed");
-    std::memcpy(mp->pinned_program, P.program.data(), P.program.size());
-  }
-  cudaError_t e = cudaMemcpyAsync(d_workspace, mp->pinned_program, n, cudaMemcpyHostToDevice,
-                                  ctx->stream);
+  uint64_t whole = 0;
+  const uint8_t* image = pinned_image(p, precision, whole);
+  if (!image) return fail(ctx, PK_ENOMEM, "pinned host allocation failed");
+  cudaError_t e = cudaMemcpyAsync(d_workspace, image, n, cudaMemcpyHostToDevice, ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "upload");
   return PK_OK;
 }
@@ -772,7 +778,8 @@ pk_status pk_group_upload(pk_ctx* ctx, pk_group* grp, int32_t inputs_only, uint6
   if (!ctx || !grp) return fail(ctx, PK_EINVAL, "bad argument");
   uint64_t total = 0;
   for (int32_t i = 0; i < grp->n; ++i) {
-    uint64_t n = grp->plans[i]->p.program.size();
+    const pk::Plan& P = grp->plans[i]->p;
+    uint64_t n = P.off_wave + P.wave[grp->precision].blob.size();
     const pk_status s =
         inputs_only ? pk_upload_inputs(ctx, grp->plans[i], grp->precision, grp->ws[i], grp->ws_bytes[i], &n)
                     : pk_upload(ctx, grp->plans[i], grp->precision, grp->ws[i], grp->ws_bytes[i]);
@@ -1007,10 +1014,11 @@ pk_status pk_grad_weights(const pk_plan* p, const double* dlogZ_dT, double* out)
 pk_status pk_plan_set_weights(pk_plan* p, const double* edge_weights) {
   if (!p || !p->p.general) return PK_EINVAL;
   if (!pk::set_weights(p->p, edge_weights)) return PK_EINVAL;
-  if (p->pinned_program) {  // refilled from the new program by the next pk_upload
-    cudaFreeHost(p->pinned_program);
-    p->pinned_program = nullptr;
-  }
+  for (uint8_t*& pin : p->pinned_program)   // refilled from the new program by the next pk_upload
+    if (pin) {
+      cudaFreeHost(pin);
+      pin = nullptr;
+    }
   return PK_OK;
 }
 
@@ -1128,9 +1136,29 @@ namespace {
 constexpr int64_t kExactMaxSlices = 1000000;
 
 bool is_prime32(uint32_t p) {
-  if (p < 2) return false;
-  for (uint32_t d = 2; (uint64_t)d * d <= p; ++d)
-    if (p % d == 0) return false;
+  // Miller-Rabin with the bases 2, 3, 5, 7: exact below 3 215 031 751 (Pomerance, Selfridge and
+  // Wagstaff 1980); trial division took 0.2 ms per modulus
+  if (p < 11) return p == 2 || p == 3 || p == 5 || p == 7;
+  if (p % 2 == 0) return false;
+  if (p >= 3215031751u) {
+    for (uint32_t d = 3; (uint64_t)d * d <= p; d += 2)
+      if (p % d == 0) return false;
+    return true;
+  }
+  uint32_t d = p - 1;
+  int s = 0;
+  for (; d % 2 == 0; d /= 2) ++s;
+  for (uint32_t a : {2u, 3u, 5u, 7u}) {
+    uint64_t x = 1, b = a;
+    for (uint32_t m = d; m; m /= 2, b = b * b % p)
+      if (m & 1) x = x * b % p;
+    bool ok = x == 1 || x == p - 1;
+    for (int i = 1; i < s && !ok; ++i) {
+      x = x * x % p;
+      ok = x == p - 1;
+    }
+    if (!ok) return false;
+  }
   return true;
 }
 
@@ -1138,15 +1166,23 @@ bool is_prime32(uint32_t p) {
 pk_status exact_residues(pk_ctx* ctx, const pk_plan* p, const uint32_t* primes, int32_t n_primes,
                          void* ws, uint32_t* zab) {
   const pk::Plan& P = p->p;
+  // as many primes per wait as the pinned record holds residues
+  constexpr int32_t kPer = (int32_t)(sizeof(pk::SliceResult) / sizeof(pk::exact::E));
   for (int32_t i = 0; i < n_primes; ++i) {
-    void* sum = (char*)ws + P.off_result;
-    cudaError_t e = pk::launch_exact(P, primes[i], ws, (char*)ws + P.off_arena, sum, ctx->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(ctx->pinned_result, sum, sizeof(pk::exact::E), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "exact evaluation");
+    if (i % kPer == 0) {
+      cudaError_t e = cudaSuccess;
+      for (int32_t j = i; e == cudaSuccess && j < std::min(n_primes, i + kPer); ++j) {
+        void* sum = (char*)ws + P.off_result;
+        e = pk::launch_exact(P, primes[j], ws, (char*)ws + P.off_arena, sum, ctx->stream);
+        if (e == cudaSuccess)
+          e = cudaMemcpyAsync((pk::exact::E*)ctx->pinned_result + (j - i), sum, sizeof(pk::exact::E),
+                              cudaMemcpyDeviceToHost, ctx->stream);
+      }
+      if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+      if (e != cudaSuccess) return cuda_fail(ctx, e, "exact evaluation");
+    }
     pk::exact::E z;
-    std::memcpy(&z, ctx->pinned_result, sizeof(z));
+    std::memcpy(&z, (pk::exact::E*)ctx->pinned_result + i % kPer, sizeof(z));
     const pk::exact::Ring r = pk::exact::make_ring(primes[i], P.q);
     pk::exact::E f = pk::exact::epow_t(-(long long)P.loop_signsum, r);  // folded loops
     if (P.loop_count & 1) f = pk::exact::eneg(f, r);

@@ -198,6 +198,7 @@ __device__ __forceinline__ void digits64_block(const Step& s, const Cx<double>* 
 // Blocks [0, nA) convert A, the rest B.
 __global__ void __launch_bounds__(d64::kConvThreads) k_digits64(const Step s, const Cx<double>* arena,
                                                                 unsigned char* scratch, long long nA) {
+  pdl_wait();
   __shared__ unsigned kt[kTc64MaxK], mx[kTcMc];
   __shared__ long long ro[kTcMc];
   const long long blk = blockIdx.x;
@@ -242,6 +243,7 @@ __device__ __forceinline__ unsigned long long to_double_bits(long long h, long l
 __global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const Step s, Cx<double>* arena, Meta* meta,
                                                              const unsigned char* scratch,
                                                              unsigned long long* err) {
+  pdl_wait();
   using namespace d64;
   using tc::bulk_g2s;
   using tc::commit;

@@ -453,6 +453,7 @@ __device__ __forceinline__ void digits_block(const Step& s, const Cx<ff>* arena,
 template <int S>
 __global__ void __launch_bounds__(tc::kConvThreads, 4) k_digits(const Step s, const Cx<ff>* arena,
                                                              unsigned char* scratch, long long nA) {
+  pdl_wait();
   __shared__ long long ro[32], kt[tc::kConvThreads];
   __shared__ long long base;
   __shared__ int ex[32];
@@ -487,6 +488,7 @@ __global__ void __launch_bounds__(tc::kThreads, DB ? 1 : 2) k_gemm_tc(const Step
                                                                       const unsigned char* scratch,
                                                                       unsigned* ticket,
                                                                       unsigned long long* err) {
+  pdl_wait();
   using namespace tc;
   constexpr int kSt = DB ? kStagesDB : kStages;     // stages of the ring
   constexpr int kTq = 4;                            // tile queue: tiles handed out ahead

@@ -187,6 +187,13 @@ struct Acc<ff> {
   }
 };
 
+// ---- programmatic dependent launch: the kernels of a launch sequence start while the one
+// before still runs and wait for its results here.  Every kernel of a sequence waits, so each
+// one's end implies the end of all before it.  Short kernels let the next one start at once;
+// long ones do not (its CTAs would hold their place on the GPU all the while).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 // ---- bookkeeping
 __device__ __forceinline__ unsigned long long max_bits(double m) {
   return (unsigned long long)__double_as_longlong(m);
@@ -241,9 +248,10 @@ __device__ __forceinline__ void recipe_value(const Recipe& r, const Slot* slots,
     sre = 1;
     return;
   }
+  bool any = false;   // the first factor and the first term are taken as they are: FP64 is slow here
   for (int s = 0; s < q; ++s) {
     double pre = 1, pim = 0;
-    bool zero = false;
+    bool zero = false, one = true;
     for (int j = 0; j < r.nslot; ++j) {
       const Slot sl = slots[r.slot0 + j];
       int x;
@@ -256,18 +264,20 @@ __device__ __forceinline__ void recipe_value(const Recipe& r, const Slot* slots,
       }
       if (sl.absorbed) {
         const double fre = s == x ? sl.dre : sl.ore, fim = s == x ? sl.dim : sl.oim;
-        const double nre = pre * fre - pim * fim;
-        const double nim = pre * fim + pim * fre;
+        const double nre = one ? fre : pre * fre - pim * fim;
+        const double nim = one ? fim : pre * fim + pim * fre;
         pre = nre;
         pim = nim;
+        one = false;
       } else if (s != x) {
         zero = true;
         break;
       }
     }
     if (!zero) {
-      sre += pre;
-      sim += pim;
+      sre = any ? sre + pre : pre;
+      sim = any ? sim + pim : pim;
+      any = true;
     }
   }
 }
@@ -279,6 +289,8 @@ __global__ void __launch_bounds__(256) k_build(const Recipe* __restrict__ rec,
                                                const Slot* __restrict__ slots,
                                                const int64_t* __restrict__ offs, Cx<R>* arena,
                                                Meta* meta, int q, long long slice, int n_sliced) {
+  pdl_next();
+  pdl_wait();
   using S = typename Traits<R>::S;
   const Recipe r = rec[blockIdx.y];
   Cx<R>* dst = arena + (offs ? (long long)offs[blockIdx.y] : (long long)r.offset);
@@ -355,6 +367,7 @@ __device__ __forceinline__ S step_scale(const Step& s, Meta* meta, bool write_ex
 // Consecutive threads take consecutive rows, so the C stores of a warp are contiguous.
 template <typename R, int KREG>
 __global__ void __launch_bounds__(256) k_rows(const Step s, Cx<R>* arena, Meta* meta, int nc) {
+  pdl_wait();
   using S = typename Traits<R>::S;
   extern __shared__ long long sm[];
   long long* kA = sm;
@@ -427,6 +440,7 @@ __global__ void __launch_bounds__(256) k_rows(const Step s, Cx<R>* arena, Meta* 
 // n * R + r is the thread's linear index).
 template <typename R>
 __global__ void __launch_bounds__(256) k_outs(const Step s, Cx<R>* arena, Meta* meta) {
+  pdl_wait();
   using S = typename Traits<R>::S;
   extern __shared__ long long sm[];
   long long* kA = sm;
@@ -467,6 +481,7 @@ __global__ void __launch_bounds__(256) k_outs(const Step s, Cx<R>* arena, Meta* 
 // offset is recomputed from the stride runs.
 template <typename R>
 __global__ void __launch_bounds__(256) k_rows_big(const Step s, Cx<R>* arena, Meta* meta) {
+  pdl_wait();
   using S = typename Traits<R>::S;
   const S scale = step_scale<S>(s, meta, blockIdx.x == 0 && threadIdx.x == 0);
   const Cx<R>* A = arena + s.off_a;
@@ -523,6 +538,7 @@ __device__ __forceinline__ void runs4(long long x, const Run4* r, int n, long lo
 
 template <typename R>
 __global__ void __launch_bounds__(256) k_gemm(const Step s, Cx<R>* arena, Meta* meta) {
+  pdl_wait();
   using S = typename Traits<R>::S;
   constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4, LDA = BM + 1, LDB = BN + 1;
   __shared__ Cx<R> As[BK * LDA];
@@ -644,6 +660,7 @@ __global__ void __launch_bounds__(256) k_gemm(const Step s, Cx<R>* arena, Meta* 
 template <typename R>
 __global__ void __launch_bounds__(256) k_splitk(const Step s, Cx<R>* arena, Meta* meta,
                                                 Cx<double>* partial, unsigned* counter) {
+  pdl_wait();
   using S = typename Traits<R>::S;
   const int chunks = s.chunks;
   const long long o = blockIdx.y;
@@ -739,6 +756,8 @@ __global__ void __launch_bounds__(256) k_splitk(const Step s, Cx<R>* arena, Meta
 template <typename R>
 __global__ void k_slice_result(const Cx<R>* arena, long long off, const Meta* meta, int tensor,
                                SliceResult* out, long long slice) {
+  pdl_next();
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const Cx<R> v = arena[off];
   out[slice].re = to_double(v.re);
@@ -756,6 +775,8 @@ __global__ void __launch_bounds__(256) k_grad_accum(const GradLeaf* __restrict__
                                                     const Cx<R>* arena, const Meta* meta,
                                                     Cx<double>* acc, long long* acc_exp, int q,
                                                     long long slice) {
+  pdl_next();
+  pdl_wait();
   const GradLeaf L = leaves[blockIdx.x];
   int sdig[2] = {0, 0};
   for (int j = 0; j < 2; ++j)
@@ -815,6 +836,23 @@ __global__ void __launch_bounds__(256) k_grad_accum(const GradLeaf* __restrict__
 
 // Sum over slices in double with a common exponent; fixed assignment and tree order.
 static __global__ void k_sum_slices(SliceResult* res, long long n) {
+  pdl_wait();
+  if (n == 1) {   // one slice: its value at the exponent the sum below would give it
+    if (threadIdx.x == 0) {
+      const SliceResult r = res[0];
+      const double m = fmax(fabs(r.re), fabs(r.im));
+      if (!isfinite(r.re) || !isfinite(r.im)) {
+        res[1].re = res[1].im = __longlong_as_double(0x7FF8000000000000LL);
+        res[1].exp = 0;
+      } else if (m > 0) {
+        const int e = bin_exp(m);
+        res[1].re = ldexp(r.re, -e);
+        res[1].im = ldexp(r.im, -e);
+        res[1].exp = r.exp + e;
+      }   // 0: the record was cleared
+    }
+    return;
+  }
   __shared__ long long emax_s[256];
   __shared__ double sre[256], sim[256];
   long long emax = LLONG_MIN;

@@ -138,6 +138,7 @@ struct Marker {
     else
       cudaEventRecord(e, st);
   }
+  bool pdl() const { return prof == nullptr; }   // event pairs time each launch by itself
   void begin(int c, double cm, double by, double fill) {
     if (nvtx) nvtxRangePushA(("step " + std::to_string(step) + " " + kClassName[c]).c_str());
     if (!prof) return;
@@ -181,7 +182,7 @@ cudaError_t launch_rows(const Step& s, Cx<R>* arena, Meta* meta, cudaStream_t st
     const long long outs = s.R * s.N;
     const long long blocks = std::max<long long>(1, std::min<long long>((outs + 255) / 256, 152 * 16));
     mk.begin(1, cm, by, gpu_fill(blocks, 8));
-    k_outs<R><<<(unsigned)blocks, 256, sizeof(long long) * 2 * (size_t)s.K, st>>>(s, arena, meta);
+    launch_kernel(k_outs<R>, dim3((unsigned)blocks), 256, sizeof(long long) * 2 * (size_t)s.K, st, mk.pdl(), 1, s, arena, meta);
     mk.end();
     return cudaGetLastError();
   }
@@ -190,7 +191,7 @@ cudaError_t launch_rows(const Step& s, Cx<R>* arena, Meta* meta, cudaStream_t st
   blocks = std::max<long long>(1, std::min<long long>(blocks, 152 * 8));
   mk.begin(1, cm, by, gpu_fill(blocks, 8));
   if (sm > 200 * 1024) {
-    k_rows_big<R><<<(unsigned)blocks, 256, 0, st>>>(s, arena, meta);
+    launch_kernel(k_rows_big<R>, dim3((unsigned)blocks), 256, 0, st, mk.pdl(), 1, s, arena, meta);
     mk.end();
     return cudaGetLastError();
   }
@@ -210,7 +211,7 @@ cudaError_t launch_rows(const Step& s, Cx<R>* arena, Meta* meta, cudaStream_t st
     fn = k_rows<R, 32>;
   else
     fn = k_rows<R, 0>;
-  fn<<<(unsigned)blocks, 256, sm, st>>>(s, arena, meta, nc);  // limit raised by prepare_kernels
+  launch_kernel(fn, dim3((unsigned)blocks), 256, sm, st, mk.pdl(), 1, s, arena, meta, nc);  // limit raised by prepare_kernels
   mk.end();
   return cudaGetLastError();
 }
@@ -229,7 +230,7 @@ cudaError_t launch_tc(const Step& s, Cx<ff>* arena, Meta* meta, unsigned char* t
                   nB = s.Bsz * L.tiles_n * L.groups;
   mk.begin(6, 0.0, (double)sizeof(Cx<ff>) * (double)(s.R * s.K + s.Bsz * s.K * s.N),
            gpu_fill(nA + nB, 4));   // 4 CTAs per SM (64 registers x 256 threads)
-  k_digits<S><<<(unsigned)(nA + nB), tc::kConvThreads, tc::Cfg<S>::kConvSmem, stream>>>(s, arena, tcs, nA);
+  launch_kernel(k_digits<S>, dim3((unsigned)(nA + nB)), tc::kConvThreads, tc::Cfg<S>::kConvSmem, stream, mk.pdl(), 1, s, arena, tcs, nA);
   mk.end();
   // persistent: at most one CTA per tile slot of the GPU, each looping over its tiles;
   // tiles of steps with at most two flush groups come from the tile counter
@@ -239,19 +240,19 @@ cudaError_t launch_tc(const Step& s, Cx<ff>* arena, Meta* meta, unsigned char* t
     const long long grid = std::min<long long>(tc_tiles, (long long)g_sms);
     mk.begin(5, cm, by, gpu_fill(grid, 1));
     if (q)
-      k_gemm_tc<S, true, true><<<(unsigned)grid, tc::kThreads, tc::Cfg<S>::kSmemDB, stream>>>(
+      launch_kernel(k_gemm_tc<S, true, true>, dim3((unsigned)grid), tc::kThreads, tc::Cfg<S>::kSmemDB, stream, mk.pdl(), 1, 
           s, arena, meta, tcs, ticket, err);
     else
-      k_gemm_tc<S, true, false><<<(unsigned)grid, tc::kThreads, tc::Cfg<S>::kSmemDB, stream>>>(
+      launch_kernel(k_gemm_tc<S, true, false>, dim3((unsigned)grid), tc::kThreads, tc::Cfg<S>::kSmemDB, stream, mk.pdl(), 1, 
           s, arena, meta, tcs, ticket, err);
   } else {
     const long long grid = std::min<long long>(tc_tiles, 2LL * g_sms);
     mk.begin(5, cm, by, gpu_fill(grid, 2));
     if (q)
-      k_gemm_tc<S, false, true><<<(unsigned)grid, tc::kThreads, tc::Cfg<S>::kSmem, stream>>>(
+      launch_kernel(k_gemm_tc<S, false, true>, dim3((unsigned)grid), tc::kThreads, tc::Cfg<S>::kSmem, stream, mk.pdl(), 1, 
           s, arena, meta, tcs, ticket, err);
     else
-      k_gemm_tc<S, false, false><<<(unsigned)grid, tc::kThreads, tc::Cfg<S>::kSmem, stream>>>(
+      launch_kernel(k_gemm_tc<S, false, false>, dim3((unsigned)grid), tc::kThreads, tc::Cfg<S>::kSmem, stream, mk.pdl(), 1, 
           s, arena, meta, tcs, ticket, err);
   }
   mk.end();
@@ -265,11 +266,11 @@ cudaError_t launch_tc64(const Step& s, Cx<double>* arena, Meta* meta, unsigned c
   const long long nA = s.Bsz * L.tiles_m * (kTcMc / 8 / d64_groups(L.chunks, kTcMc / 8)),
                   nB = s.Bsz * L.tiles_n * (kTc64Nc / 8 / d64_groups(L.chunks, kTc64Nc / 8));
   mk.begin(6, 0.0, 16.0 * (double)(s.R * s.K + s.Bsz * s.K * s.N), gpu_fill(nA + nB, 8));
-  k_digits64<<<(unsigned)(nA + nB), d64::kConvThreads, 0, stream>>>(s, arena, tcs, nA);
+  launch_kernel(k_digits64, dim3((unsigned)(nA + nB)), d64::kConvThreads, 0, stream, mk.pdl(), 1, s, arena, tcs, nA);
   mk.end();
   const long long grid = std::min<long long>(L.tiles_m * L.tiles_n * s.Bsz, (long long)g_sms);
   mk.begin(5, cm, by, gpu_fill(grid, 1));
-  k_gemm64<<<(unsigned)grid, d64::kThreads, d64::kSmem, stream>>>(s, arena, meta, tcs, err);
+  launch_kernel(k_gemm64, dim3((unsigned)grid), d64::kThreads, d64::kSmem, stream, mk.pdl(), 1, s, arena, meta, tcs, err);
   mk.end();
   return cudaGetLastError();
 }
@@ -293,12 +294,12 @@ cudaError_t launch_step(const Step& s, Cx<R>* arena, Meta* meta, Cx<double>* par
   }
   if (s.kernel == KGEMM && gemm_tiles < (1LL << 31)) {
     mk.begin(4, cm, by, gpu_fill(gemm_tiles, 8));
-    k_gemm<R><<<(unsigned)gemm_tiles, 256, 0, stream>>>(s, arena, meta);
+    launch_kernel(k_gemm<R>, dim3((unsigned)gemm_tiles), 256, 0, stream, mk.pdl(), 1, s, arena, meta);
     mk.end();
     e = cudaGetLastError();
   } else if (s.kernel == KSPLITK) {
     mk.begin(2, cm, by, gpu_fill((long long)s.chunks * s.R * s.N, 8));
-    k_splitk<R><<<dim3((unsigned)s.chunks, (unsigned)(s.R * s.N)), 256, 0, stream>>>(
+    launch_kernel(k_splitk<R>, dim3((unsigned)s.chunks, (unsigned)(s.R * s.N)), 256, 0, stream, mk.pdl(), 1, 
         s, arena, meta, partial, counter);
     mk.end();
     e = cudaGetLastError();
@@ -312,8 +313,6 @@ double step_bytes(const Plan& p, const Step& s, double elem_bytes) {
   return elem_bytes * (double)(p.tensors[s.a].elems + (s.b >= 0 ? p.tensors[s.b].elems : 0) +
                                p.tensors[s.c].elems);
 }
-
-constexpr uint32_t kWaveSmem = 100 * 1024;   // a level launch's records in shared memory: two CTAs per SM
 
 // One launch of the level schedule `w` (records at `blob` on the device); `steps` are the
 // steps it orders, its heavy ones launched alone on their offsets under the schedule.
@@ -335,27 +334,20 @@ cudaError_t launch_stage(const WaveProgram& w, const WaveStage& g, const std::ve
     const int64_t wpb = std::max<int64_t>(1, std::min<int64_t>(8, g.items / (2LL * g_sms)));
     const unsigned grid = (unsigned)((g.items + wpb - 1) / wpb);
     mk.begin(1, cm, by, gpu_fill(grid, 8));
-    k_wave_wide<R><<<grid, 32 * (unsigned)wpb, 0, stream>>>(blob, g.range, g.first, (unsigned)g.items, arena, meta);
+    launch_kernel(k_wave_wide<R>, dim3(grid), 32 * (unsigned)wpb, 0, stream, mk.pdl(), 1, blob, g.range, g.first, (unsigned)g.items, arena, meta);
     mk.end();
     return cudaGetLastError();
   }
   mk.begin(1, cm, by, gpu_fill(g.ctas, 2));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)g.ctas);
-  cfg.blockDim = dim3(32 * kWaveCtaWarps);
-  cfg.stream = stream;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = (unsigned)g.ctas;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  const uint32_t prog = g.range.rec_bytes + g.range.item_bytes + g.range.lev_bytes;
-  const int smem = prog <= kWaveSmem ? (int)prog : 0;
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_waves<R>, blob, g.range, (int)g.units, smem, arena, meta);
+  cudaError_t e = launch_cluster(g, blob, stream, mk.pdl(), g.ctas == 1 ? k_waves<R, kWaveOwn> : k_waves<R, kWaveL2>, arena, meta);
   mk.end();
   return e;
+}
+
+// The pk_precision whose storage type is R.
+template <typename R>
+constexpr int32_t precision_of() {
+  return std::is_same<R, double>::value ? PK_C128 : std::is_same<R, float>::value ? PK_C64 : PK_SPLIT;
 }
 
 // Steps [first, last) of the plan, all in storage type R: through the level schedule, or (the
@@ -372,7 +364,8 @@ cudaError_t launch_bulk(const Plan& p, char* base, char* arena_base, int32_t fir
   unsigned char* tcs = digits ? (unsigned char*)arena_base + p.tc_offset() : nullptr;
   unsigned long long* err = &((SliceResult*)(base + p.off_result))[p.n_slices].status;
   if (!o.check_finite) {
-    for (const WaveStage& g : p.wave.stages[std::is_same<R, double>::value]) {
+    const WaveProgram& w = p.wave[precision_of<R>()];
+    for (const WaveStage& g : w.stages[std::is_same<R, double>::value]) {
       if (g.step >= last) break;   // the complex128 tail's steps come last
       double cm = 0, by = 0;
       if (g.kind == WaveStage::STEP)
@@ -381,7 +374,7 @@ cudaError_t launch_bulk(const Plan& p, char* base, char* arena_base, int32_t fir
         cm += (double)p.steps[j].R * (double)p.steps[j].K * (double)p.steps[j].N;
         by += step_bytes(p, p.steps[j], (double)sizeof(Cx<R>));
       }
-      cudaError_t e = launch_stage<R>(p.wave, g, p.steps, (const unsigned char*)base + p.off_wave, arena,
+      cudaError_t e = launch_stage<R>(w, g, p.steps, (const unsigned char*)base + p.off_wave, arena,
                                       meta, partial, counters, tcs, err, p.tuning.tc_db_groups, stream, mk,
                                       cm, by);
       if (e != cudaSuccess) return e;
@@ -414,9 +407,9 @@ cudaError_t launch_build(const Plan& p, char* base, char* arena_base, long long 
   const unsigned bx = (unsigned)std::min<int64_t>((maxel + 255) / 256, 64);
   mk.step = -1;
   mk.begin(0, 0, (double)sizeof(Cx<R>) * (double)initel, gpu_fill((long long)bx * p.n_init, 8));
-  k_build<R><<<dim3(bx, (unsigned)p.n_init), 256, 0, stream>>>(
+  launch_kernel(k_build<R>, dim3(bx, (unsigned)p.n_init), 256, 0, stream, false, 1, 
       (const Recipe*)(base + p.off_recipe), (const Slot*)(base + p.off_slots),
-      o.check_finite ? nullptr : (const int64_t*)(base + p.off_wave + p.wave.init_off),
+      o.check_finite ? nullptr : (const int64_t*)(base + p.off_wave + p.wave[precision_of<R>()].init_off),
       (Cx<R>*)arena_base, (Meta*)(base + p.off_meta), p.q, sl, (int)p.sliced.size());
   mk.end();
   cudaError_t e = cudaGetLastError();
@@ -436,7 +429,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
   char* base = (char*)ws;
   char* arena_base = (char*)arena;
   Marker mk{prof, stream, o.nvtx};
-  const long long final_off = o.check_finite ? p.tensors[p.final_tensor].offset : p.wave.off[p.final_tensor];
+  const long long final_off = o.check_finite ? p.tensors[p.final_tensor].offset : p.wave[precision].off[p.final_tensor];
   SliceResult* res = (SliceResult*)(base + p.off_result);
   const int32_t n_steps = (int32_t)p.steps.size();
   const long long first = o.slice_first;
@@ -456,7 +449,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
       if ((e = launch_bulk<double>(p, base, arena_base, 0, n_steps, stream, mk, o, sl)) != cudaSuccess) return e;
       mk.step = -1;
       mk.begin(3, 0, 0, gpu_fill(1, 8));
-      k_slice_result<double><<<1, 32, 0, stream>>>((Cx<double>*)arena_base, final_off,
+      launch_kernel(k_slice_result<double>, dim3(1), 32, 0, stream, mk.pdl(), 1, (Cx<double>*)arena_base, final_off,
                                                    (Meta*)(base + p.off_meta), p.final_tensor, res, sl);
       mk.end();
     } else if (precision == PK_SPLIT) {
@@ -464,7 +457,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
       if ((e = launch_bulk<ff>(p, base, arena_base, 0, n_steps, stream, mk, o, sl)) != cudaSuccess) return e;
       mk.step = -1;
       mk.begin(3, 0, 0, gpu_fill(1, 8));
-      k_slice_result<ff><<<1, 32, 0, stream>>>((Cx<ff>*)arena_base, final_off,
+      launch_kernel(k_slice_result<ff>, dim3(1), 32, 0, stream, mk.pdl(), 1, (Cx<ff>*)arena_base, final_off,
                                                (Meta*)(base + p.off_meta), p.final_tensor, res, sl);
       mk.end();
     } else if (p.tail.empty() && p.conv.empty()) {  // complex64
@@ -472,7 +465,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
       if ((e = launch_bulk<float>(p, base, arena_base, 0, n_steps, stream, mk, o, sl)) != cudaSuccess) return e;
       mk.step = -1;
       mk.begin(3, 0, 0, gpu_fill(1, 8));
-      k_slice_result<float><<<1, 32, 0, stream>>>((Cx<float>*)arena_base, final_off,
+      launch_kernel(k_slice_result<float>, dim3(1), 32, 0, stream, mk.pdl(), 1, (Cx<float>*)arena_base, final_off,
                                                   (Meta*)(base + p.off_meta), p.final_tensor, res, sl);
       mk.end();
     } else {  // complex64 with a complex128 tail
@@ -508,7 +501,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
       }
       mk.step = -1;
       mk.begin(3, 0, 0, gpu_fill(1, 8));
-      k_slice_result<double><<<1, 32, 0, stream>>>(tail, p.final_tail_off, meta, p.final_tensor,
+      launch_kernel(k_slice_result<double>, dim3(1), 32, 0, stream, mk.pdl(), 1, tail, p.final_tail_off, meta, p.final_tensor,
                                                    res, sl);
       mk.end();
     }
@@ -516,7 +509,7 @@ cudaError_t launch_impl(const Plan& p, int32_t precision, void* ws, void* arena,
   }
   mk.step = -1;
   mk.begin(3, 0, 0, gpu_fill(1, 8));
-  k_sum_slices<<<1, 256, 0, stream>>>(res, p.n_slices);
+  launch_kernel(k_sum_slices, dim3(1), 256, 0, stream, mk.pdl(), 1, res, p.n_slices);
   mk.end();
   return cudaGetLastError();
 }
@@ -549,7 +542,7 @@ cudaError_t launch_grad_impl(const Plan& p, char* base, cudaStream_t stream) {
     e = cudaMemsetAsync(base + G.off_meta, 0, (sl == 0 ? G.off_scratch : G.off_result) - G.off_meta, stream);
     if (e != cudaSuccess) return e;
     if (p.n_init > 0) {
-      k_build<R><<<dim3(bx, (unsigned)p.n_init), 256, 0, stream>>>(
+      launch_kernel(k_build<R>, dim3(bx, (unsigned)p.n_init), 256, 0, stream, false, 1, 
           (const Recipe*)(base + G.off_recipe), (const Slot*)(base + G.off_slots), nullptr, arena, meta,
           p.q, sl, (int)p.sliced.size());
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -559,13 +552,13 @@ cudaError_t launch_grad_impl(const Plan& p, char* base, cudaStream_t stream) {
                           counters, tcs, &res[p.n_slices].status, 0, stream, mk, 0.0, 0.0);
       if (e != cudaSuccess) return e;
     }
-    k_slice_result<R><<<1, 32, 0, stream>>>(arena, G.root_offset, meta, G.root_meta, res, sl);
+    launch_kernel(k_slice_result<R>, dim3(1), 32, 0, stream, mk.pdl(), 1, arena, G.root_offset, meta, G.root_meta, res, sl);
     if (!G.leaves.empty())
-      k_grad_accum<R><<<(unsigned)G.leaves.size(), 256, 0, stream>>>(
+      launch_kernel(k_grad_accum<R>, dim3((unsigned)G.leaves.size()), 256, 0, stream, mk.pdl(), 1, 
           (const GradLeaf*)(base + G.off_leaves), arena, meta, acc, acc_exp, p.q, sl);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  k_sum_slices<<<1, 256, 0, stream>>>(res, p.n_slices);
+  launch_kernel(k_sum_slices, dim3(1), 256, 0, stream, mk.pdl(), 1, res, p.n_slices);
   return cudaGetLastError();
 }
 
@@ -582,7 +575,9 @@ cudaError_t raise_rows_smem() {
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     if (e != cudaSuccess) return e;
   }
-  cudaError_t e = cudaFuncSetAttribute(k_waves<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWaveSmem);
+  cudaError_t e = cudaFuncSetAttribute(k_waves<R, kWaveL2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWaveSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_waves<R, kWaveOwn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWaveSmem);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_outs<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }

@@ -174,7 +174,8 @@ struct WaveRec {
   uint32_t N, K, mul_r;    // mul_r: the division by R
   uint8_t nrow, nk, nn, lanes;   // lanes: log2 of the lanes that share one output's sum
   int64_t off_a, off_b;
-  int64_t off_c, pad;
+  int64_t off_c;
+  uint32_t per, pad;       // chunks of 32 lanes per item (1 but for the batch executor's large steps)
 };
 struct WaveItem {          // 32 lanes of a step's outputs: one warp's work
   uint32_t rec, chunk;     // record (16-byte units), chunk of its lanes
@@ -212,11 +213,9 @@ struct WaveProgram {
 };
 constexpr int kWaveCtaWarps = 16;          // warps per CTA of the level kernel at most
 constexpr int kWaveMaxCtas = 8;            // CTAs of its cluster at most
-constexpr int kWaveCtaWarps32 = 16, kWaveCtaWarps64 = 4;   // warps of work per CTA it aims at
-constexpr int kWavePasses = 2;             // passes over a level at most; wider levels fill the GPU
-// split precision: a row step of GEMM shape with less work than this stays a row step of its
-// level instead of a conversion and a GEMM launch
-constexpr int64_t kWaveTcWork = 1LL << 20;
+constexpr int kWaveCtaWarps32 = 16, kWaveCtaWarps64 = 8;   // warps of work per CTA it aims at
+constexpr int kWavePasses = 1;             // passes over a level at most; wider levels fill the GPU
+constexpr int kWaveK = 5;                  // terms whose operands a lane loads together
 constexpr int64_t kWaveOuts = 1LL << 18;   // outputs of a step inside a level at most
 
 struct TailStep {
@@ -287,13 +286,20 @@ PK_HD inline Tc64Scratch tc64_scratch(long long Bsz, long long M, long long N, l
   x.bytes = x.cc_off + ((x.tiles_n * kTc64Nc * 8 + 255) & ~255LL);
   return x;
 }
-// Whether complex128 runs the step there: GEMM-shaped, and enough work to pay for the
-// conversion and the second launch (about 10 us, in which FP64 does 1.5e6 multiply-adds).
+// Whether complex128 runs the step there: by the cycles it takes (152 multiprocessors).  Tensor
+// cores: two launches, the conversion at about 1500 B per cycle (16 B read, 32 B written per
+// entry), and per wave of tiles 900 cycles a chunk and 2500 for the epilogue; FP64: 76 complex
+// multiply-adds per cycle over the GPU, or half of one per multiprocessor in k_gemm's tiles.
 inline bool tc64_step(const Step& s) {
-  const long long work = s.R * s.K * s.N;
-  return s.b >= 0 && s.kernel != KSPLITK && s.M >= 64 && s.N >= 4 && s.K >= 4 && s.K <= kTc64MaxK &&
-         work >= (s.kernel == KGEMM ? 1LL << 19 : 1LL << 20) &&
-         tc64_scratch(s.Bsz, s.M, s.N, s.K).bytes <= (8LL << 30);
+  if (s.b < 0 || s.kernel == KSPLITK || s.M < 16 || s.N < 4 || s.K < 4 || s.K > kTc64MaxK) return false;
+  const Tc64Scratch x = tc64_scratch(s.Bsz, s.M, s.N, s.K);
+  if (x.bytes > (8LL << 30)) return false;
+  const double waves = (double)((x.tiles_m * x.tiles_n * s.Bsz + 151) / 152);
+  const double tc = 10000 + (double)(s.R * s.K + s.Bsz * s.K * s.N) * 0.032 + waves * (900.0 * (double)x.chunks + 2500);
+  const double fp = s.kernel == KGEMM
+                        ? 8192.0 * (double)s.K * (double)((((s.M + 63) / 64) * ((s.N + 63) / 64) * s.Bsz + 151) / 152)
+                        : (double)s.R * (double)s.K * (double)s.N / 76;
+  return tc < fp;
 }
 
 // Reverse pass: one record per clause tensor (merged edge group) of a gradient plan.
@@ -381,19 +387,24 @@ struct Plan {
   uint64_t off_recipe = 0, off_slots = 0, off_meta = 0, off_result = 0, off_scratch = 0,
            off_counter = 0, off_arena = 0;
   uint64_t ws_bytes(int32_t precision) const;
-  // elements of the arena the workspace holds: the steps' own order (arena_elems) or the
-  // level schedule's, whichever is larger
-  int64_t ws_elems() const { return arena_elems > wave.arena_elems ? arena_elems : wave.arena_elems; }
+  // elements of the arena the workspace holds: the steps' own order (arena_elems) or a level
+  // schedule's, whichever is larger
+  int64_t ws_elems() const {
+    int64_t n = arena_elems;
+    for (const WaveProgram& w : wave) n = n > w.arena_elems ? n : w.arena_elems;
+    return n;
+  }
   // byte offset of the split precision's digit scratch from the arena's start
   uint64_t tc_offset() const { return ((uint64_t)ws_elems() * 16ull + 255) & ~uint64_t(255); }
-  std::vector<uint8_t> program;      // recipe + slots blob copied by pk_upload
+  std::vector<uint8_t> program;      // recipes, slots and widening records, copied by pk_upload
+                                     // with the precision's level records behind them
   // split precision: steps >= tail_first run in complex128 in a separate tail region;
   // bulk tensors they read are up-converted there first
   int32_t tail_first = 0;
   std::vector<ConvRec> conv;
-  WaveProgram wave;                  // level schedule (records in the program at off_wave)
   std::shared_ptr<Plan> compact;     // the same plan on its own order's layout, where only that
                                      // fits pk_eval_noalloc's workspace
+  WaveProgram wave[3];               // level schedules by pk_precision (records at off_wave)
   uint64_t off_wave = 0;
   pk_tuning tuning{};                // launch shapes the plan was made with
   std::vector<TailStep> tail;        // one per step >= tail_first
@@ -453,12 +464,14 @@ bool order_stats(const Knot& k, int32_t q, int32_t order, int32_t restarts, doub
 // pinned tensors kept to the end; returns the arena's elements.  wave_hazards: the pairs that
 // a given layout orders.  wave_stages: the launches and the device records.  wave_check: a
 // replay of the units over the layout.
+enum WaveHeavy : int32_t { kHeavyTc64 = 1, kHeavyTc = 2 };   // launched alone besides: the tensor-core
+                                                             // steps of complex128 / of split
 bool wave_light(const Step& s, const pk_tuning& tune);
 // Arena offsets (multiples of 64 elements) by first fit in decreasing size over the closed
 // lifetimes [born, dies]; returns the arena's elements.
 int64_t first_fit(const std::vector<int64_t>& elems, const std::vector<int32_t>& born,
                   const std::vector<int32_t>& dies, std::vector<int64_t>& off);
-void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuning& tune, bool tc64,
+void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuning& tune, int32_t heavy,
                    bool breadth, const std::vector<std::pair<int32_t, int32_t>>* extra, int32_t first_tail,
                    std::vector<WaveUnit>& units);
 int64_t wave_layout(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
@@ -466,10 +479,13 @@ int64_t wave_layout(const std::vector<Step>& steps, const std::vector<int64_t>& 
                     std::vector<int64_t>& off);
 void wave_hazards(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
                   const std::vector<int64_t>& off, std::vector<std::pair<int32_t, int32_t>>& edges);
-void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, WaveProgram& w);
+void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, int32_t heavy, WaveProgram& w);
+// All units of a plan as levels for one CTA (the batch executor): records | items | level table
+// in `blob`, their places in `range`; returns the number of levels.
+int32_t wave_batch(const Plan& p, std::vector<uint8_t>& blob, WaveRange& range);
 bool wave_check(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
                 const std::vector<char>& pinned, const WaveProgram& w, std::string& err);
-// The plan's level schedule and the workspace layout that holds it; `compact`: on the
+// The plan's level schedules and the workspace layout that holds them; `compact`: on the
 // tensors' offsets of the steps' own order and without the complex128 digit scratch, so that
 // the workspace does not grow.
 void plan_waves(Plan& p, bool compact);

@@ -1715,7 +1715,7 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
   // fixed workspace that its own order fits: such a plan keeps a second schedule for it
   for (int32_t prec : {PK_C128, PK_C64, PK_SPLIT})
     if (!p.compact && p.ws_bytes(prec) > kNoallocBytes) {
-      const uint64_t grown = 16ull * (uint64_t)std::max<int64_t>(0, p.wave.arena_elems - p.arena_elems) + 512 +
+      const uint64_t grown = 16ull * (uint64_t)(p.ws_elems() - p.arena_elems) + 512 +
                              (prec == PK_C128 ? (uint64_t)p.tc64_bytes : 0ull);
       if (p.ws_bytes(prec) <= kNoallocBytes + grown) {
         auto c = std::make_shared<Plan>(p);

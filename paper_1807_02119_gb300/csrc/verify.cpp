@@ -198,9 +198,8 @@ bool check_forward(const Plan& p, int32_t precision, Checker& ck) {
     std::vector<char> pinned(nt, 0);
     for (const TensorInfo& t : p.tensors) elems.push_back(t.elems);
     pinned[p.final_tensor] = 1;
-    if (p.wave.arena_elems > p.ws_elems()) return ck.fail("level schedule", "arena larger than the workspace's");
     std::string e;
-    if (!wave_check(p.steps, elems, pinned, p.wave, e)) return ck.fail("plan", e);
+    if (!wave_check(p.steps, elems, pinned, p.wave[precision], e)) return ck.fail("plan", e);
   }
   // complex128 tail of the complex64 precision
   if (precision == PK_C64 && !p.tail.empty()) {
@@ -227,7 +226,7 @@ bool check_forward(const Plan& p, int32_t precision, Checker& ck) {
   // workspace layout: state records in order, the arena (and the split digit scratch or the
   // tail region) inside the workspace
   if (!(p.off_recipe <= p.off_slots && p.off_slots <= p.off_conv && p.off_conv <= p.off_wave &&
-        p.off_wave + p.wave.blob.size() <= p.off_meta && p.off_meta + 16ull * p.n_meta <= p.off_counter &&
+        p.off_wave + p.wave[precision].blob.size() <= p.off_meta && p.off_meta + 16ull * p.n_meta <= p.off_counter &&
         p.off_counter + 4ull * (uint64_t)ns <= p.off_result &&
         p.off_result + 32ull * (uint64_t)(p.n_slices + 1) <= p.off_scratch &&
         p.off_scratch + 16ull * (uint64_t)p.splitk_partials <= p.off_arena))

@@ -17,13 +17,19 @@ namespace pk {
 // for the cluster barrier, the rest one warp's 200 to 300 dependent instructions (FP64
 // multiply-adds: 63 cycles each).  A level launched alone takes 0.9 us more.
 
+// How a level's operands are read: written by other CTAs of the same launch (past L1), by
+// earlier launches only (read-only path), or by this CTA only (L1).  kWaveAny besides: steps of
+// any size, whose divisions may lack an exact multiplier (mul 0).
+enum WaveMode { kWaveL2 = 0, kWaveRO = 1, kWaveOwn = 2, kWaveAny = 4 };
+
 // Offsets in A and B of index y of a run class (`r` the class's first run, n >= 1 of them);
-// y / size = umulhi(y, ceil(2^32 / size)), exact for the steps the planner lets in.
+// y / size = umulhi(y, ceil(2^32 / size)), exact for the steps the planner gives a multiplier.
+template <int M = kWaveL2>
 __device__ __forceinline__ void wave_offsets(unsigned y, const uint4* r, int n, unsigned& oa, unsigned& ob) {
   uint4 w = *r;   // size, mul, sa, sb
 #pragma unroll 1
   for (; --n > 0; w = *++r) {
-    const unsigned t = __umulhi(y, w.y), d = y - t * w.x;
+    const unsigned t = (M & kWaveAny) && !w.y ? y / w.x : __umulhi(y, w.y), d = y - t * w.x;
     oa += d * w.z;
     ob += d * w.w;
     y = t;
@@ -44,6 +50,11 @@ __device__ __forceinline__ Cx<float> ldl2(const Cx<float>* p) {
 __device__ __forceinline__ Cx<ff> ldl2(const Cx<ff>* p) {
   const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
   return {{v.x, v.y}, {v.z, v.w}};
+}
+
+template <int M, typename R>
+__device__ __forceinline__ Cx<R> wave_ld(const Cx<R>* p) {
+  return M & kWaveOwn ? ldc(p) : M & kWaveRO ? ld(p) : ldl2(p);
 }
 
 // FP64 multiply-adds take 63 cycles each, so the four products of a term go to four sums.
@@ -108,13 +119,24 @@ __device__ __forceinline__ float pow2_of(int n, float) {
   return (unsigned)(n + 126) <= 253u ? __int_as_float((n + 127) << 23) : (float)pow2_slow(n);
 }
 
+// An output's max-abs: FP64 as bits, without FP64 instructions (0 for NaN, as fmax drops it).
+__device__ __forceinline__ unsigned long long mag_key(const Cx<double>& v) {
+  const unsigned long long abs = 0x7fffffffffffffffull, inf = 0x7ff0000000000000ull;
+  unsigned long long a = (unsigned long long)__double_as_longlong(v.re) & abs,
+                     b = (unsigned long long)__double_as_longlong(v.im) & abs;
+  a = a > inf ? 0ull : a;
+  b = b > inf ? 0ull : b;
+  return max(a, b);
+}
+__device__ __forceinline__ float mag_key(const Cx<float>& v) { return mag(v); }
+__device__ __forceinline__ float mag_key(const Cx<ff>& v) { return mag(v); }
+
 // The warp's largest magnitude as bits (integer order = value order; NaN counts as 0, as fmax
 // drops it): one or two warp reductions instead of five shuffle steps.
 __device__ __forceinline__ unsigned long long warp_max_bits(float v) {
   return __reduce_max_sync(0xffffffffu, v == v ? __float_as_uint(v) : 0u);
 }
-__device__ __forceinline__ unsigned long long warp_max_bits(double v) {
-  const unsigned long long b = v == v ? (unsigned long long)__double_as_longlong(v) : 0ull;
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long b) {
   const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32));
   const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32) == hi ? (unsigned)b : 0u);
   return (unsigned long long)hi << 32 | lo;
@@ -122,10 +144,8 @@ __device__ __forceinline__ unsigned long long warp_max_bits(double v) {
 
 // Outputs of lanes [32 chunk, 32 chunk + 32) of the step at `rec`, 2^lanes lanes sharing one
 // output's sum over k; returns the warp's max-abs bits.  Warp-synchronous; every k is added in
-// order within a lane.  The operands of kWaveK terms are loaded together: one round trip.  L1:
-// the operands were written by earlier launches.
-constexpr int kWaveK = 4;
-template <typename R, bool L1>
+// order within a lane.  The operands of kWaveK terms are loaded together: one round trip.
+template <typename R, int M>
 __device__ __forceinline__ unsigned long long wave_outputs(const uint4* rec, unsigned chunk, Cx<R>* arena,
                                                            Meta* meta, int& slot) {
   using S = typename Traits<R>::S;
@@ -139,50 +159,66 @@ __device__ __forceinline__ unsigned long long wave_outputs(const uint4* rec, uns
   const bool hasB = sb >= 0;
   const uint4 *rr = rec + 4, *rk = rr + nrow, *rn = rk + nk;
   const int lane = threadIdx.x & 31;
-  // bookkeeping of the operands (read past L1, as they are)
-  const ulonglong2 ma = __ldcg((const ulonglong2*)(meta + sa));
-  ulonglong2 mb = make_ulonglong2(0, 0);
-  if (hasB) mb = __ldcg((const ulonglong2*)(meta + sb));
-  const unsigned q = chunk * 32 + lane, o = q >> lg, k0 = q & ((1u << lg) - 1);
-  const bool live = o < Rr * N;
+  // bookkeeping of the operands (read past L1, as they are); a launch of its own first works
+  // out its indices, while the launch before it ends
+  ulonglong2 ma, mb = make_ulonglong2(0, 0);
+  auto load_meta = [&] {
+    ma = __ldcg((const ulonglong2*)(meta + sa));
+    if (hasB) mb = __ldcg((const ulonglong2*)(meta + sb));
+  };
+  if (M != kWaveRO) load_meta();
+  const unsigned q = chunk * 32 + lane, o = q >> lg;
+  unsigned k0 = q & ((1u << lg) - 1), kd = 1u << lg;
+  bool live = o < Rr * N;
+  if (std::is_same<R, float>::value && K <= 16) {   // complex64 keeps short sums in order: one lane
+    live = live && k0 == 0;
+    kd = 1;
+  }
   WaveAcc<R> part;
+  unsigned oa = 0, ob = 0;
   if (live) {
-    unsigned r = o, oa = 0, ob = 0, d = 0;
+    unsigned r = o, d = 0;
     if (N > 1) {
-      const unsigned n = Rr == 1 ? o : __umulhi(o, h1.z);
+      const unsigned n = Rr == 1 ? o : (M & kWaveAny) && !h1.z ? o / Rr : __umulhi(o, h1.z);
       r = o - n * Rr;
-      wave_offsets(n, rn, nn, d, ob);
+      wave_offsets<M>(n, rn, nn, d, ob);
     }
-    if (nrow) wave_offsets(r, rr, nrow, oa, ob);
+    if (nrow) wave_offsets<M>(r, rr, nrow, oa, ob);
+  }
+  if (M == kWaveRO) {
+    pdl_wait();
+    load_meta();
+  }
+  if (live) {
     const Cx<R>* A = arena + h2.x + oa;
     const Cx<R>* B = arena + h2.y + ob;
     uint4 w = make_uint4(1, 0, 0, 0);   // one contracted run (or none): constant strides
     if (nk) w = *rk;
 #pragma unroll 1
-    for (unsigned k = k0; k < K; k += kWaveK << lg) {
+    for (unsigned k = k0; k < K; k += kWaveK * kd) {
       unsigned ka[kWaveK], kb[kWaveK];
 #pragma unroll
       for (int u = 0; u < kWaveK; ++u) {
-        ka[u] = (k + ((unsigned)u << lg)) * w.z;
-        kb[u] = (k + ((unsigned)u << lg)) * w.w;
+        ka[u] = (k + (unsigned)u * kd) * w.z;
+        kb[u] = (k + (unsigned)u * kd) * w.w;
       }
       if (nk > 1) {
 #pragma unroll
         for (int u = 0; u < kWaveK; ++u) {
           ka[u] = kb[u] = 0;
-          wave_offsets(min(k + ((unsigned)u << lg), K - 1), rk, nk, ka[u], kb[u]);
+          wave_offsets<M>(min(k + (unsigned)u * kd, K - 1), rk, nk, ka[u], kb[u]);
         }
       }
       Cx<R> a[kWaveK], b[kWaveK];
 #pragma unroll
       for (int u = 0; u < kWaveK; ++u)
-        if (k + ((unsigned)u << lg) < K) {
-          a[u] = L1 ? ld(A + ka[u]) : ldl2(A + ka[u]);
-          if (hasB) b[u] = L1 ? ld(B + kb[u]) : ldl2(B + kb[u]);
+        if (k + (unsigned)u * kd < K) {
+          a[u] = wave_ld<M>(A + ka[u]);
+          if (hasB) b[u] = wave_ld<M>(B + kb[u]);
         }
 #pragma unroll
       for (int u = 0; u < kWaveK; ++u)
-        if (k + ((unsigned)u << lg) < K) {
+        if (k + (unsigned)u * kd < K) {
           if (hasB)
             part.mac(a[u], b[u]);
           else
@@ -191,15 +227,15 @@ __device__ __forceinline__ unsigned long long wave_outputs(const uint4* rec, uns
     }
   }
   Acc<R> acc = part.sum();
-  if (lg) lanes_sum(acc, lg);
+  if (kd > 1) lanes_sum(acc, lg);
   const int ea = exp_of_bits(ma.x, S()), eb = hasB ? exp_of_bits(mb.x, S()) : 0;
   if (chunk == 0 && lane == 0)
     meta[slot].exp = (long long)ma.y + (long long)mb.y + ea + eb;
-  S vmax = 0;
+  decltype(mag_key(Cx<R>())) vmax = 0;
   if (live && k0 == 0) {
     const Cx<R> v = acc.get(pow2_of(-(ea + eb), S()));
     st(arena + off_c + o, v);   // C is [n, r] with r innermost: o = r + n R
-    vmax = mag(v);
+    vmax = mag_key(v);
   }
   return warp_max_bits(vmax);
 }
@@ -210,10 +246,10 @@ __device__ __forceinline__ unsigned long long wave_outputs(const uint4* rec, uns
 // and are read where they are), so that a level's chain of dependent memory reads is one
 // round trip to L2: the operands and their bookkeeping.  Results go to L2 (stores and
 // atomics) and are read from there past L1; the barrier's release and acquire order them.
-template <typename R>
-__global__ void __launch_bounds__(32 * kWaveCtaWarps)
-    k_waves(const unsigned char* __restrict__ blob, WaveRange rg, int n_lev, int smem, Cx<R>* arena, Meta* meta) {
+template <class F>   // F(record, chunk): one item by the calling warp
+__device__ __forceinline__ void wave_walk(const unsigned char* blob, const WaveRange& rg, int n_lev, int smem, F&& item) {
   extern __shared__ __align__(16) unsigned char wsm[];
+  pdl_next();
   const unsigned char *recs = blob, *items = blob + rg.item - rg.item0 * sizeof(WaveItem);
   const unsigned* lev = (const unsigned*)(blob + rg.lev);
   if (smem) {
@@ -229,15 +265,14 @@ __global__ void __launch_bounds__(32 * kWaveCtaWarps)
     lev = (const unsigned*)(wsm + nr + ni);
   }
   lev += rg.lev0;
+  pdl_wait();   // the records are constant: copied while the launch before ends
   const unsigned w0 = blockIdx.x + gridDim.x * (threadIdx.x >> 5);   // consecutive items on different CTAs
   const unsigned nw = gridDim.x * kWaveCtaWarps;
   for (int l = 0; l < n_lev; ++l) {
     const unsigned end = lev[l + 1];
     for (unsigned i = lev[l] + w0; i < end; i += nw) {
       const uint2 it = ((const uint2*)items)[i];
-      int slot;
-      const unsigned long long v = wave_outputs<R, false>((const uint4*)recs + it.x, it.y, arena, meta, slot);
-      if ((threadIdx.x & 31) == 0 && v) atomicMax(&meta[slot].maxbits, v);
+      item((const uint4*)recs + it.x, it.y);
     }
     if (l + 1 == n_lev) break;
     if (gridDim.x == 1)
@@ -245,6 +280,16 @@ __global__ void __launch_bounds__(32 * kWaveCtaWarps)
     else
       asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
+}
+
+template <typename R, int M>   // kWaveOwn: a single CTA
+__global__ void __launch_bounds__(32 * kWaveCtaWarps)
+    k_waves(const unsigned char* __restrict__ blob, WaveRange rg, int n_lev, int smem, Cx<R>* arena, Meta* meta) {
+  wave_walk(blob, rg, n_lev, smem, [&](const uint4* rec, unsigned chunk) {
+    int slot;
+    const unsigned long long v = wave_outputs<R, M>(rec, chunk, arena, meta, slot);
+    if ((threadIdx.x & 31) == 0 && v) atomicMax(&meta[slot].maxbits, v);
+  });
 }
 
 // One level over the whole GPU, a warp per item; one atomic per CTA where its warps work on
@@ -255,12 +300,15 @@ __global__ void __launch_bounds__(256)
                 Cx<R>* arena, Meta* meta) {
   __shared__ unsigned long long red[8];
   __shared__ int slots[8];
+  pdl_next();
   const unsigned w = threadIdx.x >> 5, i = blockIdx.x * (blockDim.x >> 5) + w;
   int slot = -1;
   unsigned long long v = 0;
-  if (i < n_items) {
+  if (i >= n_items) {
+    pdl_wait();
+  } else {
     const uint2 it = __ldg((const uint2*)(blob + rg.item) + first + i);
-    v = wave_outputs<R, true>((const uint4*)blob + it.x, it.y, arena, meta, slot);
+    v = wave_outputs<R, kWaveRO>((const uint4*)blob + it.x, it.y, arena, meta, slot);
   }
   if ((threadIdx.x & 31) == 0) {
     red[w] = v;
@@ -278,6 +326,41 @@ __global__ void __launch_bounds__(256)
       if (j < blockDim.x >> 5) m = red[j];
     }
   }
+}
+
+// Launches `fn` on `stream`; pdl: it may start while the launch before it still runs (every
+// kernel calls pdl_wait); cluster > 1: CTAs per cluster.
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*fn)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, bool pdl,
+                          unsigned cluster, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[2];
+  if (pdl) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    at[cfg.numAttrs].val.clusterDim.x = cluster;
+    at[cfg.numAttrs].val.clusterDim.y = 1;
+    at[cfg.numAttrs++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = at;
+  return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+
+// Launches a FUSED stage as one cluster; fn: a level kernel (blob, range, levels, smem, args).
+constexpr uint32_t kWaveSmem = 100 * 1024;   // its records in shared memory: two CTAs per SM
+template <typename F, typename... A>
+cudaError_t launch_cluster(const WaveStage& g, const unsigned char* blob, cudaStream_t stream, bool pdl, F fn, A... args) {
+  const uint32_t prog = g.range.rec_bytes + g.range.item_bytes + g.range.lev_bytes;
+  const int smem = prog <= kWaveSmem ? (int)prog : 0;
+  return launch_kernel(fn, dim3((unsigned)g.ctas), 32 * kWaveCtaWarps, (size_t)smem, stream, pdl, (unsigned)g.ctas, blob,
+                       g.range, (int)g.units, smem, args...);
 }
 
 }  // namespace pk

@@ -29,18 +29,24 @@ bool overlap(const Interval& x, const Interval& y) {
   return x.off < y.off + y.len && y.off < x.off + x.len;
 }
 
-// Multiplier of the division by d >= 2: y / d = (y * mul) >> 32, exact while y d < 2^32.
-uint32_t div_mul(int64_t d) { return d < 2 ? 0 : (uint32_t)(((1ull << 32) + (uint64_t)d - 1) / (uint64_t)d); }
+// Multiplier of the division of y < top by d >= 2: y / d = (y * mul) >> 32, exact while
+// y d < 2^32; 0 (the kernel divides) otherwise.
+uint32_t div_mul(int64_t d, int64_t top) {
+  return d < 2 || top * d >= ((int64_t)1 << 32) ? 0 : (uint32_t)(((1ull << 32) + (uint64_t)d - 1) / (uint64_t)d);
+}
 
-// log2 of the lanes that share one output's sum over k: about 16 terms each, while the
-// step's lanes stay within what the GPU holds at once.
+// log2 of the lanes that share one output's sum over k: at most kWaveK terms per lane (one
+// round trip for their operands) while the step has few lanes, 16 (8 of a longer sum) while
+// they stay within what the GPU holds at once.
 int lanes_log2(int64_t outs, int64_t K) {
   int l = 0;
-  while (l < 5 && (K >> l) > 16 && (outs << (l + 1)) <= (1 << 18)) ++l;
+  while (l < 5 && (((K >> l) > kWaveK && (outs << (l + 1)) <= (1 << 13)) ||
+                   ((K >> l) > (K > 16 ? 8 : 16) && (outs << (l + 1)) <= (1 << 18))))
+    ++l;
   return l;
 }
 
-uint32_t push_record(const Step& s, const std::vector<int64_t>& off, std::vector<uint8_t>& blob) {
+uint32_t push_record(const Step& s, const std::vector<int64_t>& off, std::vector<uint8_t>& blob, uint32_t per = 1) {
   WaveRec r;
   std::memset(&r, 0, sizeof(r));
   r.a = s.a;
@@ -49,7 +55,7 @@ uint32_t push_record(const Step& s, const std::vector<int64_t>& off, std::vector
   r.R = (uint32_t)s.R;
   r.N = (uint32_t)s.N;
   r.K = (uint32_t)s.K;
-  r.mul_r = div_mul(s.R);
+  r.mul_r = div_mul(s.R, s.R * s.N);
   r.nrow = (uint8_t)s.nrow;
   r.nk = (uint8_t)s.nk;
   r.nn = (uint8_t)s.nn;
@@ -57,17 +63,18 @@ uint32_t push_record(const Step& s, const std::vector<int64_t>& off, std::vector
   r.off_a = off[s.a];
   r.off_b = s.b >= 0 ? off[s.b] : 0;
   r.off_c = off[s.c];
+  r.per = per;
   const size_t at = blob.size();
   blob.resize(at + sizeof(WaveRec) + sizeof(WaveRun) * (size_t)(s.nrow + s.nk + s.nn));
   std::memcpy(blob.data() + at, &r, sizeof(r));
   WaveRun* w = (WaveRun*)(blob.data() + at + sizeof(WaveRec));
-  auto put = [&](const Run* v, int n) {
+  auto put = [&](const Run* v, int n, int64_t top) {
     for (int i = 0; i < n; ++i, ++w)
-      *w = {(uint32_t)v[i].size, div_mul(v[i].size), (uint32_t)v[i].sa, (uint32_t)v[i].sb};
+      *w = {(uint32_t)v[i].size, div_mul(v[i].size, top), (uint32_t)v[i].sa, (uint32_t)v[i].sb};
   };
-  put(s.row, s.nrow);
-  put(s.kr, s.nk);
-  put(s.nr, s.nn);
+  put(s.row, s.nrow, s.R);
+  put(s.kr, s.nk, s.K);
+  put(s.nr, s.nn, s.N);
   return (uint32_t)(at / 16);
 }
 
@@ -107,14 +114,13 @@ int64_t first_fit(const std::vector<int64_t>& elems, const std::vector<int32_t>&
 }
 
 bool wave_light(const Step& s, const pk_tuning& tune) {
-  if (s.kernel != KROWS || s.K > tune.seq_k) return false;
+  // the top of pk_tuning's ranges leaves K and the outputs to the level kernels' own limits
+  if (s.kernel != KROWS || s.K > (tune.seq_k == 2048 ? kWaveOuts : tune.seq_k)) return false;
   const int64_t outs = s.R * s.N, work = outs * s.K;
-  // the top of pk_tuning's range leaves the outputs to the level kernels' own limit
   if (outs > (tune.seq_outs == 65536 ? kWaveOuts : tune.seq_outs)) return false;
   // K > 32: more work than that still runs better here, where lanes share a sum, than on the
   // thread-per-output kernel (the row kernel's registers hold 32 terms)
   if (work > (s.K > 32 ? 16 * tune.seq_work : tune.seq_work)) return false;
-  if (s.tc && work >= kWaveTcWork) return false;
   // the kernels' divisions y / d as umulhi(y, ceil(2^32 / d)) are exact while y d < 2^32
   if (s.N > 1 && outs * s.R >= ((int64_t)1 << 32)) return false;
   auto exact = [](const Run* r, int n) {
@@ -128,7 +134,7 @@ bool wave_light(const Step& s, const pk_tuning& tune) {
   return exact(s.row, s.nrow) && exact(s.kr, s.nk) && exact(s.nr, s.nn);
 }
 
-void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuning& tune, bool tc64,
+void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuning& tune, int32_t heavy,
                    bool breadth, const std::vector<std::pair<int32_t, int32_t>>* extra, int32_t first_tail,
                    std::vector<WaveUnit>& units) {
   const int32_t n = (int32_t)steps.size();
@@ -152,7 +158,8 @@ void wave_schedule(const std::vector<Step>& steps, int32_t n_tens, const pk_tuni
   std::vector<char> light(n);
   std::vector<int32_t> ready_l, ready_h;
   auto add = [&](int32_t i) { (light[i] ? ready_l : ready_h).push_back(i); };
-  for (int32_t i = 0; i < n; ++i) light[i] = i < first_tail && wave_light(steps[i], tune) && !(tc64 && tc64_step(steps[i]));
+  for (int32_t i = 0; i < n; ++i) light[i] = i < first_tail && wave_light(steps[i], tune) && !((heavy & kHeavyTc64) && tc64_step(steps[i])) &&
+               !((heavy & kHeavyTc) && steps[i].tc);
   for (int32_t i = 0; i < n; ++i)
     if (need[i] == 0) add(i);
   auto finish = [&](int32_t i) {
@@ -298,20 +305,23 @@ bool wave_check(const std::vector<Step>& steps, const std::vector<int64_t>& elem
   return true;
 }
 
-void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, WaveProgram& w) {
+void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, int32_t heavy, WaveProgram& w) {
   // records, items and level table of all levels in order
   std::vector<uint8_t> recs;
   std::vector<WaveItem> items;
   const size_t nu = w.units.size();
   std::vector<uint32_t> lev(nu + 1, 0), rec_at(nu + 1, 0);   // first item / record byte of a unit
+  std::vector<int64_t> weight(nu, 0);   // a unit's items, weighed by their terms per lane
   for (size_t u = 0; u < nu; ++u) {
     lev[u] = (uint32_t)items.size();
     rec_at[u] = (uint32_t)recs.size();
-    if (w.units[u].heavy && !wave_light(steps[w.units[u].steps[0]], tune)) continue;
+    const Step& s0 = steps[w.units[u].steps[0]];
+    if (w.units[u].heavy && (!wave_light(s0, tune) || ((heavy & kHeavyTc) && s0.tc))) continue;
     for (int32_t i : w.units[u].steps) {
       const uint32_t at = push_record(steps[i], w.off, recs);
       const int64_t outs = steps[i].R * steps[i].N, lanes = outs << lanes_log2(outs, steps[i].K);
       for (int64_t c = 0; c * 32 < lanes; ++c) items.push_back({at, (uint32_t)c});
+      weight[u] += (lanes + 31) / 32 * std::max<int64_t>(4, steps[i].K / (lanes / outs));
     }
   }
   lev[nu] = (uint32_t)items.size();
@@ -348,12 +358,12 @@ void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, WaveProg
         ++u;
         continue;
       }
-      int64_t most = lev[u + 1] - lev[u];
+      auto load = [&](size_t x) { return (weight[x] + 3) / 4; };   // in items of four terms
+      int64_t most = load(u);
       size_t v = u + 1;
       st.kind = most > fused_max || w.units[u].heavy ? WaveStage::WIDE : WaveStage::FUSED;
       if (st.kind == WaveStage::FUSED)
-        for (; v < nu && !w.units[v].heavy && lev[v + 1] - lev[v] <= fused_max; ++v)
-          most = std::max<int64_t>(most, lev[v + 1] - lev[v]);
+        for (; v < nu && !w.units[v].heavy && load(v) <= fused_max; ++v) most = std::max<int64_t>(most, load(v));
       st.units = (int32_t)(v - u);
       st.items = (int32_t)(lev[v] - lev[u]);
       while (st.ctas < kWaveMaxCtas && most > st.ctas * per_cta) st.ctas *= 2;
@@ -379,46 +389,80 @@ void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, WaveProg
   }
 }
 
+int32_t wave_batch(const Plan& p, std::vector<uint8_t>& blob, WaveRange& range) {
+  std::vector<WaveItem> items;
+  std::vector<uint32_t> lev;
+  blob.clear();
+  range = WaveRange{};
+  const WaveProgram& w = p.wave[PK_C64];   // no step of it is kept apart for the tensor cores
+  for (const WaveUnit& u : w.units) {
+    lev.push_back((uint32_t)items.size());
+    for (int32_t i : u.steps) {
+      const Step& s = p.steps[i];
+      const int64_t outs = s.R * s.N, lanes = outs << lanes_log2(outs, s.K);
+      const int64_t per = std::max<int64_t>(1, (lanes + 65535) / 65536);   // at most 2048 items a step
+      const uint32_t at = push_record(s, w.off, blob, (uint32_t)per);
+      for (int64_t c = 0; c * 32 * per < lanes; ++c) items.push_back({at, (uint32_t)c});
+    }
+  }
+  lev.push_back((uint32_t)items.size());
+  auto put = [&](const void* src, size_t n, uint32_t& at, uint32_t& len) {
+    at = (uint32_t)blob.size();
+    len = (uint32_t)((n + 15) / 16 * 16);
+    blob.resize(at + len, 0);
+    if (n) std::memcpy(blob.data() + at, src, n);
+  };
+  range.rec_bytes = (uint32_t)blob.size();
+  put(items.data(), sizeof(WaveItem) * items.size(), range.item, range.item_bytes);
+  put(lev.data(), 4 * lev.size(), range.lev, range.lev_bytes);
+  return (int32_t)w.units.size();
+}
+
 void plan_waves(Plan& p, bool compact) {
   const int32_t n = (int32_t)p.tensors.size(), ns = (int32_t)p.steps.size();
-  WaveProgram& w = p.wave;
-  w = WaveProgram();
-  w.n_init = p.n_init;
   std::vector<int64_t> elems(n);
   std::vector<char> pinned(n, 0);
   for (int32_t t = 0; t < n; ++t) elems[t] = p.tensors[t].elems;
   pinned[p.final_tensor] = 1;
-  const bool tc64 = p.use_tc && !compact;
   p.tc64_bytes = 0;
   for (const Step& s : p.steps)
-    if (tc64 && tc64_step(s)) p.tc64_bytes = std::max<int64_t>(p.tc64_bytes, tc64_scratch(s.Bsz, s.M, s.N, s.K).bytes);
+    if (p.use_tc && !compact && tc64_step(s))
+      p.tc64_bytes = std::max<int64_t>(p.tc64_bytes, tc64_scratch(s.Bsz, s.M, s.N, s.K).bytes);
   const int32_t tail = p.conv.empty() && p.tail.empty() ? ns : p.tail_first;
-  // breadth first over the heavy steps has the fewest rounds; one heavy step at a time needs
-  // about the memory of the steps' own order.  The widening records of a complex128 tail
-  // address the steps' own offsets, so such plans keep them, and so do plans that must stay
-  // within a memory limit: their schedule follows the offsets' reuse.
   int64_t limit = p.arena_elems;   // twice that up to 1 GiB, a quarter more up to 16 GiB
   if (limit <= (1 << 25))
     limit = 2 * limit + (1 << 12);
   else if (limit <= (1 << 30) / 5 * 4)
     limit += limit / 4;
-  for (int breadth = 1; breadth >= 0 && !compact && tail == ns; --breadth) {
-    wave_schedule(p.steps, n, p.tuning, tc64, breadth != 0, nullptr, ns, w.units);
-    w.arena_elems = wave_layout(p.steps, elems, pinned, w.units, w.off);
-    if (w.arena_elems <= limit) break;
-    w.off.clear();
+  uint64_t blob = 0;
+  for (int32_t prec : {PK_C128, PK_C64, PK_SPLIT}) {
+    WaveProgram& w = p.wave[prec];
+    w = WaveProgram();
+    w.n_init = p.n_init;
+    const int32_t heavy = prec == PK_SPLIT ? kHeavyTc : prec == PK_C128 && p.tc64_bytes > 0 ? kHeavyTc64 : 0;
+    // breadth first over the heavy steps has the fewest rounds; one heavy step at a time needs
+    // about the memory of the steps' own order.  The widening records of a complex128 tail
+    // address the steps' own offsets, so such plans keep them, and so do plans that must stay
+    // within a memory limit: their schedule follows the offsets' reuse.
+    for (int breadth = 1; breadth >= 0 && !compact && tail == ns; --breadth) {
+      wave_schedule(p.steps, n, p.tuning, heavy, breadth != 0, nullptr, ns, w.units);
+      w.arena_elems = wave_layout(p.steps, elems, pinned, w.units, w.off);
+      if (w.arena_elems <= limit) break;
+      w.off.clear();
+    }
+    if (w.off.empty()) {
+      for (int32_t t = 0; t < n; ++t) w.off.push_back(p.tensors[t].offset);
+      w.arena_elems = p.arena_elems;
+      std::vector<std::pair<int32_t, int32_t>> edges;
+      wave_hazards(p.steps, elems, w.off, edges);
+      wave_schedule(p.steps, n, p.tuning, heavy, false, &edges, tail, w.units);
+    }
+    wave_stages(p.steps, p.tuning, heavy, w);
+    blob = std::max<uint64_t>(blob, w.blob.size());
   }
-  if (w.off.empty()) {
-    for (int32_t t = 0; t < n; ++t) w.off.push_back(p.tensors[t].offset);
-    w.arena_elems = p.arena_elems;
-    std::vector<std::pair<int32_t, int32_t>> edges;
-    wave_hazards(p.steps, elems, w.off, edges);
-    wave_schedule(p.steps, n, p.tuning, tc64, false, &edges, tail, w.units);
-  }
-  wave_stages(p.steps, p.tuning, w);
-  // workspace: [recipes | slots | conv | level records] uploaded, then the device's own state
-  uint64_t off = p.off_wave;
-  off = align256(off + w.blob.size());
+  // workspace: [recipes | slots | conv | the precision's level records] uploaded, then the
+  // device's own state
+  uint64_t off = align256(p.off_wave + blob);
   p.off_meta = off;
   off = align256(off + 16ull * p.n_meta);
   p.off_counter = off;
@@ -429,9 +473,6 @@ void plan_waves(Plan& p, bool compact) {
   off = align256(off + 16ull * (uint64_t)std::max<int64_t>(1, p.splitk_partials));
   p.off_arena = off;
   p.off_tail = align256(p.off_arena + 8ull * (uint64_t)p.ws_elems());
-  p.program.resize(p.off_wave);
-  p.program.resize(p.off_meta, 0);
-  if (!w.blob.empty()) std::memcpy(p.program.data() + p.off_wave, w.blob.data(), w.blob.size());
 }
 
 }  // namespace pk
