@@ -159,13 +159,15 @@ typedef struct {
  * the defaults; pk_ctx_set_tuning changes them for plans and batches created afterwards. */
 typedef struct {
   int32_t batch_threads;     /* threads per CTA of the batch executor: 128, 256 or 512       */
-  int32_t batch_ktab;        /* batch executor: contracted-index offsets of a step kept in
-                                shared memory (steps with longer K recompute them): 256..2048 */
+  int32_t batch_ktab;        /* batch executor: shared memory for a knot's level records, in
+                                units of 32 bytes (larger knots' are read where they are):
+                                256..2048                                                     */
   int64_t seq_outs;          /* small steps, run together level by level: outputs per step at
                                 most (1..65536; 65536: as many as the level kernels take)     */
   int64_t seq_work;          /* ... complex multiply-adds per step at most (1..2^24; 16 times
                                 as many for a contracted extent above 32)                     */
-  int64_t seq_k;             /* ... contracted extent per step at most (1..2048)              */
+  int64_t seq_k;             /* ... contracted extent per step at most (1..2048; 2048: no limit
+                                of its own)                                                   */
   int64_t tc_min_k;          /* PK_SPLIT: row steps of GEMM shape (M >= 64, N >= tc_min_n)
                                 with this contracted extent or more run on the tensor cores
                                 too (4..16; 16: only steps with K >= 16)                      */

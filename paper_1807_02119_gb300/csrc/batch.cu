@@ -1,11 +1,15 @@
 // Batched evaluation: many knots (each with its own plan) in one persistent launch.
 //
-// Every CTA repeatedly takes the next knot from an atomic work counter and performs
-// that knot's whole contraction itself -- initial tensors (one warp per tensor), then
-// every pairwise step with the CTA's threads spread over the outputs and a block
-// barrier between steps, then the slice scalar -- so knots of very different sizes
-// balance across the SMs and no CTA ever waits for another one.  The launch (preceded
-// by a reset of the counter) is recorded once into a CUDA graph and replayed.
+// Every CTA repeatedly takes the next knot from an atomic work counter (the most work first)
+// and performs that knot's whole contraction itself: initial tensors (a part of a warp per
+// tensor), then the plan's levels with the CTA's warps spread over a level's outputs and a
+// block barrier between levels (records and code as in wave.cuh), then the slice scalar.  No
+// CTA ever waits for another one.  The launch (preceded by a reset of the counter) is recorded
+// once into a CUDA graph and replayed.  What bounds it is the chain of levels of the largest
+// knots: 10 to 25 levels of about 1.5 us, where one step after another took 120 times 10 us.
+// Measured on GB300, per launch: 1024 knots of 20 to 120 crossings at q = 3 in split 1.80 ->
+// 0.54 ms, 192 of 20 to 60 at q = 5 in complex128 1.20 -> 0.40 ms (one CTA per knot for all of
+// them: 0.71 and 1.40 ms; everything above half a CTA's share in clusters: 0.67 and 0.57 ms).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -18,6 +22,8 @@
 
 #include "handles.h"
 #include "kernels.cuh"
+#include "gemm_tc.cuh"
+#include "wave.cuh"
 
 namespace pk {
 
@@ -25,129 +31,66 @@ namespace pk {
 struct BatchKnot {
   int64_t recipe0, n_recipe;   // recipes of the knot
   int64_t slot_base;           // added to Recipe::slot0
-  int64_t step0, n_steps;      // steps of the knot
+  int64_t blob;                // the knot's level records in the record array (bytes)
   int64_t arena_off;           // first arena element of the knot
   int64_t meta_off;            // first bookkeeping slot of the knot
   int64_t n_slices;
   int64_t final_offset;        // final tensor (arena elements, relative)
-  int32_t n_sliced, q, final_tensor, pad;
-};
-
-// A step of the batch image: the contraction's extents and operand offsets, with its
-// stride runs packed into the batch's run array (rows, then contracted, then columns)
-// instead of the fixed-size run tables of a Step, so the image is about ten times smaller.
-struct BatchStep {
-  int32_t a, b, c;           // bookkeeping slots relative to the knot (b = -1: constant 1)
-  int16_t nrow, nk, nn, pad;
-  int64_t off_a, off_b, off_c;
-  int64_t R, K, N;
-  int64_t run0;              // first run of this step in the run array
+  int32_t n_sliced, q, final_tensor, n_meta;
+  int32_t n_lev, blob_bytes, item, lev;   // levels; bytes of the records; items and level table in them
 };
 
 namespace {
 
-
-template <typename S>
-__device__ __forceinline__ S block_max(S v, S* red) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  v = lane < (int)(blockDim.x >> 5) ? red[lane] : S(0);
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;  // every thread holds the block maximum
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
 }
 
-// One pairwise step of one knot by the whole CTA (outputs spread over the threads); the
-// step's runs are staged in shared memory first.
-template <typename R>
-__device__ void cta_step(const BatchStep& s, const Run* __restrict__ runs, Run* srun,
-                         Cx<R>* arena, Meta* meta, long long* tbl, int ktab,
-                         typename Traits<R>::S* red) {
+// The knots order[first .. last), most work first.  CL = 1: each by one CTA (T threads), taken
+// from the work counter.  CL > 1: each by a cluster of CL CTAs, for the knots that would keep
+// one CTA busy long after the others are done; cluster c takes every (number of clusters)-th.
+// A knot's records are copied to shared memory when they fit `smem` bytes.
+template <typename R, int T, int CL>
+__global__ void __launch_bounds__(T) k_batch(const BatchKnot* __restrict__ knots, const int* __restrict__ order,
+                                             int first, int last, const Recipe* recs, const Slot* slots,
+                                             const unsigned char* blobs, Cx<R>* arena,
+                                             Meta* meta_all, SliceResult* out, unsigned* next, int smem) {
   using S = typename Traits<R>::S;
-  const int nruns = s.nrow + s.nk + s.nn;
-  for (int i = threadIdx.x; i < nruns; i += blockDim.x) srun[i] = runs[s.run0 + i];
-  __syncthreads();
-  const Run* row = srun;
-  const Run* kr = srun + s.nrow;
-  const Run* nr = srun + s.nrow + s.nk;
-  const int ea = bin_exp(bits_to_val<S>(meta[s.a].maxbits));
-  int eb = 0;
-  long long xb = 0;
-  const bool hasB = s.b >= 0;
-  if (hasB) {
-    eb = bin_exp(bits_to_val<S>(meta[s.b].maxbits));
-    xb = meta[s.b].exp;
-  }
-  const long long exp_c = meta[s.a].exp + xb + ea + eb;
-  const S scale = (S)ldexp(1.0, -(ea + eb));
-  const bool tab = s.K <= ktab;
-  if (tab)
-    for (long long k = threadIdx.x; k < s.K; k += blockDim.x)
-      split_runs((unsigned long long)k, kr, s.nk, tbl[k], tbl[ktab + k]);
-  __syncthreads();
-  const Cx<R>* A = arena + s.off_a;
-  const Cx<R>* B = arena + s.off_b;
-  Cx<R>* C = arena + s.off_c;
-  const long long outs = s.R * s.N;
-  S vmax = 0;
-  for (long long o = threadIdx.x; o < outs; o += blockDim.x) {
-    const long long r = o % s.R, n = o / s.R;
-    long long oa, ob, d, nb = 0;
-    split_runs((unsigned long long)r, row, s.nrow, oa, ob);
-    if (hasB) split_runs((unsigned long long)n, nr, s.nn, d, nb);
-    Acc<R> acc;
-    for (long long k = 0; k < s.K; ++k) {
-      long long ka, kb;
-      if (tab) {
-        ka = tbl[k];
-        kb = tbl[ktab + k];
-      } else {
-        split_runs((unsigned long long)k, kr, s.nk, ka, kb);
-      }
-      const Cx<R> av = ldc(A + oa + ka);
-      if (hasB)
-        acc.mac(av, ldc(B + ob + nb + kb));
-      else
-        acc.add(av);
-    }
-    const Cx<R> v = acc.get(scale);
-    st(C + o, v);  // C is [n, r] with r innermost: entry o = r + n R
-    vmax = fmax(vmax, mag(v));
-  }
-  vmax = block_max(vmax, red);
-  if (threadIdx.x == 0) {
-    meta[s.c].maxbits = max_bits(vmax);
-    meta[s.c].exp = exp_c;
-  }
-  __syncthreads();
-}
-
-// T threads per CTA; ktab offsets of the contracted index per step in shared memory.
-template <typename R, int T>
-__global__ void __launch_bounds__(T) k_batch(const BatchKnot* __restrict__ knots, int n_knots,
-                                             const Recipe* recs, const Slot* slots,
-                                             const BatchStep* steps, const Run* runs, Cx<R>* arena,
-                                             Meta* meta_all, SliceResult* out, unsigned* next,
-                                             int ktab) {
-  using S = typename Traits<R>::S;
-  extern __shared__ long long tbl[];
-  __shared__ S red[32];
-  __shared__ Run srun[3 * kMaxRuns];
+  constexpr int kMode = (CL == 1 ? kWaveOwn : kWaveL2) | kWaveAny;
+  extern __shared__ __align__(16) unsigned char bsm[];
   __shared__ int kn_s;
-  for (;;) {
+  const int rank = CL == 1 ? 0 : (int)cluster_rank();
+  const int lane = threadIdx.x & 31, tid = rank * T + threadIdx.x, threads = CL * T;
+  // consecutive items of a level on different CTAs
+  const int warp = rank + CL * (threadIdx.x >> 5), nwarps = threads / 32;
+  auto sync = [] {
+    if (CL == 1)
+      __syncthreads();
+    else
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  };
+  for (int turn = first + (int)(blockIdx.x / CL);; turn += (int)(gridDim.x / CL)) {
     __syncthreads();
-    if (threadIdx.x == 0) kn_s = (int)atomicAdd(next, 1u);
-    __syncthreads();
-    const int kn = kn_s;
-    if (kn >= n_knots) return;
+    if (CL == 1) {
+      if (threadIdx.x == 0) kn_s = first + (int)atomicAdd(next, 1u);
+      __syncthreads();
+      turn = kn_s;
+    }
+    if (turn >= last) return;
+    const int kn = order[turn];
     const BatchKnot K = knots[kn];
+    const unsigned char* blob = blobs + K.blob;
+    if (K.blob_bytes <= smem) {
+      for (int i = threadIdx.x * 16; i < K.blob_bytes; i += T * 16) tc::cp_async16(tc::smem_u32(bsm + i), blob + i);
+      tc::cp_async_wait();   // read after the barrier below
+      blob = bsm;
+    }
     Cx<R>* A0 = arena + K.arena_off;
     Meta* meta = meta_all + K.meta_off;
     double tre = 0, tim = 0;
     long long texp = LLONG_MIN;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     for (long long sl = 0; sl < K.n_slices; ++sl) {
       int sdig[64];
       {
@@ -157,30 +100,50 @@ __global__ void __launch_bounds__(T) k_batch(const BatchKnot* __restrict__ knots
           t /= K.q;
         }
       }
-      // initial tensors: one warp per tensor
-      for (long long j = warp; j < K.n_recipe; j += nwarps) {
-        const Recipe r = recs[K.recipe0 + j];
+      for (int i = (int)K.n_recipe + tid; i < K.n_meta; i += threads) meta[i].maxbits = 0;
+      // initial tensors: `part` lanes (a power of two up to a warp) per tensor
+      int part = 1;
+      while (part < 32 && part < K.q * K.q) part *= 2;
+      for (long long j0 = (long long)warp * (32 / part); j0 < K.n_recipe; j0 += (long long)nwarps * (32 / part)) {
+        const long long j = j0 + lane / part;
         S vmax = 0;
-        for (long long e = lane; e < r.elems; e += 32) {
-          double re, im;
-          recipe_value(r, slots + K.slot_base, e, K.q, sdig, re, im);
-          const Cx<R> v{from_double<R>(re), from_double<R>(im)};
-          st(A0 + r.offset + e, v);
-          vmax = fmax(vmax, mag(v));
+        Recipe r;
+        if (j < K.n_recipe) {
+          r = recs[K.recipe0 + j];
+          for (long long e = lane & (part - 1); e < r.elems; e += part) {
+            double re, im;
+            recipe_value(r, slots + K.slot_base, e, K.q, sdig, re, im);
+            const Cx<R> v{from_double<R>(re), from_double<R>(im)};
+            st(A0 + r.offset + e, v);
+            vmax = fmax(vmax, mag(v));
+          }
         }
-        for (int o = 16; o > 0; o >>= 1) vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-        if (lane == 0) {
+        for (int o = part >> 1; o > 0; o >>= 1) vmax = fmax(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
+        if (j < K.n_recipe && (lane & (part - 1)) == 0) {
           meta[r.meta].maxbits = max_bits(vmax);
           meta[r.meta].exp = r.exp2;
         }
       }
-      __syncthreads();
-      for (long long i = 0; i < K.n_steps; ++i)
-        cta_step<R>(steps[K.step0 + i], runs, srun, A0, meta, tbl, ktab, red);
-      if (threadIdx.x == 0) {  // add this slice's scalar at a common exponent
-        const Cx<R> v = ldc(A0 + K.final_offset);
+      sync();
+      const unsigned* lev = (const unsigned*)(blob + K.lev);
+      for (int l = 0; l < K.n_lev; ++l) {
+        const unsigned end = lev[l + 1];
+        for (unsigned i = lev[l] + warp; i < end; i += nwarps) {
+          const uint2 it = ((const uint2*)(blob + K.item))[i];
+          const uint4* rec = (const uint4*)blob + it.x;
+          const unsigned per = rec[3].z;   // WaveRec::per
+          unsigned long long m = 0;
+          int slot = 0;
+          for (unsigned c = 0; c < per; ++c)
+            m = max(m, wave_outputs<R, kMode>(rec, it.y * per + c, A0, meta, slot));
+          if (lane == 0 && m) atomicMax(&meta[slot].maxbits, m);
+        }
+        sync();
+      }
+      if (tid == 0) {  // add this slice's scalar at a common exponent
+        const Cx<R> v = ldl2(A0 + K.final_offset);
         double vr = to_double(v.re), vi = to_double(v.im);
-        long long ve = meta[K.final_tensor].exp;
+        long long ve = __ldcg(&meta[K.final_tensor].exp);
         double m = fmax(fabs(vr), fabs(vi));
         if (m > 0) {
           int k;
@@ -201,15 +164,17 @@ __global__ void __launch_bounds__(T) k_batch(const BatchKnot* __restrict__ knots
           }
         }
       }
-      __syncthreads();
+      sync();
     }
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       out[kn].re = tre;
       out[kn].im = tim;
       out[kn].exp = texp == LLONG_MIN ? 0 : texp;
     }
   }
 }
+
+constexpr int kCl = 8, kClThreads = 512;   // CTAs of a cluster, threads of each
 
 uint64_t a256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
 
@@ -222,12 +187,12 @@ struct pk_batch {
   std::vector<pk::BatchKnot> knots;
   std::vector<pk::Recipe> recipes;
   std::vector<pk::Slot> slots;
-  std::vector<pk::BatchStep> steps;
-  std::vector<pk::Run> runs;
+  std::vector<uint8_t> blobs;          // every knot's level records
+  std::vector<int32_t> order;          // knots by decreasing work
   std::vector<pk::Knot> kinfo;
-  std::vector<pk::Scaled> factor;
+  std::vector<pk::Scaled> factor, prefactor;   // of Z (folded loops), and A(q)
   std::vector<int32_t> qs;
-  uint64_t off_knots = 0, off_recipes = 0, off_slots = 0, off_steps = 0, off_runs = 0, off_meta = 0,
+  uint64_t off_knots = 0, off_recipes = 0, off_slots = 0, off_order = 0, off_blobs = 0, off_meta = 0,
            off_results = 0, off_counter = 0, off_arena = 0, total = 0, image_bytes = 0;
   std::vector<uint8_t> image;
   uint8_t* pinned = nullptr;
@@ -236,7 +201,8 @@ struct pk_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   int32_t device = -1;
-  int32_t threads = 256, ktab = 2048;   // launch shape (the context's tuning at creation)
+  int32_t n_big = 0;                   // knots run by clusters (the first of `order`)
+  int32_t threads = 256, smem = 0;      // launch shape (the context's tuning at creation)
 };
 
 namespace {
@@ -247,10 +213,16 @@ pk_status bfail(pk_ctx* c, pk_status s, const std::string& m) {
 }
 
 template <typename R>
-void* batch_kernel(int threads) {
-  if (threads == 128) return (void*)pk::k_batch<R, 128>;
-  if (threads == 512) return (void*)pk::k_batch<R, 512>;
-  return (void*)pk::k_batch<R, 256>;
+void* batch_kernel(int threads, bool cluster) {
+  if (cluster) return (void*)pk::k_batch<R, pk::kClThreads, pk::kCl>;
+  if (threads == 128) return (void*)pk::k_batch<R, 128, 1>;
+  if (threads == 512) return (void*)pk::k_batch<R, 512, 1>;
+  return (void*)pk::k_batch<R, 256, 1>;
+}
+void* batch_kernel(int32_t precision, int threads, bool cluster) {
+  return precision == PK_C128 ? batch_kernel<double>(threads, cluster)
+         : precision == PK_C64 ? batch_kernel<float>(threads, cluster)
+                               : batch_kernel<pk::ff>(threads, cluster);
 }
 
 cudaError_t build_graph(pk_batch* b, void* ws, cudaStream_t stream) {
@@ -274,46 +246,52 @@ cudaError_t build_graph(pk_batch* b, void* ws, cudaStream_t stream) {
   mp.elementSize = 4;
   mp.width = 1;
   mp.height = 1;
-  cudaGraphNode_t memset_node, kernel_node;
+  cudaGraphNode_t memset_node;
   e = cudaGraphAddMemsetNode(&memset_node, b->graph, nullptr, 0, &mp);
   if (e != cudaSuccess) return e;
-  void* func;
-  if (b->precision == PK_C128)
-    func = batch_kernel<double>(b->threads);
-  else if (b->precision == PK_C64)
-    func = batch_kernel<float>(b->threads);
-  else
-    func = batch_kernel<pk::ff>(b->threads);
-  const size_t smem = sizeof(long long) * 2 * (size_t)b->ktab;
-  e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   const pk::BatchKnot* knots = (const pk::BatchKnot*)(base + b->off_knots);
-  int n = b->n;
   const pk::Recipe* recs = (const pk::Recipe*)(base + b->off_recipes);
   const pk::Slot* slots = (const pk::Slot*)(base + b->off_slots);
-  const pk::BatchStep* steps = (const pk::BatchStep*)(base + b->off_steps);
-  const pk::Run* runs = (const pk::Run*)(base + b->off_runs);
+  const int* order = (const int*)(base + b->off_order);
+  const unsigned char* blobs = (const unsigned char*)(base + b->off_blobs);
   void* arena = base + b->off_arena;
   pk::Meta* meta = (pk::Meta*)(base + b->off_meta);
   pk::SliceResult* res = (pk::SliceResult*)(base + b->off_results);
   unsigned* counter = (unsigned*)(base + b->off_counter);
-  int ktab = b->ktab;
-  void* args[] = {&knots, &n, &recs, &slots, &steps, &runs, &arena, &meta, &res, &counter, &ktab};
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, func, b->threads, smem);
-  if (e != cudaSuccess) return e;
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
-  const int grid = std::max(1, std::min(per_sm * sms, n));
-  cudaKernelNodeParams kp;
-  std::memset(&kp, 0, sizeof(kp));
-  kp.func = func;
-  kp.gridDim = dim3((unsigned)grid);
-  kp.blockDim = dim3((unsigned)b->threads);
-  kp.sharedMemBytes = (unsigned)smem;
-  kp.kernelParams = args;
-  e = cudaGraphAddKernelNode(&kernel_node, b->graph, &memset_node, 1, &kp);
-  if (e != cudaSuccess) return e;
+  // two independent launches: the knots of the most work by clusters, the others a CTA each
+  for (int big = 1; big >= 0; --big) {
+    int first = big ? 0 : b->n_big, last = big ? b->n_big : b->n;
+    if (last <= first) continue;
+    void* func = batch_kernel(b->precision, b->threads, big != 0);
+    const size_t smem = (size_t)b->smem;
+    e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int records = b->smem, per_sm = 0;
+    const int threads = big ? pk::kClThreads : b->threads;
+    void* args[] = {&knots, &order, &first, &last, &recs, &slots, &blobs, &arena, &meta, &res, &counter, &records};
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, func, threads, smem);
+    if (e != cudaSuccess) return e;
+    cudaKernelNodeParams kp;
+    std::memset(&kp, 0, sizeof(kp));
+    kp.func = func;
+    kp.gridDim = dim3((unsigned)(big ? pk::kCl * std::min(sms / pk::kCl, last - first)
+                                     : std::max(1, std::min(per_sm * sms, last - first))));
+    kp.blockDim = dim3((unsigned)threads);
+    kp.sharedMemBytes = (unsigned)smem;
+    kp.kernelParams = args;
+    cudaGraphNode_t node;
+    e = cudaGraphAddKernelNode(&node, b->graph, &memset_node, 1, &kp);
+    if (e == cudaSuccess && big) {
+      cudaLaunchAttributeValue v;
+      std::memset(&v, 0, sizeof(v));
+      v.clusterDim.x = pk::kCl;
+      v.clusterDim.y = v.clusterDim.z = 1;
+      e = cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributeClusterDimension, &v);
+    }
+    if (e != cudaSuccess) return e;
+  }
   e = cudaGraphInstantiate(&b->exec, b->graph, 0);
   if (e != cudaSuccess) return e;
   b->graph_ws = ws;
@@ -336,8 +314,10 @@ pk_status pk_batch_create(pk_ctx* ctx, const pk_plan* const* plans, int32_t n, i
   b->n = n;
   b->device = ctx ? ctx->device : -1;
   b->threads = ctx ? ctx->tuning.batch_threads : kTunedDefault.batch_threads;
-  b->ktab = ctx ? ctx->tuning.batch_ktab : kTunedDefault.batch_ktab;
+  b->smem = 32 * (ctx ? ctx->tuning.batch_ktab : kTunedDefault.batch_ktab);
   int64_t arena = 0, meta = 0;
+  std::vector<uint8_t> blob;
+  std::vector<double> work;
   for (int32_t i = 0; i < n; ++i) {
     if (!plans[i]) {
       delete b;
@@ -349,45 +329,47 @@ pk_status pk_batch_create(pk_ctx* ctx, const pk_plan* const* plans, int32_t n, i
     k.recipe0 = (int64_t)b->recipes.size();
     k.n_recipe = (int64_t)P.recipes.size();
     k.slot_base = (int64_t)b->slots.size();
-    k.step0 = (int64_t)b->steps.size();
-    k.n_steps = (int64_t)P.steps.size();
+    pk::WaveRange rg;
+    k.n_lev = pk::wave_batch(P, blob, rg);
+    k.blob = (int64_t)b->blobs.size();
+    k.blob_bytes = (int32_t)blob.size();
+    k.item = (int32_t)rg.item;
+    k.lev = (int32_t)rg.lev;
+    k.n_meta = (int32_t)P.tensors.size();
+    b->blobs.insert(b->blobs.end(), blob.begin(), blob.end());
+    work.push_back(P.cmacs);
     k.arena_off = arena;
     k.meta_off = meta;
     k.n_slices = P.n_slices;
-    k.final_offset = P.tensors[P.final_tensor].offset;
+    k.final_offset = P.wave[PK_C64].off[P.final_tensor];
     k.n_sliced = (int32_t)P.sliced.size();
     k.q = P.q;
     k.final_tensor = P.final_tensor;
     b->knots.push_back(k);
-    b->recipes.insert(b->recipes.end(), P.recipes.begin(), P.recipes.end());
-    b->slots.insert(b->slots.end(), P.slots.begin(), P.slots.end());
-    for (const pk::Step& st : P.steps) {
-      pk::BatchStep bs;
-      std::memset(&bs, 0, sizeof(bs));
-      bs.a = st.a;
-      bs.b = st.b;
-      bs.c = st.c;
-      bs.nrow = (int16_t)st.nrow;
-      bs.nk = (int16_t)st.nk;
-      bs.nn = (int16_t)st.nn;
-      bs.off_a = st.off_a;
-      bs.off_b = st.off_b;
-      bs.off_c = st.off_c;
-      bs.R = st.R;
-      bs.K = st.K;
-      bs.N = st.N;
-      bs.run0 = (int64_t)b->runs.size();
-      b->runs.insert(b->runs.end(), st.row, st.row + st.nrow);
-      b->runs.insert(b->runs.end(), st.kr, st.kr + st.nk);
-      b->runs.insert(b->runs.end(), st.nr, st.nr + st.nn);
-      b->steps.push_back(bs);
+    for (int32_t j = 0; j < P.n_init; ++j) {
+      b->recipes.push_back(P.recipes[j]);
+      b->recipes.back().offset = P.wave[PK_C64].off[j];
     }
+    b->slots.insert(b->slots.end(), P.slots.begin(), P.slots.end());
     b->kinfo.push_back(P.knot);
     b->factor.push_back(P.factor);
+    b->prefactor.push_back(pk::jones_defined(P.knot) ? pk::jones_prefactor(P.knot, P.q) : pk::Scaled());
     b->qs.push_back(P.q);
-    arena += (P.arena_elems + 63) / 64 * 64;
+    arena += (P.wave[PK_C64].arena_elems + 63) / 64 * 64;
     meta += (int64_t)P.tensors.size();
   }
+  // the most work first: the launch ends with the small knots
+  b->order.resize((size_t)n);
+  for (int32_t i = 0; i < n; ++i) b->order[i] = i;
+  std::stable_sort(b->order.begin(), b->order.end(), [&](int32_t x, int32_t y) { return work[x] > work[y]; });
+  // a knot goes to a cluster when one CTA would need both more than the levels' own latency (about
+  // 10^5 cycles) and more than its share of the whole batch; a multiprocessor does 0.5
+  // complex multiply-adds per cycle in FP64, 2.7 in float-float, 8 in complex64
+  const double rate = precision == PK_C128 ? 0.5 : precision == PK_SPLIT ? 2.7 : 8.0;
+  double total = 0;
+  for (double w : work) total += w;
+  const double share = std::max(1e5, total / rate / 152);
+  while (b->n_big < n && work[b->order[b->n_big]] / rate > share) ++b->n_big;
   const uint64_t eb = precision == PK_C64 ? 8 : 16;
   uint64_t off = 0;
   b->off_knots = off;
@@ -396,10 +378,10 @@ pk_status pk_batch_create(pk_ctx* ctx, const pk_plan* const* plans, int32_t n, i
   off = pk::a256(off + sizeof(pk::Recipe) * std::max<size_t>(1, b->recipes.size()));
   b->off_slots = off;
   off = pk::a256(off + sizeof(pk::Slot) * std::max<size_t>(1, b->slots.size()));
-  b->off_steps = off;
-  off = pk::a256(off + sizeof(pk::BatchStep) * std::max<size_t>(1, b->steps.size()));
-  b->off_runs = off;
-  off = pk::a256(off + sizeof(pk::Run) * std::max<size_t>(1, b->runs.size()));
+  b->off_order = off;
+  off = pk::a256(off + 4 * std::max<size_t>(1, b->order.size()));
+  b->off_blobs = off;
+  off = pk::a256(off + std::max<size_t>(16, b->blobs.size()));
   b->image_bytes = off;
   b->off_meta = off;
   off = pk::a256(off + 16ull * (uint64_t)std::max<int64_t>(1, meta));
@@ -417,10 +399,8 @@ pk_status pk_batch_create(pk_ctx* ctx, const pk_plan* const* plans, int32_t n, i
                 sizeof(pk::Recipe) * b->recipes.size());
   if (!b->slots.empty())
     std::memcpy(b->image.data() + b->off_slots, b->slots.data(), sizeof(pk::Slot) * b->slots.size());
-  if (!b->steps.empty())
-    std::memcpy(b->image.data() + b->off_steps, b->steps.data(), sizeof(pk::BatchStep) * b->steps.size());
-  if (!b->runs.empty())
-    std::memcpy(b->image.data() + b->off_runs, b->runs.data(), sizeof(pk::Run) * b->runs.size());
+  if (!b->order.empty()) std::memcpy(b->image.data() + b->off_order, b->order.data(), 4 * b->order.size());
+  if (!b->blobs.empty()) std::memcpy(b->image.data() + b->off_blobs, b->blobs.data(), b->blobs.size());
   *out = b;
   return PK_OK;
 }
@@ -458,8 +438,8 @@ pk_status pk_batch_upload_inputs(pk_ctx* ctx, pk_batch* b, void* d_ws, uint64_t 
       return bfail(ctx, PK_ENOMEM, "pinned host allocation failed");
     std::memcpy(b->pinned, b->image.data(), b->image_bytes);
   }
-  // knots, recipes and slots lie first in the image, the steps and runs after them
-  const uint64_t n = b->off_steps - b->off_knots;
+  // knots, recipes and slots lie first in the image, the order and the level records after them
+  const uint64_t n = b->off_order - b->off_knots;
   cudaError_t e = cudaMemcpyAsync((char*)d_ws + b->off_knots, b->pinned + b->off_knots, n,
                                   cudaMemcpyHostToDevice, ctx->stream);
   if (e != cudaSuccess) return bfail(ctx, PK_ECUDA, std::string("batch upload: ") + cudaGetErrorString(e));
@@ -507,7 +487,7 @@ pk_status pk_batch_download(pk_ctx* ctx, pk_batch* b, const void* d_ws, pk_scale
         status = PK_EINVAL;
         continue;
       }
-      pk::Scaled v = pk::s_mul(pk::jones_prefactor(k, b->qs[i]), z);
+      pk::Scaled v = pk::s_mul(b->prefactor[i], z);
       V[i].re = v.re;
       V[i].im = v.im;
       V[i].exp2 = v.e;

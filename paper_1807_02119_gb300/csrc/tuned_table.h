@@ -123,4 +123,4 @@
 #pragma once
 #include "pk.h"
 
-constexpr pk_tuning kTunedDefault = {256, 512, 65536, 1048576, 2048, 8, 0, 12, 100, 32000, 25, 4000, 65536};
+constexpr pk_tuning kTunedDefault = {512, 2048, 65536, 1048576, 2048, 8, 0, 12, 100, 32000, 25, 4000, 65536};
