@@ -530,13 +530,13 @@ pk_status pk_plan_launches(const pk_plan* p, int32_t precision, int64_t* launche
   if (!p || !launches || !valid_precision(precision)) return PK_EINVAL;
   const pk::Plan& P = p->p;
   const int64_t widen = (precision == PK_C64 && !P.conv.empty()) ? 1 : 0;
-  int64_t digits = 0;   // split and complex128: one conversion launch per tensor-core step
+  int64_t digits = 0;   // split and complex128: one conversion launch per tensor-core step of its own digit kernel
   if (precision == PK_C128 && P.tc64_bytes > 0)
     for (const pk::WaveStage& g : P.wave[PK_C128].stages[1])
       digits += g.kind == pk::WaveStage::STEP && pk::tc64_step(P.steps[g.step]);
   if (precision == PK_SPLIT)
     for (const pk::WaveStage& g : P.wave[PK_SPLIT].stages[0])
-      digits += g.kind == pk::WaveStage::STEP && P.steps[g.step].tc;
+      digits += g.kind == pk::WaveStage::STEP && P.steps[g.step].tc && P.steps[g.step].K > pk::kTcShortK;
   // steps saved by the level launches (a complex128 tail's steps are never inside one)
   const int fp64 = precision == PK_C128;
   const int64_t fused = P.wave[precision].n_fused_steps[fp64] - P.wave[precision].n_fused[fp64];

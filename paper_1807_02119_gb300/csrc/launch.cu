@@ -17,6 +17,7 @@
 #include "handles.h"
 #include "kernels.cuh"
 #include "gemm_tc.cuh"
+#include "gemm_short.cuh"
 #include "wave.cuh"
 #include "gemm_d64.cuh"
 
@@ -259,6 +260,20 @@ cudaError_t launch_tc(const Step& s, Cx<ff>* arena, Meta* meta, unsigned char* t
   return cudaGetLastError();
 }
 
+// The same step as one launch when K is short (gemm_short.cuh).
+template <int S>
+cudaError_t launch_short(const Step& s, Cx<ff>* arena, Meta* meta, unsigned long long* err, cudaStream_t stream,
+                         Marker& mk, double cm, double by) {
+  const tcs::Geom g = tcs::geom(s);
+  const int runs = tcs::col_runs(g, 2LL * g_sms);
+  const long long grid = g.row_blocks * runs;
+  mk.begin(5, cm, by, gpu_fill(grid, 2));
+  auto fn = g.octs == 1 ? k_gemm_short<S, 1> : g.octs == 2 ? k_gemm_short<S, 2> : k_gemm_short<S, 4>;
+  launch_kernel(fn, dim3((unsigned)grid), tcs::kThreads, tcs::smem_bytes(S, g.octs), stream, mk.pdl(), 1, s, arena, meta, runs, err);
+  mk.end();
+  return cudaGetLastError();
+}
+
 // complex128 on the tensor cores: the digits of both operands, then the GEMM.
 cudaError_t launch_tc64(const Step& s, Cx<double>* arena, Meta* meta, unsigned char* tcs,
                         unsigned long long* err, cudaStream_t stream, Marker& mk, double cm, double by) {
@@ -284,6 +299,10 @@ cudaError_t launch_step(const Step& s, Cx<R>* arena, Meta* meta, Cx<double>* par
   const long long gemm_tiles = ((s.M + 63) / 64) * ((s.N + 63) / 64) * s.Bsz;
   cudaError_t e;
   if constexpr (std::is_same<R, ff>::value) {
+    // K <= 32: one kernel (a step of 7.8e4 multiply-adds 23 -> TBD us)
+    if (s.tc && tc_scratch && err && s.K <= tcs::kMaxK)
+      return s.tc == 4 ? launch_short<4>(s, arena, meta, err, stream, mk, cm, by)
+                       : launch_short<5>(s, arena, meta, err, stream, mk, cm, by);
     if (s.tc && tc_scratch && err)  // digits of A and B, then the tensor-core GEMM
       return s.tc == 4
                  ? launch_tc<4>(s, arena, meta, tc_scratch, counter, err, stream, mk, cm, by, db_groups)
@@ -591,6 +610,15 @@ cudaError_t prepare_gemm_tc() {
                               cudaSharedmemCarveoutMaxShared);
 }
 
+template <int S, int OCTS>
+cudaError_t prepare_short() {
+  const cudaError_t e = cudaFuncSetAttribute(k_gemm_short<S, OCTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             tcs::smem_bytes(S, OCTS));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_gemm_short<S, OCTS>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                              cudaSharedmemCarveoutMaxShared);
+}
+
 template <int S>
 cudaError_t prepare_tc() {
   cudaError_t e;
@@ -598,6 +626,9 @@ cudaError_t prepare_tc() {
   if ((e = prepare_gemm_tc<S, false, true>()) != cudaSuccess) return e;
   if ((e = prepare_gemm_tc<S, true, false>()) != cudaSuccess) return e;
   if ((e = prepare_gemm_tc<S, true, true>()) != cudaSuccess) return e;
+  if ((e = prepare_short<S, 1>()) != cudaSuccess || (e = prepare_short<S, 2>()) != cudaSuccess ||
+      (e = prepare_short<S, 4>()) != cudaSuccess)
+    return e;
   return cudaFuncSetAttribute(k_digits<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               tc::Cfg<S>::kConvSmem);
 }

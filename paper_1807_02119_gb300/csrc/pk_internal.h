@@ -234,6 +234,7 @@ struct TailStep {
 // columns of B, each stored as two real columns [Re B; -Im B] and [Im B; Re B] (the
 // complex doubling sits on B, the operand the planner keeps smaller).
 constexpr int kTcMc = 128, kTcNc = 24, kTcKc = 16;
+constexpr int kTcShortK = 32;   // up to this K such a step is one launch without digit scratch (gemm_short.cuh)
 PK_HD constexpr long long tc_a_chunk(int S) { return (long long)S * kTcMc * (2 * kTcKc) * 2; }
 PK_HD constexpr long long tc_b_chunk(int S) { return (long long)S * (2 * kTcNc) * (2 * kTcKc) * 2; }
 // Chunks per flush group: the S digit pairs of a level, 2 kTcKc real terms per chunk and
