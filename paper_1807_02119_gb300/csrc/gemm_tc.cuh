@@ -260,52 +260,95 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
-// The S digit slices of one real component of 8 consecutive k of one tile row: x[u] =
-// (hi, lo) of k = 8 o + u, scaled by f1 f2 = 2^(7 - e) (e the row's exponent over the
-// group, |hi| < 2^e; two exact powers of two, so that any exponent the stored values can
-// have is covered), giving float-float values y = (yh + yl) with |y| < 2^7.  Digit i is
-// the nearest integer d_i of the running remainder times 2^(8i): rounding by adding and
-// subtracting 1.5 * 2^23 (exact round-to-nearest-even on the FP32 adder for |yh| < 2^22,
-// no conversion instruction); the remainder r = yh - d_i is exact and a multiple of
-// ulp(yh), while |yl| <= ulp(yh) / 2, so |r| >= |yl| unless r = 0 and the fast two-sum
-// (Dekker) that renormalises (r + yl) is exact.  An integer d_i with |d_i| <= 256 keeps
-// only the top 16 bits of its FP32 pattern, which are its BF16 pattern.  Digit i of the 8
-// values, packed into 16 bytes (one core-matrix row), goes to out + i * slice and, when
-// out2 is given, also to out2 + i * slice, negated if `neg2`.
-template <int S>
-__device__ __forceinline__ void digit_rows8(const float* xh, const float* xl, float f1, float f2,
-                                            unsigned char* out, unsigned char* out2, bool neg2,
-                                            int slice) {
-  constexpr float kRound = 12582912.0f;   // 1.5 * 2^23
-  float yh[8], yl[8];
+// 8 consecutive columns of five levels `step` columns apart, one wait.
+__device__ __forceinline__ void tmem_ld8x5(uint32_t ta, uint32_t step, float (*v)[8]) {
+  uint32_t r[40];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%40];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%41];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16, %17, %18, %19, %20, %21, %22, %23}, [%42];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24, %25, %26, %27, %28, %29, %30, %31}, [%43];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32, %33, %34, %35, %36, %37, %38, %39}, [%44];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
+        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+        "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]),
+        "=r"(r[38]), "=r"(r[39])
+      : "r"(ta), "r"(ta + step), "r"(ta + 2 * step), "r"(ta + 3 * step), "r"(ta + 4 * step));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    yh[u] = (xh[u] * f1) * f2;
-    yl[u] = (xl[u] * f1) * f2;
+  for (int i = 0; i < 40; ++i) v[i / 8][i % 8] = __uint_as_float(r[i]);
+}
+
+// The S digits of 2 NP consecutive k of one real component, two BF16 to a word: v(u) = (hi, lo)
+// of k = u, the first `cnt` of them nonzero, scaled by 2^(7 - e) (e the row's exponent over the
+// group, |hi| < 2^e; two exact powers of two, so that any exponent the stored values can have is
+// covered), giving float-float values y = (yh + yl) with |y| < 2^7.  Digit i, kept as
+// d_i 2^(-8i), is the running remainder rounded to a multiple of 2^(-8i) by adding and
+// subtracting 1.5 * 2^(23-8i) (exact round-to-nearest-even on the FP32 adder, no conversion
+// instruction); the remainder r = yh - d is exact and a multiple of ulp(yh), while
+// |yl| <= ulp(yh) / 2, so |r| >= |yl| unless r = 0 and the fast two-sum (Dekker) that
+// renormalises (r + yl) is exact.  An integer |d_i| <= 256 keeps only the top 16 bits of its
+// FP32 pattern, which are its BF16 pattern; the factor 2^(-8i) saves the remainder's scaling
+// (two of eight instructions a digit) and the epilogue's weights, since the products of a level
+// share one factor.
+template <int S, int NP, typename Get>
+__device__ __forceinline__ void digit_pairs(Get v, int cnt, int e, uint32_t (*w)[NP]) {
+  float f1, f2;
+  pow2_pair(7 - e, f1, f2);
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    if (2 * p >= cnt) {
+#pragma unroll
+      for (int i = 0; i < S; ++i) w[i][p] = 0;
+      continue;
+    }
+    const float2 v0 = v(2 * p), v1 = v(2 * p + 1);
+    float y[4] = {(v0.x * f1) * f2, (v1.x * f1) * f2, (v0.y * f1) * f2, (v1.y * f1) * f2};
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      const float round = __int_as_float(((127 + 23 - 8 * i) << 23) | 0x400000);   // 1.5 * 2^(23-8i)
+      float d[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        d[u] = __fsub_rn(__fadd_rn(y[u], round), round);
+        if (i + 1 < S) {
+          const float r = __fsub_rn(y[u], d[u]);
+          const float sum = __fadd_rn(r, y[u + 2]);
+          y[u + 2] = __fsub_rn(y[u + 2], __fsub_rn(sum, r));
+          y[u] = sum;
+        }
+      }
+      w[i][p] = __byte_perm(__float_as_uint(d[0]), __float_as_uint(d[1]), 0x7632);
+    }
   }
-  const uint32_t flip = neg2 ? 0x80008000u : 0u;   // negate the BF16 digits (exact)
+}
+
+// Digit i of 2 NP values to out + i * slice, negated if `flip`.
+template <int S, int NP>
+__device__ __forceinline__ void store_pairs(const uint32_t (*w)[NP], unsigned char* out, uint32_t flip, int slice) {
 #pragma unroll
   for (int i = 0; i < S; ++i) {
-    uint32_t w[4];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const float di = __fsub_rn(__fadd_rn(yh[u], kRound), kRound);
-      if (u & 1)   // BF16 of value u - 1 in the low half, of u in the high half
-        w[u >> 1] = __byte_perm(w[u >> 1], __float_as_uint(di), 0x7632);
-      else
-        w[u >> 1] = __float_as_uint(di);
-      if (i + 1 < S) {
-        const float r = __fsub_rn(yh[u], di);
-        const float sum = __fadd_rn(r, yl[u]);
-        const float err = __fsub_rn(yl[u], __fsub_rn(sum, r));
-        yh[u] = sum * 256.0f;
-        yl[u] = err * 256.0f;
-      }
-    }
-    *(uint4*)(out + i * slice) = make_uint4(w[0], w[1], w[2], w[3]);
-    if (out2)
-      *(uint4*)(out2 + i * slice) = make_uint4(w[0] ^ flip, w[1] ^ flip, w[2] ^ flip, w[3] ^ flip);
+    if constexpr (NP == 4)
+      *(uint4*)(out + i * slice) = make_uint4(w[i][0] ^ flip, w[i][1] ^ flip, w[i][2] ^ flip, w[i][3] ^ flip);
+    else if constexpr (NP == 2)
+      *(uint2*)(out + i * slice) = make_uint2(w[i][0] ^ flip, w[i][1] ^ flip);
+    else
+      *(uint32_t*)(out + i * slice) = w[i][0] ^ flip;
   }
+}
+
+// 8 consecutive k (one core-matrix row, 16 bytes) to out and, when given, to out2, there
+// negated if `neg2` (exact).
+template <int S, typename Get>
+__device__ __forceinline__ void digit_rows8(Get v, int cnt, int e, unsigned char* out,
+                                            unsigned char* out2, bool neg2, int slice) {
+  uint32_t w[S][4];
+  digit_pairs<S, 4>(v, cnt, e, w);
+  store_pairs<S, 4>(w, out, 0u, slice);
+  if (out2) store_pairs<S, 4>(w, out2, neg2 ? 0x80008000u : 0u, slice);
 }
 
 }  // namespace tc
@@ -420,29 +463,23 @@ __device__ __forceinline__ void digits_block(const Step& s, const Cx<ff>* arena,
   const int octs = kgn / 8;
   for (int idx = tid; idx < kRows * octs; idx += kConvThreads) {
     const int r = idx % kRows, o = idx / kRows;
-    float sc1, sc2;   // 2^(7 - e): the row's largest entry below 2^7
-    pow2_pair(7 - ex[r], sc1, sc2);
     const long long k = k0 + 8 * o;
     const int kl = (int)(k % kKc);   // 0 or 8
     unsigned char* ch = dst0 + (k / kKc) * (long long)kChunkBytes;
     const float4* row = tile + r * kLd + 8 * o;
+    const int cnt = (int)min(8LL, s.K - k);   // the rest of a padded chunk is 0
 #pragma unroll
     for (int part = 0; part < 2; ++part) {   // the real, then the imaginary components
-      float xh[8], xl[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float4 v = row[u];
-        xh[u] = part ? v.z : v.x;
-        xl[u] = part ? v.w : v.y;
-      }
+      const float2* half = (const float2*)row + part;
+      auto x = [&](int u) { return half[2 * u]; };
       if (IS_A)   // row [Re | Im]
-        digit_rows8<S>(xh, xl, sc1, sc2, ch + tile_off(r0 + r, part * kKc + kl, kKcores), nullptr,
+        digit_rows8<S>(x, cnt, ex[r], ch + tile_off(r0 + r, part * kKc + kl, kKcores), nullptr,
                        false, kSlice);
       else if (part == 0)   // Re: row 2r first half, row 2r + 1 second half
-        digit_rows8<S>(xh, xl, sc1, sc2, ch + tile_off(2 * r, kl, kKcores),
+        digit_rows8<S>(x, cnt, ex[r], ch + tile_off(2 * r, kl, kKcores),
                        ch + tile_off(2 * r + 1, kKc + kl, kKcores), false, kSlice);
       else                  // Im: row 2r + 1 first half, -Im: row 2r second half
-        digit_rows8<S>(xh, xl, sc1, sc2, ch + tile_off(2 * r + 1, kl, kKcores),
+        digit_rows8<S>(x, cnt, ex[r], ch + tile_off(2 * r + 1, kl, kKcores),
                        ch + tile_off(2 * r, kKc + kl, kKcores), true, kSlice);
     }
   }
@@ -728,10 +765,10 @@ __global__ void __launch_bounds__(tc::kThreads, DB ? 1 : 2) k_gemm_tc(const Step
           break;
         }
         fence_after();
-        // level L holds an integer sum of digit products (below 2^24 in magnitude) at weight
-        // 2^(-14-8L).  Per 8 columns: levels 0 and 1 are added exactly (TwoSum); levels 2 ..
-        // S-1, at most 2^-16 of level 0's scale, are folded into the low part with FP32 FMAs,
-        // whose rounding (below 2^-40 of level 0's scale) is under the digits' truncation.
+        // level L holds 2^(-8L) times an integer sum of digit products (below 2^24 in
+        // magnitude).  Per 8 columns: levels 0 and 1 are added exactly (TwoSum); levels 2 ..
+        // S-1, at most 2^-16 of level 0's scale, are added to the low part in FP32, whose
+        // rounding (below 2^-40 of level 0's scale) is under the digits' truncation.
         // The sum is scaled by the group's 2^(e(m) + e(n) - 14) (powers of two: exact) and
         // added to the float-float accumulators.
         const uint32_t ta0 =
@@ -742,25 +779,24 @@ __global__ void __launch_bounds__(tc::kThreads, DB ? 1 : 2) k_gemm_tc(const Step
           float hi[8], lo[8];
           tmem_ld8x2(ta0 + c8 * 8, ta0 + kN + c8 * 8, hi, lo);   // levels 0 and 1
 #pragma unroll
-          for (int i = 0; i < 8; ++i) two_sum(hi[i], lo[i] * 0.00390625f, hi[i], lo[i]);   // exact
+          for (int i = 0; i < 8; ++i) two_sum(hi[i], lo[i], hi[i], lo[i]);   // exact
 #pragma unroll
           for (int lv = 2; lv < S; lv += 2) {
             float v[8], v2[8];
-            const float w = __int_as_float((127 - 8 * lv) << 23);   // 2^(-8L) relative to level 0
             if (lv + 1 < S) {
               tmem_ld8x2(ta0 + lv * kN + c8 * 8, ta0 + (lv + 1) * kN + c8 * 8, v, v2);
-              const float w2 = w * 0.00390625f;
 #pragma unroll
-              for (int i = 0; i < 8; ++i) lo[i] = fmaf(v2[i], w2, fmaf(v[i], w, lo[i]));
+              for (int i = 0; i < 8; ++i) lo[i] = (lo[i] + v[i]) + v2[i];
             } else {
               tmem_ld8(ta0 + lv * kN + c8 * 8, v);
 #pragma unroll
-              for (int i = 0; i < 8; ++i) lo[i] = fmaf(v[i], w, lo[i]);
+              for (int i = 0; i < 8; ++i) lo[i] += v[i];
             }
           }
 #pragma unroll
           for (int i = 0; i < 8; i += 2) {
-            float f1, f2;   // one exponent per complex column: (re, im) = columns i, i + 1
+            // one exponent per complex column: (re, im) = columns i, i + 1
+            float f1, f2;
             pow2_pair(eam - 14 + eb_s[ew][(c8 * 8 + i) >> 1], f1, f2);
 #pragma unroll
             for (int u = i; u < i + 2; ++u) {

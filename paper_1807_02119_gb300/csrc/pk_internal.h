@@ -163,6 +163,12 @@ struct ConvRec {
   int64_t elems;
   int32_t src_meta, dst_meta;
 };
+// Multiplier of the division of y < top by d >= 2: y / d = (y * mul) >> 32, exact while
+// y d < 2^32; 0 (the kernel divides) otherwise.
+inline uint32_t div_mul(int64_t d, int64_t top) {
+  return d < 2 || top * d >= ((int64_t)1 << 32) ? 0 : (uint32_t)(((1ull << 32) + (uint64_t)d - 1) / (uint64_t)d);
+}
+
 // ---- level schedule (wave_plan.cpp): steps of the same tree level run at the same time
 struct WaveRun {           // a stride run with 32-bit extents; y / size = (y mul) >> 32
   uint32_t size, mul, sa, sb;

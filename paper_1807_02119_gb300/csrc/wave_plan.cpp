@@ -29,12 +29,6 @@ bool overlap(const Interval& x, const Interval& y) {
   return x.off < y.off + y.len && y.off < x.off + x.len;
 }
 
-// Multiplier of the division of y < top by d >= 2: y / d = (y * mul) >> 32, exact while
-// y d < 2^32; 0 (the kernel divides) otherwise.
-uint32_t div_mul(int64_t d, int64_t top) {
-  return d < 2 || top * d >= ((int64_t)1 << 32) ? 0 : (uint32_t)(((1ull << 32) + (uint64_t)d - 1) / (uint64_t)d);
-}
-
 // log2 of the lanes that share one output's sum over k: at most kWaveK terms per lane (one
 // round trip for their operands) while the step has few lanes, 16 (8 of a longer sum) while
 // they stay within what the GPU holds at once.
