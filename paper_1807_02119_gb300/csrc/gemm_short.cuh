@@ -170,9 +170,9 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_gemm_short(const __grid_co
   const int col = tid >> 3, bpart = tid & 1, bo = ((tid >> 1) & 3) * OCTS / 4, p0 = ((tid >> 1) & 3) * OCTS & 3;
   const int bk = 8 * bo + 2 * p0;
   const int t0 = s.tiles_n * run / runs, t1 = s.tiles_n * (run + 1) / runs;
-  float2 bv[2 * kPairs];
+  float2 bv[2 * kPairs];   // loaded one tile ahead
   uint32_t bw[S][kPairs];
-  unsigned bcn = 0;
+  unsigned bcn = 0, bwcn = 0;
   int be = 0;
   auto load_b = [&](int t) {
     const unsigned n = (unsigned)(t * s.W + col);
@@ -186,12 +186,13 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_gemm_short(const __grid_co
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
     be = bin_exp(top);
+    bwcn = bcn;
     tc::digit_pairs<S, kPairs>([&](int u) { return bv[u]; }, col < s.W ? K - bk : 0, be, bw);
   };
   auto put_b = [&](int buf) {   // Re: row 2c first half, 2c + 1 second; Im: 2c + 1 first, -Im: 2c second
     if (col >= s.W) return;
     if ((tid & 7) == 0) {
-      cn[buf][col] = bcn;
+      cn[buf][col] = bwcn;
       eb_s[buf][col] = be;
     }
     unsigned char* at = bsm + bo * S * slice + p0 * 4;
@@ -222,6 +223,7 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_gemm_short(const __grid_co
   }
   conv_b();
   put_b(0);
+  if (t0 + 1 < t1) load_b(t0 + 1);
   top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 8));
   const int e = bin_exp(top);
   if (part == 0) ea_s[arow] = e;
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_gemm_short(const __grid_co
   bool failed = false;
   for (int t = t0; t < t1; ++t) {
     const int buf = (t - t0) & 1;
-    if (tid == 0) {   // A digit i meets B digits 0 .. S-1-i: levels i .. S-1 lie one after another
+    if (tid == kThreads - 32) {   // a warp without columns of B.  A digit i meets B digits 0 .. S-1-i: levels i .. S-1 lie one after another
       const uint64_t da0 = tc::smem_desc(smem_u32(dsm), 128, 256), db0 = tc::smem_desc(smem_u32(bsm), 128, 256);
 #pragma unroll 1
       for (int o = 0; o < OCTS; ++o)
@@ -271,8 +273,8 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_gemm_short(const __grid_co
     }
     __syncwarp();
     if (t + 1 < t1) {   // the next tile's digits, in registers while the tensor cores read this one's
-      load_b(t + 1);
       conv_b();
+      if (t + 2 < t1) load_b(t + 2);
     }
     if (!tc::mbar_wait(smem_u32(&done), (uint32_t)buf, err)) {
       if (lane == 0) {
@@ -351,7 +353,7 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_gemm_short(const __grid_co
   // ---- give-up path: the MMAs in flight are waited for (bounded) before their memory is freed;
   // tiles not reached are left to the error word, which turns the result into a timeout
   if (bad) {
-    if (tid == 0) {
+    if (tid == kThreads - 32) {
       tc::commit(smem_u32(&drain));
       tc::mbar_wait(smem_u32(&drain), 0u, nullptr);
     }
