@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_gemm_short(const __grid_co
   const int en = bin_exp(bits_to_val<float>(ma.maxbits)) + bin_exp(bits_to_val<float>(mb.maxbits));
   if (blockIdx.x == 0 && run == 0 && tid == 0) meta[s.c].exp = ma.exp + mb.exp + en;
   const bool plain = en >= -126 && en <= 126;
-  const int ex0 = (plain ? -en : 0) - 14;
+  const int ex0 = (plain ? -en : 0) - 14 + 127;   // biased as a float's exponent
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   tc::fence_before();
   __syncthreads();
@@ -307,37 +307,31 @@ __global__ void __launch_bounds__(tcs::kThreads, 2) k_gemm_short(const __grid_co
         for (int l = 2; l < S; ++l) lo[i] += lv[l][i];
       }
       float f[4];
-      bool far = false;
+      bool far = !plain;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         // the row's and the column's exponent and the step's normalisation (a power of two) at once
-        const int x = ea + eb_s[buf][min(b * 4 + j, tc::kNc - 1)], xc = max(-126, min(127, x));
-        f[j] = __int_as_float((xc + 127) << 23);
-        far |= x != xc;
+        const int x = ea + eb_s[buf][b * 4 + j];
+        f[j] = __int_as_float(x << 23);
+        far |= (unsigned)(x - 1) >= 254u;
       }
-      if (__any_sync(0xffffffffu, far)) {   // beyond a float's exponents: in three factors
+      if (__any_sync(0xffffffffu, far)) {   // beyond a float's exponents: factor by factor
+        const float scale = plain ? 1.f : (float)ldexp(1.0, -en);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           float f1, f2;
-          const int x = ea + eb_s[buf][min(b * 4 + i / 2, tc::kNc - 1)];
-          tc::pow2_pair(x - max(-126, min(127, x)), f1, f2);
-          hi[i] = (hi[i] * f1) * f2;
-          lo[i] = (lo[i] * f1) * f2;
+          tc::pow2_pair(ea + eb_s[buf][b * 4 + i / 2] - 127, f1, f2);
+          hi[i] = ((hi[i] * f1) * f2) * scale;
+          lo[i] = ((lo[i] * f1) * f2) * scale;
         }
+        f[0] = f[1] = f[2] = f[3] = 1.f;
       }
+      if (failed) f[0] = f[1] = f[2] = f[3] = __int_as_float(0x7fc00000);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int c = b * 4 + j;
         if (!live || c >= nv) continue;
-        ff re = ff_norm(hi[2 * j] * f[j], lo[2 * j] * f[j]), im = ff_norm(hi[2 * j + 1] * f[j], lo[2 * j + 1] * f[j]);
-        if (!plain) {
-          const float scale = (float)ldexp(1.0, -en);
-          re.hi *= scale;
-          re.lo *= scale;
-          im.hi *= scale;
-          im.lo *= scale;
-        }
-        if (failed) re.hi = re.lo = im.hi = im.lo = __int_as_float(0x7fc00000);
+        const ff re = ff_norm(hi[2 * j] * f[j], lo[2 * j] * f[j]), im = ff_norm(hi[2 * j + 1] * f[j], lo[2 * j + 1] * f[j]);
         const Cx<ff> out{re, im};
         st(C + cn[buf][c], out);
         vmax = fmaxf(vmax, mag(out));
