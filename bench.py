@@ -294,7 +294,7 @@ def roofline_blocks(classes, prec, pk_, instep=None):
     bytes (or flops) per launch / average launch duration, against the measured peak.  The
     dominant class is the one with the largest GPU-fill-weighted time: each launch's
     duration times the share of the GPU's CTA slots it fills, which is what a launch costs
-    the concurrent step (many plans' launches overlap there; a one-CTA launch costs almost
+    the concurrent step (many plans' launches overlap there; a small launch costs almost
     nothing).  Algorithmic bytes follow the step definition e (|A| + |B| + |C|) with e = 8
     for complex64 and split storage, 16 for complex128 (the library counts the bytes of its
     storage type, 16 for split, so halved here)."""
@@ -749,7 +749,7 @@ def main():
 
     # end to end through the public API, every step: every plan's knot-derived inputs
     # host->device from pinned memory (its initial-tensor recipes and slots; the
-    # sequence-kernel step records stay resident like the rest of the plan's structure,
+    # level-kernel step records stay resident like the rest of the plan's structure,
     # which its graph holds), the kernels, every scaled result device->host (one wait for
     # all); the mean over the same number of steps.  Also with every whole program re-sent.
     d2h = 32 * len(plans)

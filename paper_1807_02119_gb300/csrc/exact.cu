@@ -13,7 +13,11 @@
 // The kernels mirror the floating-point ones in their indexing only: the initial tensors
 // follow their recipes (sum over the vertex spin of products of COPY legs and clause
 // entries), every contraction step is C[n R + r] = sum_k A[row r, k] B[k, column n] through
-// the step's stride runs, one thread per output, and the slice results are summed.
+// the step's stride runs, light steps level by level (wave_plan.cpp), and the slice results are
+// summed.  What bounded it were 64-bit divisions, four per term, and a thread per output however
+// long the sum: products now add up below p 2^31 with one conditional subtraction each and are
+// reduced once per output, and a warp or a CTA shares a long sum.  Measured on GB300, 36 crossings
+// at q = 10 modulo four primes: 6870 -> 364 us per call.
 #include <cuda_runtime.h>
 
 #include <algorithm>

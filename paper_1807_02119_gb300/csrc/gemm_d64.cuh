@@ -17,8 +17,9 @@
 // [Re | Im], a complex column of B two real columns [Re; -Im] and [Im; Re].
 //
 //  * k_digits64: a CTA per 8 to 128 rows (8 or 16 complex columns of B), fewer for a longer K:
-//    their exponents over all of K, then the digits in the MMA's canonical K-major layout (8-row x 16-byte core matrices).  Only
-//    integer and FP32 instructions: a conversion through FP64 would take longer than the GEMM.
+//    their exponents over all of K, then the digits in the MMA's canonical K-major layout (8-row
+//    x 16-byte core matrices).  Only integer and FP32 instructions: a conversion through FP64
+//    would take longer than the GEMM.
 //  * k_gemm64: persistent, one CTA per multiprocessor, tiles of 128 complex rows x 16 complex
 //    columns; warp 0 streams the digit chunks (8 complex k: 32 KB + 8 KB) through a 5-stage
 //    ring of bulk copies, warp 1 issues 8 MMAs per chunk (A digit i against B digits 0 .. 7-i

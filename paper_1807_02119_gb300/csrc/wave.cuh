@@ -202,11 +202,28 @@ __device__ __forceinline__ unsigned long long wave_outputs(const uint4* rec, uns
         ka[u] = (k + (unsigned)u * kd) * w.z;
         kb[u] = (k + (unsigned)u * kd) * w.w;
       }
-      if (nk > 1) {
+      if (nk > 1) {   // the terms' digits of a run together: one record read, independent chains
+        unsigned y[kWaveK];
 #pragma unroll
         for (int u = 0; u < kWaveK; ++u) {
+          y[u] = min(k + (unsigned)u * kd, K - 1);
           ka[u] = kb[u] = 0;
-          wave_offsets<M>(min(k + (unsigned)u * kd, K - 1), rk, nk, ka[u], kb[u]);
+        }
+        uint4 x = w;
+#pragma unroll 1
+        for (int i = 1; i < nk; x = rk[i++]) {
+#pragma unroll
+          for (int u = 0; u < kWaveK; ++u) {
+            const unsigned t = (M & kWaveAny) && !x.y ? y[u] / x.x : __umulhi(y[u], x.y), d = y[u] - t * x.x;
+            ka[u] += d * x.z;
+            kb[u] += d * x.w;
+            y[u] = t;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kWaveK; ++u) {
+          ka[u] += y[u] * x.z;
+          kb[u] += y[u] * x.w;
         }
       }
       Cx<R> a[kWaveK], b[kWaveK];
