@@ -515,11 +515,13 @@ __global__ void __launch_bounds__(256) k_rows_big(const Step s, Cx<R>* arena, Me
 }
 
 // ------------------------------------------------------------------ GEMM-shaped steps
-// Per batch index b: C_b[m, n] = sum_k A_b[m, k] B_b[k, n] on 64 x 64 output tiles,
-// K in chunks of 16.  Operand tiles are gathered through the stride runs (the index
-// permutation) into shared memory, coalesced along whichever of m/k (A) or k/n (B) is
-// unit-stride in memory; each of the 256 threads accumulates a 4 x 4 block of complex
-// outputs in registers.
+// Per batch index b: C_b[m, n] = sum_k A_b[m, k] B_b[k, n] on 16 T x 16 T output tiles (T = 4, or 2
+// where that leaves most of the GPU idle: launch_step), K in chunks of 16.  Operand tiles are
+// gathered through the stride runs (the index permutation) into shared memory, coalesced along
+// whichever of m/k (A) or k/n (B) is unit-stride in memory; each of the 256 threads accumulates a
+// T x T block of complex outputs in registers, k in order.  A chunk's chain of offsets, gather and
+// two barriers bounds a step of few tiles: the offsets are made a chunk ahead, and with T = 2, whose
+// registers allow it, the gather too, while the chunk before is multiplied.
 // Offsets in A, B and C of index x of a GEMM-view run class (x below the class's extent,
 // at most 2^31: 32-bit division).
 __device__ __forceinline__ void runs4(long long x, const Run4* r, int n, long long& oa,
@@ -536,14 +538,15 @@ __device__ __forceinline__ void runs4(long long x, const Run4* r, int n, long lo
   }
 }
 
-template <typename R>
+template <typename R, int T>
 __global__ void __launch_bounds__(256) k_gemm(const Step s, Cx<R>* arena, Meta* meta) {
   pdl_wait();
   using S = typename Traits<R>::S;
-  constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4, LDA = BM + 1, LDB = BN + 1;
+  constexpr int BM = 16 * T, BN = 16 * T, BK = 16, TM = T, TN = T, LDA = BM + 1, LDB = BN + 1;
+  constexpr bool kAhead = T == 2;
   __shared__ Cx<R> As[BK * LDA];
   __shared__ Cx<R> Bs[BK * LDB];
-  __shared__ long long am[BM], cm[BM], bn[BN], cn[BN], ak[BK], bk[BK];
+  __shared__ long long am[BM], cm[BM], bn[BN], cn[BN], ak[2][BK], bk[2][BK];
   __shared__ long long base[3];
   const int tid = threadIdx.x;
   const long long tiles_m = (s.M + BM - 1) / BM, tiles_n = (s.N + BN - 1) / BN;
@@ -579,49 +582,49 @@ __global__ void __launch_bounds__(256) k_gemm(const Step s, Cx<R>* arena, Meta* 
   const Cx<R>* B = arena + s.off_b + base[1];
   Acc<R> acc[TM][TN];
   const int tx = tid & 15, ty = tid >> 4;
-  for (long long k0 = 0; k0 < s.K; k0 += BK) {
+  auto offsets = [&](long long k0, int buf) {
     if (tid < BK) {
-      long long k = k0 + tid;
-      if (k < s.K) {
-        long long ka, kb;
-        split_runs((unsigned long long)k, s.kr, s.nk, ka, kb);
-        ak[tid] = ka;
-        bk[tid] = kb;
-      } else {
-        ak[tid] = -1;
-        bk[tid] = -1;
-      }
+      long long k = k0 + tid, ka = -1, kb = -1;
+      if (k < s.K) split_runs((unsigned long long)k, s.kr, s.nk, ka, kb);
+      ak[buf][tid] = ka;
+      bk[buf][tid] = kb;
     }
-    __syncthreads();
+  };
+  constexpr int PA = BM * BK / 256, PB = BN * BK / 256;   // gathered entries per thread
+  Cx<R> va[PA], vb[PB];
+  auto gather = [&](int buf) {
 #pragma unroll
-    for (int p = 0; p < (BM * BK) / 256; ++p) {
-      int idx = tid + p * 256, i, j;
-      if (s.a_kinner) {
-        i = idx / BK;
-        j = idx % BK;
-      } else {
-        i = idx % BM;
-        j = idx / BM;
-      }
-      Cx<R> v = czero<R>();
-      if (am[i] >= 0 && ak[j] >= 0) v = ld(A + am[i] + ak[j]);
-      As[j * LDA + i] = v;
+    for (int p = 0; p < PA; ++p) {
+      const int idx = tid + p * 256, i = s.a_kinner ? idx / BK : idx % BM, j = s.a_kinner ? idx % BK : idx / BM;
+      va[p] = czero<R>();
+      if (am[i] >= 0 && ak[buf][j] >= 0) va[p] = ld(A + am[i] + ak[buf][j]);
     }
 #pragma unroll
-    for (int p = 0; p < (BN * BK) / 256; ++p) {
-      int idx = tid + p * 256, j, kk;
-      if (s.b_kinner) {
-        j = idx / BK;
-        kk = idx % BK;
-      } else {
-        j = idx % BN;
-        kk = idx / BN;
-      }
-      Cx<R> v = czero<R>();
-      if (bn[j] >= 0 && bk[kk] >= 0) v = ld(B + bk[kk] + bn[j]);
-      Bs[kk * LDB + j] = v;
+    for (int p = 0; p < PB; ++p) {
+      const int idx = tid + p * 256, j = s.b_kinner ? idx / BK : idx % BN, kk = s.b_kinner ? idx % BK : idx / BN;
+      vb[p] = czero<R>();
+      if (bn[j] >= 0 && bk[buf][kk] >= 0) vb[p] = ld(B + bk[buf][kk] + bn[j]);
     }
+  };
+  offsets(0, 0);
+  __syncthreads();
+  if (kAhead) gather(0);
+  int buf = 0;
+  for (long long k0 = 0; k0 < s.K; k0 += BK, buf ^= 1) {
+    if (!kAhead) gather(buf);
+#pragma unroll
+    for (int p = 0; p < PA; ++p) {
+      const int idx = tid + p * 256, i = s.a_kinner ? idx / BK : idx % BM, j = s.a_kinner ? idx % BK : idx / BM;
+      As[j * LDA + i] = va[p];
+    }
+#pragma unroll
+    for (int p = 0; p < PB; ++p) {
+      const int idx = tid + p * 256, j = s.b_kinner ? idx / BK : idx % BN, kk = s.b_kinner ? idx % BK : idx / BN;
+      Bs[kk * LDB + j] = vb[p];
+    }
+    if (k0 + BK < s.K) offsets(k0 + BK, buf ^ 1);
     __syncthreads();
+    if (kAhead && k0 + BK < s.K) gather(buf ^ 1);
 #pragma unroll 4
     for (int kk = 0; kk < BK; ++kk) {
       Cx<R> a[TM], b[TN];
