@@ -275,7 +275,7 @@ def run_reference(args):
 CLASS_KERNEL = {"build": "k_build", "rows": "k_rows / k_outs / k_waves / k_wave_wide (fused permute-and-contract)",
                 "splitk": "k_splitk", "results": "k_slice_result / k_sum_slices",
                 "gemm": "k_gemm (tiled strided complex GEMM, CUDA cores)",
-                "gemm_tc": "k_gemm_tc (complex GEMM on tcgen05 tensor cores, BF16 digit products)",
+                "gemm_tc": "k_gemm_tc, k_gemm_short (complex GEMM on tcgen05 tensor cores, BF16 digit products)",
                 "digits": "k_digits (operand digits for k_gemm_tc)"}
 # DRAM traffic (ncu dram__bytes_read.sum + dram__bytes_write.sum) of one captured launch
 # divided by that launch's algorithmic bytes as the library counts them (its storage type,
