@@ -10,9 +10,9 @@
 
 namespace pk {
 
-// Measured on GB300, whole evaluations: 205 crossings at q = 3 in complex64 1.11 -> 0.32 ms
-// and 167 crossings at q = 5 in split 1.34 -> 0.56 ms against one small step after another in
-// one CTA; the reverse pass of a 99-crossing knot at q = 5 in split 2.09 -> 0.43 ms.  A level
+// Measured on GB300, whole evaluations: 330 crossings at q = 3 in complex64 1.17 -> 0.35 ms
+// and 167 crossings at q = 5 in split 1.71 -> 0.47 ms (with gemm_short.cuh) against one small step
+// after another in one CTA; the reverse pass of 99 crossings at q = 5 in split 2.11 -> 0.37 ms.  A level
 // of the cluster kernel takes 1.5 to 2 us: 0.16 us for an operand's round trip to L2, 0.3 us
 // for the cluster barrier, the rest one warp's 200 to 300 dependent instructions (FP64
 // multiply-adds: 63 cycles each).  A level launched alone takes 0.9 us more.
