@@ -71,19 +71,27 @@ pk_status check_ws(pk_ctx* ctx, const pk_plan* p, int32_t precision, void*& ws, 
   return check_ws_need(ctx, p->p.ws_bytes(precision), ws, bytes);
 }
 
-// What pk_upload copies for a precision, in pinned memory (kept with the plan): the program and
-// the precision's level records behind it.  NULL when the allocation fails.
-const uint8_t* pinned_image(const pk_plan* p, int32_t precision, uint64_t& n) {
+// What pk_upload copies for a level schedule (a precision or kWaveExact), in pinned memory (kept
+// with the plan): the program and the schedule's records behind it.  NULL when the allocation fails.
+const uint8_t* pinned_image(const pk_plan* p, int32_t sched, uint64_t& n) {
   const pk::Plan& P = p->p;
-  const std::vector<uint8_t>& blob = P.wave[precision].blob;
+  const std::vector<uint8_t>& blob = P.wave[sched].blob;
   n = P.off_wave + blob.size();
-  uint8_t*& pin = const_cast<pk_plan*>(p)->pinned_program[precision];
+  uint8_t*& pin = const_cast<pk_plan*>(p)->pinned_program[sched];
   if (!pin) {
     if (cudaMallocHost((void**)&pin, n + 1) != cudaSuccess) return pin = nullptr;
     std::memcpy(pin, P.program.data(), P.off_wave);
     if (!blob.empty()) std::memcpy(pin + P.off_wave, blob.data(), blob.size());
   }
   return pin;
+}
+
+pk_status upload_image(pk_ctx* ctx, const pk_plan* p, int32_t sched, void* d_workspace) {
+  uint64_t n = 0;
+  const uint8_t* image = pinned_image(p, sched, n);
+  if (!image) return fail(ctx, PK_ENOMEM, "pinned host allocation failed");
+  cudaError_t e = cudaMemcpyAsync(d_workspace, image, n, cudaMemcpyHostToDevice, ctx->stream);
+  return e == cudaSuccess ? PK_OK : cuda_fail(ctx, e, "upload");
 }
 
 // Enqueues the plan's kernels on the context's stream.  The launch sequence is recorded
@@ -566,12 +574,7 @@ pk_status pk_upload(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_wo
   else if (workspace_bytes < p->p.off_arena)
     s = fail(ctx, PK_ENOMEM, "buffer smaller than the plan state (pk_plan_state_bytes)");
   if (s != PK_OK) return s;
-  uint64_t n = 0;
-  const uint8_t* image = pinned_image(p, precision, n);
-  if (!image) return fail(ctx, PK_ENOMEM, "pinned host allocation failed");
-  cudaError_t e = cudaMemcpyAsync(d_workspace, image, n, cudaMemcpyHostToDevice, ctx->stream);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "upload");
-  return PK_OK;
+  return upload_image(ctx, p, precision, d_workspace);
 }
 
 pk_status pk_upload_inputs(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_workspace,
@@ -1214,7 +1217,7 @@ pk_status pk_eval_exact(pk_ctx* ctx, const pk_plan* p, const uint32_t* primes, i
   uint64_t bytes = workspace_bytes;
   pk_status s = check_ws(ctx, p, PK_C64, ws, bytes);
   if (s != PK_OK) return s;
-  if ((s = pk_upload(ctx, p, PK_C64, ws, bytes)) != PK_OK) return s;
+  if ((s = upload_image(ctx, p, pk::kWaveExact, ws)) != PK_OK) return s;
   return exact_residues(ctx, p, primes, n_primes, ws, zab);
 }
 
@@ -1303,7 +1306,7 @@ pk_status pk_jones_coefficients(pk_ctx* ctx, const pk_knot* k, int32_t capacity,
     void* ws = nullptr;
     uint64_t bytes = 0;
     s = check_ws(ctx, p, PK_C64, ws, bytes);
-    if (s == PK_OK) s = pk_upload(ctx, p, PK_C64, ws, bytes);
+    if (s == PK_OK) s = upload_image(ctx, p, pk::kWaveExact, ws);
     if (s == PK_OK) s = exact_residues(ctx, p, primes.data(), np, ws, zab.data() + 2 * (size_t)iq * np);
     pk_plan_destroy(p);
     if (s != PK_OK) return s;

@@ -330,7 +330,7 @@ pk_status pk_batch_create(pk_ctx* ctx, const pk_plan* const* plans, int32_t n, i
     k.n_recipe = (int64_t)P.recipes.size();
     k.slot_base = (int64_t)b->slots.size();
     pk::WaveRange rg;
-    k.n_lev = pk::wave_batch(P, blob, rg);
+    k.n_lev = pk::wave_batch(P, precision != PK_C64, blob, rg);
     k.blob = (int64_t)b->blobs.size();
     k.blob_bytes = (int32_t)blob.size();
     k.item = (int32_t)rg.item;

@@ -278,7 +278,7 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
     for (const Op& op : ops) by_meta.push_back(op.st);
     for (Step& x : by_meta) x.tc = 0;
     G.arena_elems = w.arena_elems;
-    wave_stages(by_meta, tune, kHeavyTc64, w);
+    wave_stages(by_meta, tune, kHeavyTc64, true, w);
     G.tc64_bytes = 0;
     for (const Step& x : by_meta)
       if (p.use_tc && tc64_step(x))

@@ -223,6 +223,7 @@ constexpr int kWaveCtaWarps32 = 16, kWaveCtaWarps64 = 8;   // warps of work per 
 constexpr int kWavePasses = 1;             // passes over a level at most; wider levels fill the GPU
 constexpr int kWaveK = 5;                  // terms whose operands a lane loads together
 constexpr int64_t kWaveOuts = 1LL << 18;   // outputs of a step inside a level at most
+constexpr int32_t kWaveExact = 3;          // Plan::wave of the exact residues (after the precisions')
 
 struct TailStep {
   int32_t step;
@@ -411,7 +412,7 @@ struct Plan {
   std::vector<ConvRec> conv;
   std::shared_ptr<Plan> compact;     // the same plan on its own order's layout, where only that
                                      // fits pk_eval_noalloc's workspace
-  WaveProgram wave[3];               // level schedules by pk_precision (records at off_wave)
+  WaveProgram wave[4];               // level schedules by pk_precision, and kWaveExact (records at off_wave)
   uint64_t off_wave = 0;
   pk_tuning tuning{};                // launch shapes the plan was made with
   std::vector<TailStep> tail;        // one per step >= tail_first
@@ -469,8 +470,8 @@ bool order_stats(const Knot& k, int32_t q, int32_t order, int32_t restarts, doub
 // order (breadth: every ready heavy step before the next levels; otherwise one at a time);
 // `extra` orders further pairs of steps.  wave_layout: first fit over the units' lifetimes,
 // pinned tensors kept to the end; returns the arena's elements.  wave_hazards: the pairs that
-// a given layout orders.  wave_stages: the launches and the device records.  wave_check: a
-// replay of the units over the layout.
+// a given layout orders.  wave_stages: the launches and the device records; shared: lanes may
+// share an output's sum.  wave_check: a replay of the units over the layout.
 enum WaveHeavy : int32_t { kHeavyTc64 = 1, kHeavyTc = 2 };   // launched alone besides: the tensor-core
                                                              // steps of complex128 / of split
 bool wave_light(const Step& s, const pk_tuning& tune);
@@ -486,10 +487,10 @@ int64_t wave_layout(const std::vector<Step>& steps, const std::vector<int64_t>& 
                     std::vector<int64_t>& off);
 void wave_hazards(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
                   const std::vector<int64_t>& off, std::vector<std::pair<int32_t, int32_t>>& edges);
-void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, int32_t heavy, WaveProgram& w);
+void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, int32_t heavy, bool shared, WaveProgram& w);
 // All units of a plan as levels for one CTA (the batch executor): records | items | level table
 // in `blob`, their places in `range`; returns the number of levels.
-int32_t wave_batch(const Plan& p, std::vector<uint8_t>& blob, WaveRange& range);
+int32_t wave_batch(const Plan& p, bool shared, std::vector<uint8_t>& blob, WaveRange& range);
 bool wave_check(const std::vector<Step>& steps, const std::vector<int64_t>& elems,
                 const std::vector<char>& pinned, const WaveProgram& w, std::string& err);
 // The plan's level schedules and the workspace layout that holds them; `compact`: on the

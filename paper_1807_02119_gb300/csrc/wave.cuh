@@ -170,8 +170,8 @@ __device__ __forceinline__ unsigned long long wave_outputs(const uint4* rec, uns
   const unsigned q = chunk * 32 + lane, o = q >> lg;
   unsigned k0 = q & ((1u << lg) - 1), kd = 1u << lg;
   bool live = o < Rr * N;
-  if (std::is_same<R, float>::value && K <= 16) {   // complex64 keeps short sums in order: one lane
-    live = live && k0 == 0;
+  if (std::is_same<R, float>::value) {   // complex64 keeps its sums in order, bit for bit: one lane each
+    live = live && k0 == 0;   // (records made for complex64 alone have one)
     kd = 1;
   }
   WaveAcc<R> part;

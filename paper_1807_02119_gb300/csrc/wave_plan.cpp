@@ -40,7 +40,8 @@ int lanes_log2(int64_t outs, int64_t K) {
   return l;
 }
 
-uint32_t push_record(const Step& s, const std::vector<int64_t>& off, std::vector<uint8_t>& blob, uint32_t per = 1) {
+uint32_t push_record(const Step& s, const std::vector<int64_t>& off, std::vector<uint8_t>& blob, int lanes,
+                     uint32_t per = 1) {
   WaveRec r;
   std::memset(&r, 0, sizeof(r));
   r.a = s.a;
@@ -53,7 +54,7 @@ uint32_t push_record(const Step& s, const std::vector<int64_t>& off, std::vector
   r.nrow = (uint8_t)s.nrow;
   r.nk = (uint8_t)s.nk;
   r.nn = (uint8_t)s.nn;
-  r.lanes = (uint8_t)lanes_log2(s.R * s.N, s.K);
+  r.lanes = (uint8_t)lanes;
   r.off_a = off[s.a];
   r.off_b = s.b >= 0 ? off[s.b] : 0;
   r.off_c = off[s.c];
@@ -299,7 +300,7 @@ bool wave_check(const std::vector<Step>& steps, const std::vector<int64_t>& elem
   return true;
 }
 
-void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, int32_t heavy, WaveProgram& w) {
+void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, int32_t heavy, bool shared, WaveProgram& w) {
   // records, items and level table of all levels in order
   std::vector<uint8_t> recs;
   std::vector<WaveItem> items;
@@ -312,8 +313,10 @@ void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, int32_t 
     const Step& s0 = steps[w.units[u].steps[0]];
     if (w.units[u].heavy && (!wave_light(s0, tune) || ((heavy & kHeavyTc) && s0.tc))) continue;
     for (int32_t i : w.units[u].steps) {
-      const uint32_t at = push_record(steps[i], w.off, recs);
-      const int64_t outs = steps[i].R * steps[i].N, lanes = outs << lanes_log2(outs, steps[i].K);
+      const int64_t outs = steps[i].R * steps[i].N;
+      const int lg = shared ? lanes_log2(outs, steps[i].K) : 0;
+      const uint32_t at = push_record(steps[i], w.off, recs, lg);
+      const int64_t lanes = outs << lg;
       for (int64_t c = 0; c * 32 < lanes; ++c) items.push_back({at, (uint32_t)c});
       weight[u] += (lanes + 31) / 32 * std::max<int64_t>(4, steps[i].K / (lanes / outs));
     }
@@ -383,7 +386,7 @@ void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, int32_t 
   }
 }
 
-int32_t wave_batch(const Plan& p, std::vector<uint8_t>& blob, WaveRange& range) {
+int32_t wave_batch(const Plan& p, bool shared, std::vector<uint8_t>& blob, WaveRange& range) {
   std::vector<WaveItem> items;
   std::vector<uint32_t> lev;
   blob.clear();
@@ -393,9 +396,11 @@ int32_t wave_batch(const Plan& p, std::vector<uint8_t>& blob, WaveRange& range) 
     lev.push_back((uint32_t)items.size());
     for (int32_t i : u.steps) {
       const Step& s = p.steps[i];
-      const int64_t outs = s.R * s.N, lanes = outs << lanes_log2(outs, s.K);
+      const int64_t outs = s.R * s.N;
+      const int lg = shared ? lanes_log2(outs, s.K) : 0;
+      const int64_t lanes = outs << lg;
       const int64_t per = std::max<int64_t>(1, (lanes + 65535) / 65536);   // at most 2048 items a step
-      const uint32_t at = push_record(s, w.off, blob, (uint32_t)per);
+      const uint32_t at = push_record(s, w.off, blob, lg, (uint32_t)per);
       for (int64_t c = 0; c * 32 * per < lanes; ++c) items.push_back({at, (uint32_t)c});
     }
   }
@@ -451,7 +456,14 @@ void plan_waves(Plan& p, bool compact) {
       wave_hazards(p.steps, elems, w.off, edges);
       wave_schedule(p.steps, n, p.tuning, heavy, false, &edges, tail, w.units);
     }
-    wave_stages(p.steps, p.tuning, heavy, w);
+    // complex64 sums keep the steps' own order, a lane each (wave.cuh); the exact residues, whose
+    // sums do not depend on it, share them on the same units and offsets
+    if (prec == PK_C64) {
+      p.wave[kWaveExact] = w;
+      wave_stages(p.steps, p.tuning, heavy, true, p.wave[kWaveExact]);
+      blob = std::max<uint64_t>(blob, p.wave[kWaveExact].blob.size());
+    }
+    wave_stages(p.steps, p.tuning, heavy, prec != PK_C64, w);
     blob = std::max<uint64_t>(blob, w.blob.size());
   }
   // workspace: [recipes | slots | conv | the precision's level records] uploaded, then the
