@@ -24,7 +24,7 @@ def bits(s):
     (57, 9, 314, 346, 3, 81),
     (40, 12, 100, 300, 3, 81),
     (33, 4, 100, 200, 5, 125),
-    (34, 22, 70, 200, 4, 64),
+    (34, 22, 70, 200, 4, 16),
     (20, 3, 30, 60, 3, 9),
 ])
 def test_levels_keep_the_order_of_single_steps(ctx, L, seed, lo, hi, q, longest):
