@@ -76,34 +76,18 @@ __device__ __forceinline__ void ff_acc(float& hi, float& lo, float p, float e) {
 }
 
 // ---- loads, stores, conversions
-template <typename R>
-__device__ __forceinline__ Cx<R> ld(const Cx<R>* p);
-template <>
+// Operands are read by plain loads.  The read-only path (__ldg, ld.global.nc) is for what nothing
+// writes while the kernel runs: the kernels of a launch sequence start while the ones before
+// still write the arena, so only uploaded records may be read through it.
 __device__ __forceinline__ Cx<double> ld(const Cx<double>* p) {
-  double2 v = __ldg(reinterpret_cast<const double2*>(p));
-  return {v.x, v.y};
-}
-template <>
-__device__ __forceinline__ Cx<float> ld(const Cx<float>* p) {
-  float2 v = __ldg(reinterpret_cast<const float2*>(p));
-  return {v.x, v.y};
-}
-template <>
-__device__ __forceinline__ Cx<ff> ld(const Cx<ff>* p) {
-  float4 v = __ldg(reinterpret_cast<const float4*>(p));
-  return {{v.x, v.y}, {v.z, v.w}};
-}
-// Coherent loads (plain ld.global): for data the same CTA wrote earlier, which the
-// read-only path of __ldg does not guarantee to see.
-__device__ __forceinline__ Cx<double> ldc(const Cx<double>* p) {
   double2 v = *reinterpret_cast<const double2*>(p);
   return {v.x, v.y};
 }
-__device__ __forceinline__ Cx<float> ldc(const Cx<float>* p) {
+__device__ __forceinline__ Cx<float> ld(const Cx<float>* p) {
   float2 v = *reinterpret_cast<const float2*>(p);
   return {v.x, v.y};
 }
-__device__ __forceinline__ Cx<ff> ldc(const Cx<ff>* p) {
+__device__ __forceinline__ Cx<ff> ld(const Cx<ff>* p) {
   float4 v = *reinterpret_cast<const float4*>(p);
   return {{v.x, v.y}, {v.z, v.w}};
 }
@@ -361,8 +345,7 @@ __device__ __forceinline__ S step_scale(const Step& s, Meta* meta, bool write_ex
 
 // Thread per (output row r, chunk of nc columns): the row's offsets are decoded once and
 // its K values A[r, :] loaded once (registers when K <= KREG), then each output C[n, r] of
-// the chunk is formed against B (read through the L1/texture path: it is small or shared
-// across the warp).  nc = N gives one thread per row; smaller chunks give steps with few
+// the chunk is formed against B (read through L1: it is small or shared across the warp).  nc = N gives one thread per row; smaller chunks give steps with few
 // rows enough threads to fill the GPU while the decoding stays amortised over nc outputs.
 // Consecutive threads take consecutive rows, so the C stores of a warp are contiguous.
 template <typename R, int KREG>

@@ -18,9 +18,9 @@ namespace pk {
 // multiply-adds: 63 cycles each).  A level launched alone takes 0.9 us more.
 
 // How a level's operands are read: written by other CTAs of the same launch (past L1), by
-// earlier launches only (read-only path), or by this CTA only (L1).  kWaveAny besides: steps of
-// any size, whose divisions may lack an exact multiplier (mul 0).
-enum WaveMode { kWaveL2 = 0, kWaveRO = 1, kWaveOwn = 2, kWaveAny = 4 };
+// earlier launches only (L1, once those have ended), or by this CTA only (L1).  kWaveAny besides:
+// steps of any size, whose divisions may lack an exact multiplier (mul 0).
+enum WaveMode { kWaveL2 = 0, kWaveEarlier = 1, kWaveOwn = 2, kWaveAny = 4 };
 
 // Offsets in A and B of index y of a run class (`r` the class's first run, n >= 1 of them);
 // y / size = umulhi(y, ceil(2^32 / size)), exact for the steps the planner gives a multiplier.
@@ -54,7 +54,7 @@ __device__ __forceinline__ Cx<ff> ldl2(const Cx<ff>* p) {
 
 template <int M, typename R>
 __device__ __forceinline__ Cx<R> wave_ld(const Cx<R>* p) {
-  return M & kWaveOwn ? ldc(p) : M & kWaveRO ? ld(p) : ldl2(p);
+  return M & (kWaveOwn | kWaveEarlier) ? ld(p) : ldl2(p);
 }
 
 // FP64 multiply-adds take 63 cycles each, so the four products of a term go to four sums.
@@ -166,7 +166,7 @@ __device__ __forceinline__ unsigned long long wave_outputs(const uint4* rec, uns
     ma = __ldcg((const ulonglong2*)(meta + sa));
     if (hasB) mb = __ldcg((const ulonglong2*)(meta + sb));
   };
-  if (M != kWaveRO) load_meta();
+  if (M != kWaveEarlier) load_meta();
   const unsigned q = chunk * 32 + lane, o = q >> lg;
   unsigned k0 = q & ((1u << lg) - 1), kd = 1u << lg;
   bool live = o < Rr * N;
@@ -185,7 +185,7 @@ __device__ __forceinline__ unsigned long long wave_outputs(const uint4* rec, uns
     }
     if (nrow) wave_offsets<M>(r, rr, nrow, oa, ob);
   }
-  if (M == kWaveRO) {
+  if (M == kWaveEarlier) {
     pdl_wait();
     load_meta();
   }
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(256)
     pdl_wait();
   } else {
     const uint2 it = __ldg((const uint2*)(blob + rg.item) + first + i);
-    v = wave_outputs<R, kWaveRO>((const uint4*)blob + it.x, it.y, arena, meta, slot);
+    v = wave_outputs<R, kWaveEarlier>((const uint4*)blob + it.x, it.y, arena, meta, slot);
   }
   if ((threadIdx.x & 31) == 0) {
     red[w] = v;
