@@ -58,8 +58,8 @@ typedef enum {
 
 typedef enum {
   PK_C128 = 0,       /* complex128 storage, FP64 arithmetic; large GEMM-shaped steps on the
-                        tensor cores in exact 62-bit fixed point per row and column, with
-                        errors below FP64's own                                           */
+                        tensor cores in 62-bit fixed point per row and column; outputs too
+                        small for that (q > 4 or general weights) again in FP64           */
   PK_C64 = 1,        /* complex64 storage, FP32 arithmetic; with pk_plan_opts.tail_steps
                         > 0 the final contractions run in complex128                      */
   PK_SPLIT = 2       /* split FP32: every real number is an unevaluated pair of floats

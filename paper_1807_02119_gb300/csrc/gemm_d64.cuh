@@ -8,10 +8,22 @@
 //     F = round(x 2^(62 - e)),  |F| <= 2^62,  F = sum_{i<8} d_i 256^(7-i),  -128 <= d_i < 128,
 // a digit per byte of F + 0x8080808080808080.  A digit is exact in BF16, digit products and
 // their FP32 sums over one flush group of K are exact integers (below 2^24), and the groups'
-// sums are added as 64-bit integers, so the only errors are the rounding of F (2^-63 of the
-// row's largest entry), the dropped levels i + j >= 8 (about 2^-62 of the row's and the
-// column's largest entries per term) and the final rounding to 53 bits: below FP64's own
-// rounding of every multiply-add (2^-53).  Rows or columns with an infinity or a NaN give NaN.
+// sums are added as 64-bit integers.  What is lost is the rounding of F (2^-63 of the row's
+// largest entry), the dropped levels i + j >= 8 (per term up to 2^-59 of the product of the
+// row's and the column's largest entries, 2^-62 as a rule) and the final rounding to 53 bits:
+// about sqrt(K) 2^-61 of that product P(m, n), whatever the output's own size.
+//
+// FP64's own rounding is a share of the terms, not of P.  With the standard weights and q <= 4
+// every clause matrix is the exponential of a quadratic form (over Z_2, Z_3 or Z_2^2), every
+// tensor a Gauss sum, and its nonzero entries have one magnitude: an output has a term as large
+// as P or none at all.  Elsewhere (q > 4, general weights) the entries of a row may lie any
+// number of powers of two apart.  There an output is kept if it is above 2^-kSure of P, or one of
+// its terms is above 2^-(kSure + 2) of P (marks, k_digits64): the loss is then about sqrt(K) 2^-53 of
+// that, as FP64's.  Any other is formed again in FP64 (small_outputs), and so is every output of a
+// row or column with an infinity or a NaN.  Counted on the CPU over the steps of nine knots at
+// q = 5 to 12: 0 to 4 % of a step's outputs are small as a rule (up to 87 %), and 0 to 0.3 % are
+// formed again (up to 14 %).  Cost on GB300, 167 crossings at q = 5: 871 -> 884 us per launch
+// sequence, 786 -> 849 us with the over / under bits that form most outputs again.
 //
 // The complex product is arranged as in gemm_tc.cuh: a complex row of A is one real row
 // [Re | Im], a complex column of B two real columns [Re; -Im] and [Im; Re].
@@ -50,6 +62,11 @@ constexpr int kFlush = ((1 << 10) - 1) / (kS * 2 * kKc);
 constexpr int kEpiWarps = 16, kThreads = 32 * (2 + kEpiWarps);
 constexpr int kConvThreads = 128;
 constexpr int kBad = 1 << 28;                // exponent of a row with a non-finite entry
+constexpr int kSure = 8;
+// An entry's marks: it reaches 2^-mark(j) of its row's largest entry (a column's: the marks in turn
+// from the last); a pair with a common mark has a product above 2^-(kSure + 2) of P.
+constexpr int kMarks = 3;
+__device__ __forceinline__ constexpr int mark(int j) { return kSure / (kMarks - 1) * j; }
 static_assert(kS * kN <= 256 && kSmem <= 220 * 1024 && kFlush * kS * 2 * kKc < 1024, "tile geometry");
 static_assert(kAChunk == kTc64AChunk && kBChunk == kTc64BChunk, "scratch layout");
 
@@ -99,7 +116,8 @@ __host__ __device__ inline int d64_groups(long long chunks, int parts) {
 
 template <bool IS_A>
 __device__ __forceinline__ void digits64_block(const Step& s, const Cx<double>* arena, unsigned char* scratch,
-                                               long long blk, unsigned* kt, unsigned* mx, long long* ro) {
+                                               const int* even, long long blk, unsigned* kt, unsigned* mx,
+                                               long long* ro) {
   using namespace d64;
   const Tc64Scratch L = tc64_scratch(s.Bsz, s.M, s.N, s.K);
   constexpr int kT = IS_A ? kMc : kNc, kParts = kT / 8;
@@ -110,6 +128,7 @@ __device__ __forceinline__ void digits64_block(const Step& s, const Cx<double>* 
   const long long ext = IS_A ? s.M : s.N;
   const long long r0 = tile * kT + part * RB;
   const int tid = threadIdx.x, K = (int)s.K;
+  const bool own = *even == 0;
   if (tid < RB) {
     mx[tid] = 0;
     long long a = 0, b = 0, c, ba, bo, bc, off = -1, cc = -1;
@@ -126,11 +145,14 @@ __device__ __forceinline__ void digits64_block(const Step& s, const Cx<double>* 
     // the row's (column's) C offset for the GEMM's epilogue; columns do not depend on bb
     if (IS_A || bb == 0)
       ((long long*)(scratch + (IS_A ? L.cr_off : L.cc_off)))[(IS_A ? bb * tiles + tile : tile) * kT + part * RB + tid] = cc;
+    if (own)
+      ((unsigned*)(scratch + (IS_A ? L.oa_off : L.ob_off)))[(bb * tiles + tile) * kT + part * RB + tid] = (unsigned)max(off, 0LL);
   }
   for (int k = tid; k < K; k += kConvThreads) {
     long long ka, kb;
     split_runs32((unsigned)k, s.kr, s.nk, ka, kb);
     kt[k] = (unsigned)(IS_A ? ka : kb);
+    if (own && IS_A && blk == 0) ((uint2*)(scratch + L.ok_off))[k] = make_uint2((unsigned)ka, (unsigned)kb);
   }
   __syncthreads();
   if (r0 >= ext) return;   // rows past the edge are multiplied but not stored
@@ -173,6 +195,19 @@ __device__ __forceinline__ void digits64_block(const Step& s, const Cx<double>* 
         im[u] = v.im;
       }
     }
+    if (own) {   // the 8 entries' marks, a byte for each threshold
+      unsigned m = 0, least[kMarks];   // high words; entries below the normal range have no mark
+#pragma unroll
+      for (int j = 0; j < kMarks; ++j) least[j] = (unsigned)max(1, min(2047, e + 1022 - mark(IS_A ? j : kMarks - 1 - j))) << 20;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const unsigned top = max((unsigned)__double2hiint(re[u]) & 0x7fffffffu, (unsigned)__double2hiint(im[u]) & 0x7fffffffu);
+#pragma unroll
+        for (int j = 0; j < kMarks; ++j)
+          if (top >= least[j]) m |= 1u << (8 * j + u);
+      }
+      ((unsigned*)(scratch + (IS_A ? L.xa_off : L.xb_off)))[((bb * tiles + tile) * L.chunks + c) * kT + part * RB + r] = m;
+    }
 #pragma unroll
     for (int part2 = 0; part2 < 2; ++part2) {   // the real, then the imaginary components
       unsigned long long f[8];
@@ -197,16 +232,16 @@ __device__ __forceinline__ void digits64_block(const Step& s, const Cx<double>* 
 }
 
 // Blocks [0, nA) convert A, the rest B.
-__global__ void __launch_bounds__(d64::kConvThreads) k_digits64(const Step s, const Cx<double>* arena,
-                                                                unsigned char* scratch, long long nA) {
+__global__ void __launch_bounds__(d64::kConvThreads, 8) k_digits64(const Step s, const Cx<double>* arena,
+                                                                unsigned char* scratch, const int* even, long long nA) {
   pdl_wait();
   __shared__ unsigned kt[kTc64MaxK], mx[kTcMc];
   __shared__ long long ro[kTcMc];
   const long long blk = blockIdx.x;
   if (blk < nA)
-    digits64_block<true>(s, arena, scratch, blk, kt, mx, ro);
+    digits64_block<true>(s, arena, scratch, even, blk, kt, mx, ro);
   else
-    digits64_block<false>(s, arena, scratch, blk - nA, kt, mx, ro);
+    digits64_block<false>(s, arena, scratch, even, blk - nA, kt, mx, ro);
 }
 
 namespace d64 {
@@ -239,10 +274,76 @@ __device__ __forceinline__ unsigned long long to_double_bits(long long h, long l
   if (ef >= 2046) return sign | 0x7ff0000000000000ull;
   return sign | (((unsigned long long)ef << 52) + u);
 }
+
+// A warp's small outputs again in FP64: bit j of `again`, column j of the warp's four in the lane's
+// row, to crow + cc[j].  Returns the lane's largest magnitude.  Out of line and not unrolled:
+// inlined, its instructions cost every launch of k_gemm64 2 us.
+__device__ __noinline__ unsigned long long small_outputs(const Step& s, Cx<double>* arena, const unsigned char* scratch,
+                                                         long long row, long long tn, long long crow, unsigned again, int e) {
+  const Tc64Scratch L = tc64_scratch(s.Bsz, s.M, s.N, s.K);
+  const int lane = threadIdx.x & 31, quarter = (threadIdx.x >> 5) & 3, cq = ((threadIdx.x >> 5) - 2) >> 2, K = (int)s.K;
+  const unsigned oa = ((const unsigned*)(scratch + L.oa_off))[row * kMc + quarter * 32 + lane];
+  const unsigned* ob = (const unsigned*)(scratch + L.ob_off) + (row / L.tiles_m * L.tiles_n + tn) * kNc + cq * 4;
+  const long long* cc = (const long long*)(scratch + L.cc_off) + tn * kNc + cq * 4;
+  const uint2* ok = (const uint2*)(scratch + L.ok_off);
+  const Cx<double>*A0 = arena + s.off_a, *B0 = arena + s.off_b;
+  Cx<double>* C = arena + s.off_c;
+  const double scale = ldexp(1.0, e);
+  unsigned long long vmax = 0;
+  auto put = [&](const Acc<double>& sum, long long at) {
+    const Cx<double> v = sum.get(scale);
+    vmax = max(vmax, mag_key(v));
+    st(C + at, v);
+  };
+  __syncwarp();   // the stores before the call come before those of other lanes here
+#pragma unroll 1
+  for (int j = 0; j < 4; ++j) {
+    const bool mine = again >> j & 1;
+    unsigned todo = __ballot_sync(0xffffffffu, mine);
+    if (!todo) continue;
+    const Cx<double>* B = B0 + ob[j];
+    const long long c = cc[j];
+    // FP64 instructions: a lane per output, or eight (and their sum) for four outputs at a time
+    if (4 * K + 6 < ((__popc(todo) + 3) >> 2) * (4 * ((K + 7) >> 3) + 10)) {
+      Acc64 acc;
+      if (mine) {
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) {
+          const uint2 o = ok[k];
+          acc.mac(ld(A0 + oa + o.x), ld(B + o.y));
+        }
+        put(acc.sum(), crow + c);
+      }
+      continue;
+    }
+#pragma unroll 1
+    while (todo) {
+      int src = -1;   // this group's lane: of the first four in turn
+#pragma unroll 1
+      for (int i = 0; i < 4 && todo; ++i, todo &= todo - 1)
+        if (i == lane >> 3) src = __ffs(todo) - 1;
+      const Cx<double>* A = A0 + __shfl_sync(0xffffffffu, oa, max(src, 0));
+      const long long at = __shfl_sync(0xffffffffu, crow, max(src, 0)) + c;
+      Acc64 acc;
+      if (src >= 0) {
+#pragma unroll 2
+        for (int k = lane & 7; k < K; k += 8) {
+          const uint2 o = ok[k];
+          acc.mac(ld(A + o.x), ld(B + o.y));
+        }
+      }
+      Acc<double> sum = acc.sum();
+      lanes_sum(sum, 3);
+      if (src >= 0 && (lane & 7) == 0) put(sum, at);
+    }
+  }
+  return vmax;
+}
 }  // namespace d64
 
-__global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const Step s, Cx<double>* arena, Meta* meta,
-                                                             const unsigned char* scratch,
+// even: a word of the uploaded program, nonzero where no output needs small_outputs.
+__global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const __grid_constant__ Step s, Cx<double>* arena, Meta* meta,
+                                                             const unsigned char* scratch, const int* even,
                                                              unsigned long long* err) {
   pdl_wait();
   using namespace d64;
@@ -343,6 +444,7 @@ __global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const Step s, Cx<do
     }
   } else {
     const int quarter = warp & 3, cq = (warp - 2) >> 2;   // lanes and 8 real columns of this warp
+    const bool check = *even == 0;
     int gg = 0;
     bool failed = false;
     for (int t = blockIdx.x; t < ntiles && !failed; t += gridDim.x) {
@@ -357,7 +459,7 @@ __global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const Step s, Cx<do
       for (int j = 0; j < 8; ++j) h[j] = l[j] = 0;
       for (int g = 0; g < ngroups; ++g, ++gg) {
         const int set = gg & 1;
-        if (!mbar_wait(smem_u32(&acc_full[set]), (uint32_t)((gg >> 1) & 1), err)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full[set]), (uint32_t)((gg >> 1) & 1), err))) {
           if (lane == 0) {
             bad = 1;
             atomicOr(err, 1ull);
@@ -396,19 +498,42 @@ __global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const Step s, Cx<do
       }
       // the tile, while the next one's products run
       Cx<double>* C = arena + s.off_c;
+      unsigned again = 0;   // outputs that are small against P
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const long long cc = any ? ccp[j] : -1;
         if (crow < 0 || cc < 0) continue;
         const int en = enp[j];
         unsigned long long re = 0x7ff8000000000000ull, im = re;   // NaN
+        bool sure = failed || !check;
         if (!failed && em < kBad && en < kBad) {
           const int x = em + en - 68 - ea - eb;
           re = to_double_bits(h[2 * j], l[2 * j], x);
           im = to_double_bits(h[2 * j + 1], l[2 * j + 1], x);
-          vmax = max(vmax, max(re & 0x7fffffffffffffffull, im & 0x7fffffffffffffffull));
+          const unsigned long long top = max(re & 0x7fffffffffffffffull, im & 0x7fffffffffffffffull);
+          const int et = (int)(top >> 52);   // 0: zero, or below the normal range
+          sure = sure || (et > 0 && et - 1023 >= x + 68 - kSure);
+          vmax = max(vmax, top);
         }
+        if (!sure) again |= 1u << j;
         st(C + crow + cc, Cx<double>{__longlong_as_double((long long)re), __longlong_as_double((long long)im)});
+      }
+      if (__any_sync(0xffffffffu, again)) {   // those with two entries that share a mark are kept
+        const unsigned* xa = (const unsigned*)(scratch + L.xa_off) + row * nchunks * kMc + quarter * 32 + lane;
+        const uint4* xb = (const uint4*)(scratch + L.xb_off) + (bb * L.tiles_n + tn) * nchunks * (kNc / 4) + cq;
+        uint4 hit = make_uint4(0, 0, 0, 0);
+#pragma unroll 4
+        for (int c = 0; c < nchunks; ++c) {
+          const unsigned a = xa[c * kMc];
+          const uint4 b = xb[c * (kNc / 4)];
+          hit.x |= a & b.x;
+          hit.y |= a & b.y;
+          hit.z |= a & b.z;
+          hit.w |= a & b.w;
+        }
+        again &= (hit.x == 0) | (hit.y == 0) << 1 | (hit.z == 0) << 2 | (hit.w == 0) << 3;
+        if (__any_sync(0xffffffffu, again))
+          vmax = max(vmax, small_outputs(s, arena, scratch, row, tn, crow, again, -(ea + eb)));
       }
     }
   }

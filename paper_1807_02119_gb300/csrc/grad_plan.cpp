@@ -335,7 +335,8 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
   G.off_recipe = off;
   off = a256(off + sizeof(Recipe) * G.recipes.size());
   G.off_slots = off;
-  off = a256(off + sizeof(Slot) * std::max<size_t>(1, p.slots.size()));
+  G.off_even = off + sizeof(Slot) * std::max<size_t>(1, p.slots.size());
+  off = a256(G.off_even + 4);
   G.off_leaves = off;
   off = a256(off + sizeof(GradLeaf) * nl);
   G.off_wave = off;

@@ -278,16 +278,16 @@ cudaError_t launch_short(const Step& s, Cx<ff>* arena, Meta* meta, unsigned long
 
 // complex128 on the tensor cores: the digits of both operands, then the GEMM.
 cudaError_t launch_tc64(const Step& s, Cx<double>* arena, Meta* meta, unsigned char* tcs,
-                        unsigned long long* err, cudaStream_t stream, Marker& mk, double cm, double by) {
+                        const int* even, unsigned long long* err, cudaStream_t stream, Marker& mk, double cm, double by) {
   const Tc64Scratch L = tc64_scratch(s.Bsz, s.M, s.N, s.K);
   const long long nA = s.Bsz * L.tiles_m * (kTcMc / 8 / d64_groups(L.chunks, kTcMc / 8)),
                   nB = s.Bsz * L.tiles_n * (kTc64Nc / 8 / d64_groups(L.chunks, kTc64Nc / 8));
   mk.begin(6, 0.0, 16.0 * (double)(s.R * s.K + s.Bsz * s.K * s.N), gpu_fill(nA + nB, 8));
-  launch_kernel(k_digits64, dim3((unsigned)(nA + nB)), d64::kConvThreads, 0, stream, mk.pdl(), 1, s, arena, tcs, nA);
+  launch_kernel(k_digits64, dim3((unsigned)(nA + nB)), d64::kConvThreads, 0, stream, mk.pdl(), 1, s, arena, tcs, even, nA);
   mk.end();
   const long long grid = std::min<long long>(L.tiles_m * L.tiles_n * s.Bsz, (long long)g_sms);
   mk.begin(5, cm, by, gpu_fill(grid, 1));
-  launch_kernel(k_gemm64, dim3((unsigned)grid), d64::kThreads, d64::kSmem, stream, mk.pdl(), 1, s, arena, meta, tcs, err);
+  launch_kernel(k_gemm64, dim3((unsigned)grid), d64::kThreads, d64::kSmem, stream, mk.pdl(), 1, s, arena, meta, tcs, even, err);
   mk.end();
   return cudaGetLastError();
 }
@@ -295,8 +295,8 @@ cudaError_t launch_tc64(const Step& s, Cx<double>* arena, Meta* meta, unsigned c
 template <typename R>
 cudaError_t launch_step(const Step& s, Cx<R>* arena, Meta* meta, Cx<double>* partial,
                         unsigned* counter, cudaStream_t stream, Marker& mk, double by,
-                        unsigned char* tc_scratch = nullptr, unsigned long long* err = nullptr,
-                        int64_t db_groups = 0) {
+                        unsigned char* tc_scratch = nullptr, const int* even = nullptr,
+                        unsigned long long* err = nullptr, int64_t db_groups = 0) {
   const double cm = (double)s.R * (double)s.K * (double)s.N;
   const long long gemm_tiles = ((s.M + 63) / 64) * ((s.N + 63) / 64) * s.Bsz;
   cudaError_t e;
@@ -311,7 +311,7 @@ cudaError_t launch_step(const Step& s, Cx<R>* arena, Meta* meta, Cx<double>* par
                  : launch_tc<5>(s, arena, meta, tc_scratch, counter, err, stream, mk, cm, by, db_groups);
   }
   if constexpr (std::is_same<R, double>::value) {
-    if (tc_scratch && err && tc64_step(s)) return launch_tc64(s, arena, meta, tc_scratch, err, stream, mk, cm, by);
+    if (tc_scratch && err && tc64_step(s)) return launch_tc64(s, arena, meta, tc_scratch, even, err, stream, mk, cm, by);
   }
   if (s.kernel == KGEMM && gemm_tiles < (1LL << 31)) {
     // fewer than two 64 x 64 tiles per multiprocessor: a quarter of the work per CTA (243 x 243 x
@@ -347,7 +347,7 @@ double step_bytes(const Plan& p, const Step& s, double elem_bytes) {
 template <typename R>
 cudaError_t launch_stage(const WaveProgram& w, const WaveStage& g, const std::vector<Step>& steps,
                          const unsigned char* blob, Cx<R>* arena, Meta* meta, Cx<double>* partial,
-                         unsigned* counters, unsigned char* tcs, unsigned long long* err, int64_t db_groups,
+                         unsigned* counters, unsigned char* tcs, const int* even, unsigned long long* err, int64_t db_groups,
                          cudaStream_t stream, Marker& mk, double cm, double by) {
   mk.step = g.step;
   if (g.kind == WaveStage::STEP) {
@@ -355,7 +355,7 @@ cudaError_t launch_stage(const WaveProgram& w, const WaveStage& g, const std::ve
     s.off_a = w.off[s.a];
     s.off_b = s.b >= 0 ? w.off[s.b] : 0;
     s.off_c = w.off[s.c];
-    return launch_step<R>(s, arena, meta, partial, counters + g.step, stream, mk, by, tcs, err, db_groups);
+    return launch_step<R>(s, arena, meta, partial, counters + g.step, stream, mk, by, tcs, even, err, db_groups);
   }
   if (g.kind == WaveStage::WIDE) {
     // few warps per CTA while that spreads the level over more multiprocessors
@@ -390,6 +390,7 @@ cudaError_t launch_bulk(const Plan& p, char* base, char* arena_base, int32_t fir
   // digit scratch of the tensor-core steps
   const bool digits = std::is_same<R, ff>::value ? p.tc_bytes > 0 : std::is_same<R, double>::value && p.tc64_bytes > 0;
   unsigned char* tcs = digits ? (unsigned char*)arena_base + p.tc_offset() : nullptr;
+  const int* even = (const int*)(base + p.off_even);
   unsigned long long* err = &((SliceResult*)(base + p.off_result))[p.n_slices].status;
   if (!o.check_finite) {
     const WaveProgram& w = p.wave[precision_of<R>()];
@@ -403,7 +404,7 @@ cudaError_t launch_bulk(const Plan& p, char* base, char* arena_base, int32_t fir
         by += step_bytes(p, p.steps[j], (double)sizeof(Cx<R>));
       }
       cudaError_t e = launch_stage<R>(w, g, p.steps, (const unsigned char*)base + p.off_wave, arena,
-                                      meta, partial, counters, tcs, err, p.tuning.tc_db_groups, stream, mk,
+                                      meta, partial, counters, tcs, even, err, p.tuning.tc_db_groups, stream, mk,
                                       cm, by);
       if (e != cudaSuccess) return e;
     }
@@ -412,7 +413,7 @@ cudaError_t launch_bulk(const Plan& p, char* base, char* arena_base, int32_t fir
   for (int32_t i = first; i < last; ++i) {
     mk.step = i;
     cudaError_t e = launch_step<R>(p.steps[i], arena, meta, partial, counters + i, stream, mk,
-                                   step_bytes(p, p.steps[i], (double)sizeof(Cx<R>)), tcs, err,
+                                   step_bytes(p, p.steps[i], (double)sizeof(Cx<R>)), tcs, even, err,
                                    p.tuning.tc_db_groups);
     if (e == cudaSuccess)
       e = check_tensor<R>(arena + p.steps[i].off_c, p.tensors[p.steps[i].c].elems, err,
@@ -577,7 +578,7 @@ cudaError_t launch_grad_impl(const Plan& p, char* base, cudaStream_t stream) {
     }
     for (const WaveStage& g : G.wave.stages[std::is_same<R, double>::value]) {
       e = launch_stage<R>(G.wave, g, G.steps, (const unsigned char*)base + G.off_wave, arena, meta, partial,
-                          counters, tcs, &res[p.n_slices].status, 0, stream, mk, 0.0, 0.0);
+                          counters, tcs, (const int*)(base + G.off_even), &res[p.n_slices].status, 0, stream, mk, 0.0, 0.0);
       if (e != cudaSuccess) return e;
     }
     launch_kernel(k_slice_result<R>, dim3(1), 32, 0, stream, mk.pdl(), 1, arena, G.root_offset, meta, G.root_meta, res, sl);

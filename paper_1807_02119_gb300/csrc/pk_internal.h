@@ -252,7 +252,7 @@ PK_HD constexpr int tc_flush(int S) { return ((1 << 10) - 1) / (S * 2 * kTcKc); 
 // the digit kernel for the GEMM's epilogue.
 struct TcScratch {
   long long tiles_m, tiles_n, chunks, groups;
-  long long a_off, b_off, ea_off, eb_off, cr_off, cc_off, bytes;
+  long long a_off, b_off, xa_off, xb_off, ea_off, eb_off, cr_off, cc_off, oa_off, ob_off, ok_off, bytes;
 };
 PK_HD inline TcScratch tc_scratch(long long Bsz, long long M, long long N, long long K, int S) {
   TcScratch x;
@@ -272,13 +272,15 @@ PK_HD inline TcScratch tc_scratch(long long Bsz, long long M, long long N, long 
 
 // GEMM steps of the complex128 precision on the tensor cores (gemm_d64.cuh): eight digits,
 // tiles of kTcMc x kTc64Nc complex, chunks of kTc64Kc complex k, one exponent per row and
-// column; the digits, exponents and C offsets lie after the arena as above.
+// column; the digits, exponents and C offsets lie after the arena as above, and what small outputs
+// need: marks of the larger entries (xa, xb: a word per chunk of a row or column) and the offsets
+// in A and B of rows, columns and the contracted index (oa, ob, ok).
 constexpr int kTc64Nc = 16, kTc64Kc = 8;
 constexpr long long kTc64AChunk = 8LL * kTcMc * (2 * kTc64Kc) * 2, kTc64BChunk = 8LL * (2 * kTc64Nc) * (2 * kTc64Kc) * 2;
 constexpr long long kTc64MaxK = 4096;   // offsets of the contracted index in shared memory
 struct Tc64Scratch {
   long long tiles_m, tiles_n, chunks;
-  long long a_off, b_off, ea_off, eb_off, cr_off, cc_off, bytes;
+  long long a_off, b_off, xa_off, xb_off, ea_off, eb_off, cr_off, cc_off, oa_off, ob_off, ok_off, bytes;
 };
 PK_HD inline Tc64Scratch tc64_scratch(long long Bsz, long long M, long long N, long long K) {
   Tc64Scratch x;
@@ -287,11 +289,16 @@ PK_HD inline Tc64Scratch tc64_scratch(long long Bsz, long long M, long long N, l
   x.chunks = (K + kTc64Kc - 1) / kTc64Kc;
   x.a_off = 0;
   x.b_off = x.a_off + Bsz * x.tiles_m * x.chunks * kTc64AChunk;
-  x.ea_off = x.b_off + Bsz * x.tiles_n * x.chunks * kTc64BChunk;
+  x.xa_off = x.b_off + Bsz * x.tiles_n * x.chunks * kTc64BChunk;
+  x.xb_off = x.xa_off + Bsz * x.tiles_m * x.chunks * (kTcMc * 4);
+  x.ea_off = (x.xb_off + Bsz * x.tiles_n * x.chunks * (kTc64Nc * 4) + 255) & ~255LL;
   x.eb_off = x.ea_off + ((Bsz * x.tiles_m * kTcMc * 4 + 255) & ~255LL);
   x.cr_off = x.eb_off + ((Bsz * x.tiles_n * kTc64Nc * 4 + 255) & ~255LL);
   x.cc_off = x.cr_off + ((Bsz * x.tiles_m * kTcMc * 8 + 255) & ~255LL);
-  x.bytes = x.cc_off + ((x.tiles_n * kTc64Nc * 8 + 255) & ~255LL);
+  x.oa_off = x.cc_off + ((x.tiles_n * kTc64Nc * 8 + 255) & ~255LL);
+  x.ob_off = x.oa_off + Bsz * x.tiles_m * (kTcMc * 4);
+  x.ok_off = x.ob_off + ((Bsz * x.tiles_n * (kTc64Nc * 4) + 255) & ~255LL);
+  x.bytes = x.ok_off + ((K * 8 + 255) & ~255LL);
   return x;
 }
 // Whether complex128 runs the step there: by the cycles it takes (152 multiprocessors).  Tensor
@@ -348,7 +355,7 @@ struct GradProgram {
   int64_t root_offset = 0;
   int32_t root_meta = 0;
   double cmacs[3] = {0, 0, 0};       // per slice, by phase
-  uint64_t off_recipe = 0, off_slots = 0, off_leaves = 0, off_wave = 0, off_meta = 0,
+  uint64_t off_recipe = 0, off_slots = 0, off_even = 0, off_leaves = 0, off_wave = 0, off_meta = 0,
            off_counter = 0, off_result = 0, off_scratch = 0, off_acc = 0, off_arena = 0;
   std::vector<uint8_t> program;      // recipes | slots | leaves | level records, copied by pk_grad
   uint64_t tc_offset() const { return ((uint64_t)arena_elems * 16ull + 255) & ~uint64_t(255); }
@@ -391,8 +398,8 @@ struct Plan {
   double est_cost = 0;   // the planner's estimated cost of the chosen sequence (all slices)
   int64_t arena_elems = 0;
   int64_t splitk_partials = 0;      // complex scratch entries for split-K steps
-  // device program layout (byte offsets inside the workspace)
-  uint64_t off_recipe = 0, off_slots = 0, off_meta = 0, off_result = 0, off_scratch = 0,
+  // device program layout (byte offsets inside the workspace); off_even: the word of put_even
+  uint64_t off_recipe = 0, off_slots = 0, off_even = 0, off_meta = 0, off_result = 0, off_scratch = 0,
            off_counter = 0, off_arena = 0;
   uint64_t ws_bytes(int32_t precision) const;
   // elements of the arena the workspace holds: the steps' own order (arena_elems) or a level
@@ -501,6 +508,8 @@ bool valid_tuning(const pk_tuning& t);
 bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& tune, std::string& err);
 // Writes the clause values of p.weights into p.slots and both program blobs.
 void apply_weights(Plan& p);
+// Writes into both whether a tensor's nonzero entries have one magnitude (gemm_d64.cuh).
+void put_even(Plan& p);
 // New per-edge weights (4 doubles per Tait edge; NULL: the standard weights of t(q)) for a
 // general plan; false if a weight is not finite.
 bool set_weights(Plan& p, const double* w);

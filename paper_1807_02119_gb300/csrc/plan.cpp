@@ -1699,7 +1699,8 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
   p.off_recipe = off;
   off = align256(off + sizeof(Recipe) * p.recipes.size());
   p.off_slots = off;
-  off = align256(off + sizeof(Slot) * std::max<size_t>(1, p.slots.size()));
+  p.off_even = off + sizeof(Slot) * std::max<size_t>(1, p.slots.size());
+  off = align256(p.off_even + 4);
   p.off_conv = off;
   off = align256(off + sizeof(ConvRec) * std::max<size_t>(1, p.conv.size()));
   p.off_wave = off;
@@ -1710,6 +1711,7 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
     std::memcpy(p.program.data() + p.off_slots, p.slots.data(), sizeof(Slot) * p.slots.size());
   if (!p.conv.empty())
     std::memcpy(p.program.data() + p.off_conv, p.conv.data(), sizeof(ConvRec) * p.conv.size());
+  put_even(p);
   plan_waves(p, false);
   // the level schedule's layout may not push a plan over the allocation-free entry point's
   // fixed workspace that its own order fits: such a plan keeps a second schedule for it
@@ -1755,7 +1757,14 @@ static int32_t max_exp4(double a, double b, double c, double d) {
   return e;
 }
 
+void put_even(Plan& p) {
+  const int32_t even = p.std_weights && p.q <= 4;
+  std::memcpy(p.program.data() + p.off_even, &even, 4);
+  if (p.grad.built) std::memcpy(p.grad.program.data() + p.grad.off_even, &even, 4);
+}
+
 void apply_weights(Plan& p) {
+  put_even(p);
   if (p.compact) {
     p.compact->weights = p.weights;
     p.compact->std_weights = p.std_weights;
