@@ -91,6 +91,7 @@ typedef enum {
  * the planner choose per step by its shape). */
 #define PK_FLAG_FORCE_GEMM 1 /* every two-operand step on the tiled GEMM kernel           */
 #define PK_FLAG_FORCE_ROWS 2 /* every step on the row kernel                               */
+                             /* (both: in PK_C128 on the FP64 units)                       */
 #define PK_FLAG_NO_TC 8      /* PK_SPLIT, PK_C128: run GEMM-shaped steps on the CUDA cores
                                 (float-float or FP64 SIMT kernels) instead of the tensor cores */
 #define PK_FLAG_TC_DIGITS4 16 /* PK_SPLIT tensor-core steps: four BF16 digits per operand

@@ -249,7 +249,7 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
     for (int32_t i = 0; i < no; ++i)
       if (ops[i].after >= 0) held.push_back({ops[i].after, i});
     for (int breadth = 1; breadth >= 0; --breadth) {
-      wave_schedule(st, ni, tune, p.use_tc ? kHeavyTc64 : 0, breadth != 0, &held, no, w.units);
+      wave_schedule(st, ni, tune, p.use_tc64 ? kHeavyTc64 : 0, breadth != 0, &held, no, w.units);
       w.arena_elems = wave_layout(st, elems, pinned, w.units, w.off);
       if (w.arena_elems <= limit) break;
       w.off.clear();
@@ -258,7 +258,7 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
       w.off = seq_off;
       w.arena_elems = top;
       wave_hazards(st, elems, w.off, edges);
-      wave_schedule(st, ni, tune, p.use_tc ? kHeavyTc64 : 0, false, &edges, no, w.units);
+      wave_schedule(st, ni, tune, p.use_tc64 ? kHeavyTc64 : 0, false, &edges, no, w.units);
     }
     // the operations in launch order, on the schedule's offsets; bookkeeping slots in a, b, c
     std::vector<Op> sorted;
@@ -281,7 +281,7 @@ bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& 
     wave_stages(by_meta, tune, kHeavyTc64, true, w);
     G.tc64_bytes = 0;
     for (const Step& x : by_meta)
-      if (p.use_tc && tc64_step(x))
+      if (p.use_tc64 && tc64_step(x))
         G.tc64_bytes = std::max<int64_t>(G.tc64_bytes, tc64_scratch(x.Bsz, x.M, x.N, x.K).bytes);
   }
 

@@ -430,7 +430,7 @@ struct Plan {
   int64_t tc_bytes = 0;              // split precision: digit scratch of the largest
                                      // tensor-core step (after the arena)
   int32_t n_tc = 0;                  // tensor-core steps per slice
-  bool use_tc = true;                // made without PK_FLAG_NO_TC
+  bool use_tc64 = true;              // complex128 GEMM steps on the tensor cores (gemm_d64.cuh)
   int64_t tc64_bytes = 0;            // complex128: digit scratch of the largest tensor-core step
                                      // (0: every step on the FP64 units)
   uint64_t off_conv = 0;             // byte offset of the ConvRec records (in the program)

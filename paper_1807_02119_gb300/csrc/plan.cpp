@@ -1377,7 +1377,7 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
     return false;
   }
   p.q = q;
-  p.use_tc = !(opts.flags & PK_FLAG_NO_TC);
+  p.use_tc64 = !(opts.flags & (PK_FLAG_NO_TC | PK_FLAG_FORCE_GEMM | PK_FLAG_FORCE_ROWS));
   p.knot = k;
   const double lq = std::log2((double)q);
   double max_log2 = opts.max_log2_elems > 0 ? opts.max_log2_elems : 31.0;

@@ -425,7 +425,7 @@ void plan_waves(Plan& p, bool compact) {
   pinned[p.final_tensor] = 1;
   p.tc64_bytes = 0;
   for (const Step& s : p.steps)
-    if (p.use_tc && !compact && tc64_step(s))
+    if (p.use_tc64 && !compact && tc64_step(s))
       p.tc64_bytes = std::max<int64_t>(p.tc64_bytes, tc64_scratch(s.Bsz, s.M, s.N, s.K).bytes);
   const int32_t tail = p.conv.empty() && p.tail.empty() ? ns : p.tail_first;
   int64_t limit = p.arena_elems;   // twice that up to 1 GiB, a quarter more up to 16 GiB
