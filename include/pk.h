@@ -307,7 +307,7 @@ pk_status pk_eval(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_work
 /* The three stages of pk_eval, asynchronous on the context's stream:
  * pk_upload copies the plan's initial-tensor recipe into the workspace (host->device);
  * pk_launch enqueues every kernel of every slice (the workspace must hold an uploaded
- * recipe of the same plan and precision); the first launch for a given workspace and
+ * recipe of the same plan, in any precision); the first launch for a given workspace and
  * precision records the sequence into a CUDA graph (on a private stream of the
  * context), later launches replay it, so a plan should keep using the same buffers;
  * pk_download waits for the stream, copies the scaled result back and applies A(q). */
@@ -315,8 +315,8 @@ pk_status pk_upload(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_wo
                     uint64_t workspace_bytes);
 /* As pk_upload, but only the knot-derived part of the program: the initial-tensor recipes
  * and their slots (the program's first bytes).  The plan's other records (conversion and
- * level records) stay as an earlier pk_upload of this plan and precision
- * left them in the same workspace, which the caller must have done (not checked).  For
+ * level records) stay as an earlier pk_upload of this plan left them
+ * in the same workspace, which the caller must have done (not checked).  For
  * repeated evaluations of the same plan.  *copied (may be NULL): the bytes copied. */
 pk_status pk_upload_inputs(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_workspace,
                            uint64_t workspace_bytes, uint64_t* copied);

@@ -71,27 +71,34 @@ pk_status check_ws(pk_ctx* ctx, const pk_plan* p, int32_t precision, void*& ws, 
   return check_ws_need(ctx, p->p.ws_bytes(precision), ws, bytes);
 }
 
-// What pk_upload copies for a level schedule (a precision or kWaveExact), in pinned memory (kept
-// with the plan): the program and the schedule's records behind it.  NULL when the allocation fails.
-const uint8_t* pinned_image(const pk_plan* p, int32_t sched, uint64_t& n) {
+// What pk_upload copies, in pinned memory (kept with the plan): the program and every level
+// schedule's records behind it.  NULL when the allocation fails.
+const uint8_t* pinned_image(const pk_plan* p) {
   const pk::Plan& P = p->p;
-  const std::vector<uint8_t>& blob = P.wave[sched].blob;
-  n = P.off_wave + blob.size();
-  uint8_t*& pin = const_cast<pk_plan*>(p)->pinned_program[sched];
+  uint8_t*& pin = const_cast<pk_plan*>(p)->pinned_program;
   if (!pin) {
-    if (cudaMallocHost((void**)&pin, n + 1) != cudaSuccess) return pin = nullptr;
-    std::memcpy(pin, P.program.data(), P.off_wave);
-    if (!blob.empty()) std::memcpy(pin + P.off_wave, blob.data(), blob.size());
+    if (cudaMallocHost((void**)&pin, P.off_records + 1) != cudaSuccess) return pin = nullptr;
+    std::memset(pin, 0, P.off_records);
+    std::memcpy(pin, P.program.data(), P.program.size());
+    for (int i = 0; i < 4; ++i)
+      if (!P.wave[i].blob.empty()) std::memcpy(pin + P.off_wave[i], P.wave[i].blob.data(), P.wave[i].blob.size());
   }
   return pin;
 }
 
-pk_status upload_image(pk_ctx* ctx, const pk_plan* p, int32_t sched, void* d_workspace) {
-  uint64_t n = 0;
-  const uint8_t* image = pinned_image(p, sched, n);
+pk_status upload_image(pk_ctx* ctx, const pk_plan* p, void* d_workspace, uint64_t n) {
+  const uint8_t* image = pinned_image(p);
   if (!image) return fail(ctx, PK_ENOMEM, "pinned host allocation failed");
-  cudaError_t e = cudaMemcpyAsync(d_workspace, image, n, cudaMemcpyHostToDevice, ctx->stream);
+  const cudaError_t e = cudaMemcpyAsync(d_workspace, image, n, cudaMemcpyHostToDevice, ctx->stream);
   return e == cudaSuccess ? PK_OK : cuda_fail(ctx, e, "upload");
+}
+
+// The workspace an upload goes to: at least the plan's state.
+pk_status check_state(pk_ctx* ctx, const pk_plan* p, int32_t precision, void*& d_workspace, uint64_t& workspace_bytes) {
+  if (d_workspace == nullptr) return check_ws(ctx, p, precision, d_workspace, workspace_bytes);
+  if (workspace_bytes < p->p.off_arena)
+    return fail(ctx, PK_ENOMEM, "buffer smaller than the plan state (pk_plan_state_bytes)");
+  return PK_OK;
 }
 
 // Enqueues the plan's kernels on the context's stream.  The launch sequence is recorded
@@ -555,8 +562,7 @@ pk_status pk_plan_launches(const pk_plan* p, int32_t precision, int64_t* launche
 
 void pk_plan_destroy(pk_plan* p) {
   if (!p) return;
-  for (uint8_t* pin : p->pinned_program)
-    if (pin) cudaFreeHost(pin);
+  if (p->pinned_program) cudaFreeHost(p->pinned_program);
   if (p->pinned_grad) cudaFreeHost(p->pinned_grad);
   if (p->graph.exec) cudaGraphExecDestroy(p->graph.exec);
   if (p->grad_graph.exec) cudaGraphExecDestroy(p->grad_graph.exec);
@@ -568,13 +574,9 @@ pk_status pk_upload(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_wo
   if (!ctx || !p || !valid_precision(precision)) return fail(ctx, PK_EINVAL, "bad argument");
   if (ctx->device < 0) return fail(ctx, PK_ENODEVICE, "host-only context");
   DeviceGuard g(ctx->device);
-  pk_status s = PK_OK;
-  if (d_workspace == nullptr)
-    s = check_ws(ctx, p, precision, d_workspace, workspace_bytes);
-  else if (workspace_bytes < p->p.off_arena)
-    s = fail(ctx, PK_ENOMEM, "buffer smaller than the plan state (pk_plan_state_bytes)");
+  const pk_status s = check_state(ctx, p, precision, d_workspace, workspace_bytes);
   if (s != PK_OK) return s;
-  return upload_image(ctx, p, precision, d_workspace);
+  return upload_image(ctx, p, d_workspace, p->p.off_records);
 }
 
 pk_status pk_upload_inputs(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_workspace,
@@ -582,23 +584,13 @@ pk_status pk_upload_inputs(pk_ctx* ctx, const pk_plan* p, int32_t precision, voi
   if (!ctx || !p || !valid_precision(precision)) return fail(ctx, PK_EINVAL, "bad argument");
   if (ctx->device < 0) return fail(ctx, PK_ENODEVICE, "host-only context");
   DeviceGuard g(ctx->device);
-  pk_status s = PK_OK;
-  if (d_workspace == nullptr)
-    s = check_ws(ctx, p, precision, d_workspace, workspace_bytes);
-  else if (workspace_bytes < p->p.off_arena)
-    s = fail(ctx, PK_ENOMEM, "buffer smaller than the plan state (pk_plan_state_bytes)");
+  const pk_status s = check_state(ctx, p, precision, d_workspace, workspace_bytes);
   if (s != PK_OK) return s;
   const pk::Plan& P = p->p;
   // recipes and slots lie first in the program, the conversion and level records after
   const uint64_t n = std::min<uint64_t>(P.off_conv, P.program.size());
   if (copied) *copied = n;
-  if (n == 0) return PK_OK;
-  uint64_t whole = 0;
-  const uint8_t* image = pinned_image(p, precision, whole);
-  if (!image) return fail(ctx, PK_ENOMEM, "pinned host allocation failed");
-  cudaError_t e = cudaMemcpyAsync(d_workspace, image, n, cudaMemcpyHostToDevice, ctx->stream);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "upload");
-  return PK_OK;
+  return n == 0 ? PK_OK : upload_image(ctx, p, d_workspace, n);
 }
 
 pk_status pk_launch(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_workspace,
@@ -782,7 +774,7 @@ pk_status pk_group_upload(pk_ctx* ctx, pk_group* grp, int32_t inputs_only, uint6
   uint64_t total = 0;
   for (int32_t i = 0; i < grp->n; ++i) {
     const pk::Plan& P = grp->plans[i]->p;
-    uint64_t n = P.off_wave + P.wave[grp->precision].blob.size();
+    uint64_t n = P.off_records;
     const pk_status s =
         inputs_only ? pk_upload_inputs(ctx, grp->plans[i], grp->precision, grp->ws[i], grp->ws_bytes[i], &n)
                     : pk_upload(ctx, grp->plans[i], grp->precision, grp->ws[i], grp->ws_bytes[i]);
@@ -1017,11 +1009,10 @@ pk_status pk_grad_weights(const pk_plan* p, const double* dlogZ_dT, double* out)
 pk_status pk_plan_set_weights(pk_plan* p, const double* edge_weights) {
   if (!p || !p->p.general) return PK_EINVAL;
   if (!pk::set_weights(p->p, edge_weights)) return PK_EINVAL;
-  for (uint8_t*& pin : p->pinned_program)   // refilled from the new program by the next pk_upload
-    if (pin) {
-      cudaFreeHost(pin);
-      pin = nullptr;
-    }
+  if (p->pinned_program) {   // refilled from the new program by the next upload
+    cudaFreeHost(p->pinned_program);
+    p->pinned_program = nullptr;
+  }
   return PK_OK;
 }
 
@@ -1217,7 +1208,7 @@ pk_status pk_eval_exact(pk_ctx* ctx, const pk_plan* p, const uint32_t* primes, i
   uint64_t bytes = workspace_bytes;
   pk_status s = check_ws(ctx, p, PK_C64, ws, bytes);
   if (s != PK_OK) return s;
-  if ((s = upload_image(ctx, p, pk::kWaveExact, ws)) != PK_OK) return s;
+  if ((s = upload_image(ctx, p, ws, p->p.off_records)) != PK_OK) return s;
   return exact_residues(ctx, p, primes, n_primes, ws, zab);
 }
 
@@ -1306,7 +1297,7 @@ pk_status pk_jones_coefficients(pk_ctx* ctx, const pk_knot* k, int32_t capacity,
     void* ws = nullptr;
     uint64_t bytes = 0;
     s = check_ws(ctx, p, PK_C64, ws, bytes);
-    if (s == PK_OK) s = upload_image(ctx, p, pk::kWaveExact, ws);
+    if (s == PK_OK) s = upload_image(ctx, p, ws, p->p.off_records);
     if (s == PK_OK) s = exact_residues(ctx, p, primes.data(), np, ws, zab.data() + 2 * (size_t)iq * np);
     pk_plan_destroy(p);
     if (s != PK_OK) return s;

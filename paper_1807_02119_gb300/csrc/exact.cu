@@ -259,7 +259,7 @@ cudaError_t launch_exact(const Plan& p, uint32_t prime, void* ws, void* arena, v
   E* ar = (E*)arena;
   E* sum = (E*)d_sum;
   const WaveProgram& w = p.wave[kWaveExact];
-  const unsigned char* blob = (const unsigned char*)base + p.off_wave;
+  const unsigned char* blob = (const unsigned char*)base + p.off_wave[kWaveExact];
   const Ring ring = make_ring(prime, p.q);
   cudaError_t e = cudaMemsetAsync(sum, 0, sizeof(E), stream);
   if (e != cudaSuccess) return e;

@@ -34,7 +34,7 @@ struct PlanGraph {
 };
 struct pk_plan {
   pk::Plan p;
-  uint8_t* pinned_program[4] = {};   // by level schedule (Plan::wave): what pk_upload copies
+  uint8_t* pinned_program = nullptr;   // what pk_upload copies
   uint8_t* pinned_grad = nullptr;  // the reverse-pass program and its downloaded results
   PlanGraph graph;
   PlanGraph grad_graph;            // the reverse-pass launch sequence (arena = null)

@@ -403,7 +403,7 @@ cudaError_t launch_bulk(const Plan& p, char* base, char* arena_base, int32_t fir
         cm += (double)p.steps[j].R * (double)p.steps[j].K * (double)p.steps[j].N;
         by += step_bytes(p, p.steps[j], (double)sizeof(Cx<R>));
       }
-      cudaError_t e = launch_stage<R>(w, g, p.steps, (const unsigned char*)base + p.off_wave, arena,
+      cudaError_t e = launch_stage<R>(w, g, p.steps, (const unsigned char*)base + p.off_wave[precision_of<R>()], arena,
                                       meta, partial, counters, tcs, even, err, p.tuning.tc_db_groups, stream, mk,
                                       cm, by);
       if (e != cudaSuccess) return e;
@@ -438,7 +438,7 @@ cudaError_t launch_build(const Plan& p, char* base, char* arena_base, long long 
   mk.begin(0, 0, (double)sizeof(Cx<R>) * (double)initel, gpu_fill((long long)bx * p.n_init, 8));
   launch_kernel(k_build<R>, dim3(bx, (unsigned)p.n_init), 256, 0, stream, false, 1, 
       (const Recipe*)(base + p.off_recipe), (const Slot*)(base + p.off_slots),
-      o.check_finite ? nullptr : (const int64_t*)(base + p.off_wave + p.wave[precision_of<R>()].init_off),
+      o.check_finite ? nullptr : (const int64_t*)(base + p.off_wave[precision_of<R>()] + p.wave[precision_of<R>()].init_off),
       (Cx<R>*)arena_base, (Meta*)(base + p.off_meta), p.q, sl, (int)p.sliced.size());
   mk.end();
   cudaError_t e = cudaGetLastError();

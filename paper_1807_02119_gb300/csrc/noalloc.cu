@@ -75,10 +75,10 @@ extern "C" pk_status pk_eval_noalloc(pk_ctx* ctx, const pk_plan* p, int32_t prec
   void* ws = nullptr;
   e = scratch_address(ctx->device, &ws);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(ws, P.program.data(), P.off_wave, cudaMemcpyHostToDevice, ctx->stream);
+    e = cudaMemcpyAsync(ws, P.program.data(), P.program.size(), cudaMemcpyHostToDevice, ctx->stream);
   const std::vector<uint8_t>& blob = P.wave[precision].blob;
   if (e == cudaSuccess && !blob.empty())
-    e = cudaMemcpyAsync((char*)ws + P.off_wave, blob.data(), blob.size(), cudaMemcpyHostToDevice, ctx->stream);
+    e = cudaMemcpyAsync((char*)ws + P.off_wave[precision], blob.data(), blob.size(), cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess)
     e = pk::launch_plan(P, precision, ws, (char*)ws + P.off_arena, ctx->stream);
   if (e == cudaSuccess)

@@ -419,8 +419,9 @@ struct Plan {
   std::vector<ConvRec> conv;
   std::shared_ptr<Plan> compact;     // the same plan on its own order's layout, where only that
                                      // fits pk_eval_noalloc's workspace
-  WaveProgram wave[4];               // level schedules by pk_precision, and kWaveExact (records at off_wave)
-  uint64_t off_wave = 0;
+  WaveProgram wave[4];               // level schedules by pk_precision, and kWaveExact
+  uint64_t off_wave[4] = {};         // their records, one after another behind the program
+  uint64_t off_records = 0;          // end of the last
   pk_tuning tuning{};                // launch shapes the plan was made with
   std::vector<TailStep> tail;        // one per step >= tail_first
   int64_t tail_elems = 0;            // complex128 elements of the tail region
@@ -502,8 +503,8 @@ bool wave_check(const std::vector<Step>& steps, const std::vector<int64_t>& elem
                 const std::vector<char>& pinned, const WaveProgram& w, std::string& err);
 // The plan's level schedules and the workspace layout that holds them; `compact`: on the
 // tensors' offsets of the steps' own order and without the complex128 digit scratch, so that
-// the workspace does not grow.
-void plan_waves(Plan& p, bool compact);
+// the workspace does not grow; `one`: room for one schedule's records at a time.
+void plan_waves(Plan& p, bool compact, bool one = false);
 bool valid_tuning(const pk_tuning& t);
 bool make_grad_program(Plan& p, int32_t stride, int32_t flags, const pk_tuning& tune, std::string& err);
 // Writes the clause values of p.weights into p.slots and both program blobs.

@@ -1703,8 +1703,8 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
   off = align256(p.off_even + 4);
   p.off_conv = off;
   off = align256(off + sizeof(ConvRec) * std::max<size_t>(1, p.conv.size()));
-  p.off_wave = off;
-  p.program.assign(p.off_wave, 0);
+  p.off_wave[0] = off;
+  p.program.assign(off, 0);
   if (!p.recipes.empty())
     std::memcpy(p.program.data() + p.off_recipe, p.recipes.data(), sizeof(Recipe) * p.recipes.size());
   if (!p.slots.empty())
@@ -1718,10 +1718,10 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
   for (int32_t prec : {PK_C128, PK_C64, PK_SPLIT})
     if (!p.compact && p.ws_bytes(prec) > kNoallocBytes) {
       const uint64_t grown = 16ull * (uint64_t)(p.ws_elems() - p.arena_elems) + 512 +
-                             (prec == PK_C128 ? (uint64_t)p.tc64_bytes : 0ull);
+                             (prec == PK_C128 ? (uint64_t)p.tc64_bytes : 0ull) + (p.off_records - p.off_wave[0]);
       if (p.ws_bytes(prec) <= kNoallocBytes + grown) {
         auto c = std::make_shared<Plan>(p);
-        plan_waves(*c, true);
+        plan_waves(*c, true, true);
         p.compact = c;
       }
     }

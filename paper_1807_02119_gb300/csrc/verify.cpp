@@ -225,8 +225,8 @@ bool check_forward(const Plan& p, int32_t precision, Checker& ck) {
   }
   // workspace layout: state records in order, the arena (and the split digit scratch or the
   // tail region) inside the workspace
-  if (!(p.off_recipe <= p.off_slots && p.off_slots <= p.off_conv && p.off_conv <= p.off_wave &&
-        p.off_wave + p.wave[precision].blob.size() <= p.off_meta && p.off_meta + 16ull * p.n_meta <= p.off_counter &&
+  if (!(p.off_recipe <= p.off_slots && p.off_slots <= p.off_conv && p.off_conv <= p.off_wave[0] &&
+        p.off_records <= p.off_meta && p.off_meta + 16ull * p.n_meta <= p.off_counter &&
         p.off_counter + 4ull * (uint64_t)ns <= p.off_result &&
         p.off_result + 32ull * (uint64_t)(p.n_slices + 1) <= p.off_scratch &&
         p.off_scratch + 16ull * (uint64_t)p.splitk_partials <= p.off_arena))

@@ -417,7 +417,7 @@ int32_t wave_batch(const Plan& p, bool shared, std::vector<uint8_t>& blob, WaveR
   return (int32_t)w.units.size();
 }
 
-void plan_waves(Plan& p, bool compact) {
+void plan_waves(Plan& p, bool compact, bool one) {
   const int32_t n = (int32_t)p.tensors.size(), ns = (int32_t)p.steps.size();
   std::vector<int64_t> elems(n);
   std::vector<char> pinned(n, 0);
@@ -433,7 +433,6 @@ void plan_waves(Plan& p, bool compact) {
     limit = 2 * limit + (1 << 12);
   else if (limit <= (1 << 30) / 5 * 4)
     limit += limit / 4;
-  uint64_t blob = 0;
   for (int32_t prec : {PK_C128, PK_C64, PK_SPLIT}) {
     WaveProgram& w = p.wave[prec];
     w = WaveProgram();
@@ -461,14 +460,20 @@ void plan_waves(Plan& p, bool compact) {
     if (prec == PK_C64) {
       p.wave[kWaveExact] = w;
       wave_stages(p.steps, p.tuning, heavy, true, p.wave[kWaveExact]);
-      blob = std::max<uint64_t>(blob, p.wave[kWaveExact].blob.size());
     }
     wave_stages(p.steps, p.tuning, heavy, prec != PK_C64, w);
-    blob = std::max<uint64_t>(blob, w.blob.size());
   }
-  // workspace: [recipes | slots | conv | the precision's level records] uploaded, then the
-  // device's own state
-  uint64_t off = align256(p.off_wave + blob);
+  // workspace: [recipes | slots | conv | every schedule's level records] uploaded, then the
+  // device's own state.  A launch in any precision after any upload finds its own records;
+  // schedules with equal ones (as a rule those of small plans) share them.
+  uint64_t off = p.off_wave[0];
+  for (int i = 0; i < 4; ++i) {
+    int same = 0;
+    while (same < i && p.wave[same].blob != p.wave[i].blob) ++same;
+    p.off_wave[i] = one ? p.off_wave[0] : same < i ? p.off_wave[same] : off;
+    off = align256(std::max<uint64_t>(off, p.off_wave[i] + p.wave[i].blob.size()));
+  }
+  p.off_records = off;
   p.off_meta = off;
   off = align256(off + 16ull * p.n_meta);
   p.off_counter = off;
