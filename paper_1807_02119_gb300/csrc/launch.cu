@@ -302,7 +302,7 @@ cudaError_t launch_step(const Step& s, Cx<R>* arena, Meta* meta, Cx<double>* par
   cudaError_t e;
   if constexpr (std::is_same<R, ff>::value) {
     // K <= 32: one kernel (a step of 7.8e4 multiply-adds 23 -> 8 us)
-    if (s.tc && tc_scratch && err && s.K <= tcs::kMaxK)
+    if (s.tc && err && s.K <= tcs::kMaxK)
       return s.tc == 4 ? launch_short<4>(s, arena, meta, err, stream, mk, cm, by)
                        : launch_short<5>(s, arena, meta, err, stream, mk, cm, by);
     if (s.tc && tc_scratch && err)  // digits of A and B, then the tensor-core GEMM

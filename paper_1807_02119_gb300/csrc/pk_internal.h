@@ -428,7 +428,7 @@ struct Plan {
   int64_t final_tail_off = 0;        // final tensor's offset in the tail region
   int32_t n_meta = 0;                // tensors + converted copies
   uint64_t off_tail = 0;             // byte offset of the tail region (split only)
-  int64_t tc_bytes = 0;              // split precision: digit scratch of the largest
+  int64_t tc_bytes = 0;              // split precision: digit scratch of the largest long
                                      // tensor-core step (after the arena)
   int32_t n_tc = 0;                  // tensor-core steps per slice
   bool use_tc64 = true;              // complex128 GEMM steps on the tensor cores (gemm_d64.cuh)

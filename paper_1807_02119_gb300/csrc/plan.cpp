@@ -1547,7 +1547,8 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
   for (const Step& st : p.steps)
     if (st.tc) {
       p.n_tc++;
-      p.tc_bytes = std::max<int64_t>(p.tc_bytes, tc_scratch(st.Bsz, st.M, st.N, st.K, st.tc).bytes);
+      if (st.K > kTcShortK)   // shorter ones take no digit scratch (gemm_short.cuh)
+        p.tc_bytes = std::max<int64_t>(p.tc_bytes, tc_scratch(st.Bsz, st.M, st.N, st.K, st.tc).bytes);
     }
 
   // ---- sizes, lifetimes, stats

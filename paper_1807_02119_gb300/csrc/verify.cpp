@@ -187,7 +187,7 @@ bool check_forward(const Plan& p, int32_t precision, Checker& ck) {
     if (!check_step(s, p.tensors[s.a].elems, s.b >= 0 ? p.tensors[s.b].elems : 0,
                     p.tensors[s.c].elems, w, ck))
       return false;
-    if (precision == PK_SPLIT && s.tc) {
+    if (precision == PK_SPLIT && s.tc && s.K > kTcShortK) {
       const TcScratch x = tc_scratch(s.Bsz, s.M, s.N, s.K, s.tc);
       if (x.bytes > p.tc_bytes) return ck.fail(w, "digit scratch larger than the plan reserves");
     }
