@@ -78,7 +78,6 @@ const uint8_t* pinned_image(const pk_plan* p) {
   uint8_t*& pin = const_cast<pk_plan*>(p)->pinned_program;
   if (!pin) {
     if (cudaMallocHost((void**)&pin, P.off_records + 1) != cudaSuccess) return pin = nullptr;
-    std::memset(pin, 0, P.off_records);
     std::memcpy(pin, P.program.data(), P.program.size());
     for (int i = 0; i < 4; ++i)
       if (!P.wave[i].blob.empty()) std::memcpy(pin + P.off_wave[i], P.wave[i].blob.data(), P.wave[i].blob.size());
