@@ -586,10 +586,10 @@ pk_status pk_upload_inputs(pk_ctx* ctx, const pk_plan* p, int32_t precision, voi
   const pk_status s = check_state(ctx, p, precision, d_workspace, workspace_bytes);
   if (s != PK_OK) return s;
   const pk::Plan& P = p->p;
-  // recipes and slots lie first in the program, the conversion and level records after
-  const uint64_t n = std::min<uint64_t>(P.off_conv, P.program.size());
+  // what depends on the knot and its weights lies first, the level records after
+  const uint64_t n = P.off_even + 4;
   if (copied) *copied = n;
-  return n == 0 ? PK_OK : upload_image(ctx, p, d_workspace, n);
+  return upload_image(ctx, p, d_workspace, n);
 }
 
 pk_status pk_launch(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_workspace,

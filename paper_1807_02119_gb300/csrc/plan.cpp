@@ -1700,10 +1700,11 @@ bool make_plan(const Knot& k, int32_t q, const pk_plan_opts& opts, const pk_tuni
   p.off_recipe = off;
   off = align256(off + sizeof(Recipe) * p.recipes.size());
   p.off_slots = off;
-  p.off_even = off + sizeof(Slot) * std::max<size_t>(1, p.slots.size());
-  off = align256(p.off_even + 4);
+  off = align256(off + sizeof(Slot) * std::max<size_t>(1, p.slots.size()));
   p.off_conv = off;
   off = align256(off + sizeof(ConvRec) * std::max<size_t>(1, p.conv.size()));
+  p.off_even = off;   // behind the offsets that a stored evaluation's fingerprint holds
+  off = align256(off + 4);
   p.off_wave[0] = off;
   p.program.assign(off, 0);
   if (!p.recipes.empty())

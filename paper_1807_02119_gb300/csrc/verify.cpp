@@ -225,7 +225,7 @@ bool check_forward(const Plan& p, int32_t precision, Checker& ck) {
   }
   // workspace layout: state records in order, the arena (and the split digit scratch or the
   // tail region) inside the workspace
-  if (!(p.off_recipe <= p.off_slots && p.off_slots <= p.off_conv && p.off_conv <= p.off_wave[0] &&
+  if (!(p.off_recipe <= p.off_slots && p.off_slots <= p.off_conv && p.off_conv <= p.off_even && p.off_even + 4 <= p.off_wave[0] &&
         p.off_records <= p.off_meta && p.off_meta + 16ull * p.n_meta <= p.off_counter &&
         p.off_counter + 4ull * (uint64_t)ns <= p.off_result &&
         p.off_result + 32ull * (uint64_t)(p.n_slices + 1) <= p.off_scratch &&

@@ -1,7 +1,5 @@
 """With the standard weights and q <= 4 the nonzero entries of every tensor have one magnitude
 (Gauss sums): the ground on which complex128's fixed point needs no second look there."""
-import ctypes as C
-
 import numpy as np
 import pytest
 
@@ -10,8 +8,7 @@ import plan_replay as pr
 
 
 def word(p):
-    sc = np.frombuffer(p.debug_blob(3), dtype=np.int64)
-    return int(np.frombuffer(p.debug_blob(0), dtype=np.int32)[(int(sc[7]) + max(1, int(sc[8])) * C.sizeof(pr.Slot)) // 4])
+    return int(np.frombuffer(p.debug_blob(0), dtype=np.int32)[-64])   # first of the program's last 256 bytes
 
 
 @pytest.mark.parametrize("q", [1, 2, 3, 4])
@@ -43,3 +40,18 @@ def test_word_follows_weights():
     assert word(p) == 0
     p.set_weights(None)
     assert word(p) == 1
+
+
+def test_stored_evaluations_keep_their_fingerprint():
+    """The word lies behind the offsets that plan_fingerprint covers: widening records follow
+    the slots (48 bytes each), rounded up to 256, also where these fill their last 256 bytes."""
+    ctx = pk.Context(-1)
+    full = 0
+    for L in (10, 12, 14, 16, 18, 20):
+        for seed in range(1, 9):
+            p = pk.Plan(ctx, pk.Knot.from_grid_walk(ctx, L, seed, True, 3, 150), 3)
+            sc = [int(v) for v in np.frombuffer(p.debug_blob(3), dtype=np.int64)]
+            end = sc[7] + 48 * max(1, sc[8])
+            full += end % 256 == 0
+            assert sc[13] == (end + 255) // 256 * 256
+    assert full
