@@ -3,8 +3,8 @@ against its row's and column's largest entries keeps its digits on the tensor-co
 
 All weights are positive, so no sum cancels and the relative errors of all steps add up: FP64's
 are at most (K + 8) 2^-53 per step.  The tensor cores keep outputs above 2^-8 of the product of
-the maxima, whose dropped digits are at most K 7 2^14 2^48 / 2^124 = K 2^-59.2 of it, hence
-4 K 2^-53 of the output."""
+the maxima, or with a term above 2^-10 of it; their dropped digits are at most K 7 2^14 2^48 / 2^124
+= K 2^-59.2 of it, hence 14 K 2^-53 of the output."""
 import math
 
 import numpy as np
@@ -35,7 +35,7 @@ def graded(n, J, seed):
 
 
 def bound(ks):
-    return sum(5 * k + 16 for k in ks) * 2.0 ** -53
+    return sum(15 * k + 16 for k in ks) * 2.0 ** -53
 
 
 def conversions(p):
