@@ -22,8 +22,8 @@
 // that, as FP64's.  Any other is formed again in FP64 (small_outputs), and so is every output of a
 // row or column with an infinity or a NaN.  Counted on the CPU over the steps of nine knots at
 // q = 5 to 12: 0 to 4 % of a step's outputs are small as a rule (up to 87 %), and 0 to 0.3 % are
-// formed again (up to 14 %).  Cost on GB300, 167 crossings at q = 5: 871 -> 884 us per launch
-// sequence, 786 -> 849 us with the over / under bits that form most outputs again.
+// formed again (up to 14 %).  Cost on GB300, 167 crossings at q = 5: 872 -> 886 us per launch
+// sequence, 788 -> 806 to 822 us with over / under bits that form outputs again.
 //
 // The complex product is arranged as in gemm_tc.cuh: a complex row of A is one real row
 // [Re | Im], a complex column of B two real columns [Re; -Im] and [Im; Re].
@@ -41,9 +41,9 @@
 //    copy writes of shared memory, 850 cycles at 128 B per cycle, against 576 of the tensor
 //    pipe: 47 complex TFLOP/s at most.
 //
-// Measured on GB300, per call: 167 crossings at q = 5 6070 -> 807 us, 205 crossings at q = 3
-// 1250 -> 214 us, the reverse pass of 300 crossings 3860 -> 2147 us; the step of 2.4e8
-// multiply-adds 2090 -> 94 us and 35 us of conversion.  Error of Z against exact integers,
+// Measured on GB300, per call, this path alone: 167 crossings at q = 5 6070 -> 807 us (without the
+// small outputs), 205 crossings at q = 3 1250 -> 214 us, the reverse pass of 300 crossings 3860 ->
+// 2147 us; the step of 2.4e8 multiply-adds 2090 -> 94 us and 35 us of conversion.  Error of Z against exact integers,
 // 36 knots at q = 3, 4, 5: rms 2.5e-15 -> 1.6e-15, largest 1.2e-14 -> 3.7e-15.
 #pragma once
 
@@ -63,6 +63,7 @@ constexpr int kEpiWarps = 16, kThreads = 32 * (2 + kEpiWarps);
 constexpr int kConvThreads = 128;
 constexpr int kBad = 1 << 28;                // exponent of a row with a non-finite entry
 constexpr int kSure = 8;
+constexpr int kListed = 2048, kListWarp = 24;   // small outputs a CTA leaves to its end, at most; of a warp's 128
 // An entry's marks: it reaches 2^-mark(j) of its row's largest entry (a column's: the marks in turn
 // from the last); a pair with a common mark has a product above 2^-(kSure + 2) of P.
 constexpr int kMarks = 3;
@@ -275,9 +276,51 @@ __device__ __forceinline__ unsigned long long to_double_bits(long long h, long l
   return sign | (((unsigned long long)ef << 52) + u);
 }
 
-// A warp's small outputs again in FP64: bit j of `again`, column j of the warp's four in the lane's
-// row, to crow + cc[j].  Returns the lane's largest magnitude.  Out of line and not unrolled:
-// inlined, its instructions cost every launch of k_gemm64 2 us.
+// A sum over k by eight lanes.
+__device__ __forceinline__ Acc<double> eighth_sum(const Cx<double>* A, const Cx<double>* B, const uint2* ok, int K) {
+  Acc64 acc;
+#pragma unroll 2
+  for (int k = threadIdx.x & 7; k < K; k += 8) {
+    const uint2 o = ok[k];
+    acc.mac(ld(A + o.x), ld(B + o.y));
+  }
+  Acc<double> sum = acc.sum();
+  lanes_sum(sum, 3);
+  return sum;
+}
+
+// The listed small outputs (tile, row << 4 | column in it) in FP64, by the epilogue warps: four at a
+// time, eight lanes each.  Returns the lane's largest magnitude.  This and the next one are out of
+// line and not unrolled: inlined, their instructions cost every launch of k_gemm64 2 us.
+__device__ __noinline__ unsigned long long listed_outputs(const Step& s, Cx<double>* arena, const unsigned char* scratch,
+                                                          const uint2* list, int n, int e) {
+  const Tc64Scratch L = tc64_scratch(s.Bsz, s.M, s.N, s.K);
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) - 2;
+  const double scale = ldexp(1.0, e);
+  unsigned long long vmax = 0;
+#pragma unroll 1
+  for (int i0 = 4 * warp; i0 < n; i0 += 4 * kEpiWarps) {
+    const int i = i0 + (lane >> 3);
+    const uint2 at = list[min(i, n - 1)];
+    const bool has = i < n && at.x != ~0u;
+    const unsigned t = has ? at.x : 0, tiles_n = (unsigned)L.tiles_n, row = t / tiles_n, tn = t - row * tiles_n;
+    const unsigned r = row * kMc + (at.y >> 4), c = tn * kNc + (at.y & 15);
+    const unsigned oa = ((const unsigned*)(scratch + L.oa_off))[r];
+    const unsigned ob = ((const unsigned*)(scratch + L.ob_off))[row / (unsigned)L.tiles_m * tiles_n * kNc + c];
+    const long long out = ((const long long*)(scratch + L.cr_off))[r] + ((const long long*)(scratch + L.cc_off))[c];
+    const Acc<double> sum = eighth_sum(arena + s.off_a + oa, arena + s.off_b + ob, (const uint2*)(scratch + L.ok_off),
+                                       has ? (int)s.K : 0);
+    if (has && (lane & 7) == 0) {
+      const Cx<double> v = sum.get(scale);
+      vmax = max(vmax, mag_key(v));
+      st(arena + s.off_c + out, v);
+    }
+  }
+  return vmax;
+}
+
+// A warp's small outputs in FP64 at once: bit j of `again`, column j of the warp's four in the lane's
+// row, to crow + cc[j].  Returns the lane's largest magnitude.
 __device__ __noinline__ unsigned long long small_outputs(const Step& s, Cx<double>* arena, const unsigned char* scratch,
                                                          long long row, long long tn, long long crow, unsigned again, int e) {
   const Tc64Scratch L = tc64_scratch(s.Bsz, s.M, s.N, s.K);
@@ -324,16 +367,7 @@ __device__ __noinline__ unsigned long long small_outputs(const Step& s, Cx<doubl
         if (i == lane >> 3) src = __ffs(todo) - 1;
       const Cx<double>* A = A0 + __shfl_sync(0xffffffffu, oa, max(src, 0));
       const long long at = __shfl_sync(0xffffffffu, crow, max(src, 0)) + c;
-      Acc64 acc;
-      if (src >= 0) {
-#pragma unroll 2
-        for (int k = lane & 7; k < K; k += 8) {
-          const uint2 o = ok[k];
-          acc.mac(ld(A + o.x), ld(B + o.y));
-        }
-      }
-      Acc<double> sum = acc.sum();
-      lanes_sum(sum, 3);
+      const Acc<double> sum = eighth_sum(A, B, ok, src < 0 ? 0 : K);
       if (src >= 0 && (lane & 7) == 0) put(sum, at);
     }
   }
@@ -358,12 +392,13 @@ __global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const __grid_consta
   __shared__ __align__(8) unsigned long long full[kStages], empty[kStages], acc_full[2], acc_empty[2], drain;
   __shared__ unsigned long long red[kEpiWarps + 2];
   __shared__ uint32_t tmem_slot;
-  __shared__ int bad;
+  __shared__ int bad, listed;
+  __shared__ uint2 list[kListed];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Tc64Scratch L = tc64_scratch(s.Bsz, s.M, s.N, s.K);
   const int ntiles = (int)(L.tiles_m * L.tiles_n * s.Bsz);
   if (tid == 0) {
-    bad = 0;
+    bad = listed = 0;
     for (int i = 0; i < kStages; ++i) {
       mbar_init(smem_u32(&full[i]), 1);
       mbar_init(smem_u32(&empty[i]), 1);
@@ -532,9 +567,32 @@ __global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const __grid_consta
           hit.w |= a & b.w;
         }
         again &= (hit.x == 0) | (hit.y == 0) << 1 | (hit.z == 0) << 2 | (hit.w == 0) << 3;
-        if (__any_sync(0xffffffffu, again))
-          vmax = max(vmax, small_outputs(s, arena, scratch, row, tn, crow, again, -(ea + eb)));
+        const int most = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(again));
+        if (most > 0) {
+          // few: left to the end of the CTA's tiles, where their chains of loads run side by side
+          // (167 crossings at q = 5 with 0.2 % of one K = 5 step's outputs: 849 -> 822 us)
+          int at = kListed;
+          if (most <= kListWarp) {
+            if (lane == 0) at = atomicAdd(&listed, most);
+            at = __shfl_sync(0xffffffffu, at, 0);
+          }
+          const bool fits = at + most <= kListed;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const unsigned who = __ballot_sync(0xffffffffu, again >> j & 1);
+            const int i = at + __popc(who & ((1u << lane) - 1));
+            if ((again >> j & 1) && i < kListed)   // where they no longer fit: empty entries
+              list[i] = make_uint2(fits ? (unsigned)t : ~0u, (unsigned)((quarter * 32 + lane) << 4 | (cq * 4 + j)));
+            at += __popc(who);
+          }
+          if (!fits) vmax = max(vmax, small_outputs(s, arena, scratch, row, tn, crow, again, -(ea + eb)));
+        }
       }
+    }
+    if (check) {
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+      const int n = min(listed, kListed);
+      if (n > 0 && !failed) vmax = max(vmax, listed_outputs(s, arena, scratch, list, n, -(ea + eb)));
     }
   }
   {  // max-abs of the CTA's outputs
