@@ -277,15 +277,11 @@ CLASS_KERNEL = {"build": "k_build", "rows": "k_rows / k_outs / k_waves / k_wave_
                 "gemm": "k_gemm (tiled strided complex GEMM, CUDA cores)",
                 "gemm_tc": "k_gemm_tc, k_gemm_short (complex GEMM on tcgen05 tensor cores, BF16 digit products)",
                 "digits": "k_digits (operand digits for k_gemm_tc)"}
-# DRAM traffic (ncu dram__bytes_read.sum + dram__bytes_write.sum) of one captured launch
-# divided by that launch's algorithmic bytes as the library counts them (its storage type,
-# 16 bytes per complex entry in split): the multiple applied to a class's average launch.
-# Sources (the heaviest launch of each class in the workload, knot seed 11 at q = 5):
-# tensor-core GEMM profiles/k_gemm_tc_split_q5_seed11.md (2.008 GB against (9.77 M + 9.77 M
-# + 48.8 M) x 16 B), digits profiles/k_digits_split_q5_seed11.md (2.599 GB against the
-# operands it reads, (48.8 M + 9.77 M) x 16 B).  The row kernels (2% of the step) have no
-# capture of a launch large enough to leave its output in DRAM.
-NCU_TRAFFIC_RATIO = {"gemm_tc": 2.008012 / 1.09375, "digits": 2.599281 / 0.9375}
+# DRAM traffic (ncu dram__bytes_read.sum + dram__bytes_write.sum) of all of a class's launches
+# in one replay of the step, divided by their algorithmic bytes as the library counts them (its
+# storage type, 16 bytes per complex entry in split): the multiple applied to a class's average
+# launch.  Source: profiles/launches_scale192_split.md (GB).  The other classes are 4% of the step.
+NCU_TRAFFIC_RATIO = {"gemm_tc": 28.76 / 25.83, "digits": 22.97 / 10.32}
 
 
 def roofline_blocks(classes, prec, pk_, instep=None):
