@@ -206,7 +206,11 @@ pk_status pk_tuning_default(pk_tuning* out);
 pk_status pk_ctx_create(int32_t device, void* stream, pk_ctx** out);
 pk_status pk_ctx_set_stream(pk_ctx* ctx, void* stream);
 /* Device-memory budget for the plans created afterwards (0: none, the default): a plan
- * whose workspace at any precision (pk_plan_workspace_bytes) would exceed `bytes` is sliced
+ * whose workspace at any precision (pk_plan_workspace_bytes) would exceed `bytes` first gives
+ * up what only buys time, in all precisions: its level schedules keep to the memory of the
+ * steps' own order (without a budget they may take twice that up to 1 GiB, a quarter more up to
+ * 16 GiB), and complex128 runs without the digit scratch of the tensor cores (without a budget
+ * up to 8 GiB), so on the FP64 units.  Where that is not enough the plan is sliced
  * further -- one index fewer on its largest tensor at a time, more slices of less memory
  * (Sec. III.B names memory as the bottleneck) -- until it fits; PK_ETOOWIDE from
  * pk_plan_create when the slice limit (pk_plan_opts.max_log2_slices) is reached first. */
@@ -313,9 +317,9 @@ pk_status pk_eval(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_work
  * pk_download waits for the stream, copies the scaled result back and applies A(q). */
 pk_status pk_upload(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_workspace,
                     uint64_t workspace_bytes);
-/* As pk_upload, but only the knot-derived part of the program: the initial-tensor recipes
- * and their slots (the program's first bytes).  The plan's other records (conversion and
- * level records) stay as an earlier pk_upload of this plan left them
+/* As pk_upload, but only the knot-derived part of the program: the initial-tensor recipes,
+ * their slots and the short records behind them (the program's first bytes).  The plan's
+ * level records stay as an earlier pk_upload of this plan left them
  * in the same workspace, which the caller must have done (not checked).  For
  * repeated evaluations of the same plan.  *copied (may be NULL): the bytes copied. */
 pk_status pk_upload_inputs(pk_ctx* ctx, const pk_plan* p, int32_t precision, void* d_workspace,

@@ -17,7 +17,7 @@
 // summed.  What bounded it were 64-bit divisions, four per term, and a thread per output however
 // long the sum: products now add up below p 2^31 with one conditional subtraction each and are
 // reduced once per output, and a warp or a CTA shares a long sum.  Measured on GB300, 36 crossings
-// at q = 10 modulo four primes: 6870 -> 364 us per call.
+// at q = 10 modulo four primes (perf/cases.py): 4589 -> 340 us per call.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -316,7 +316,8 @@ cudaError_t launch_step(const Step& s, Cx<R>* arena, Meta* meta, Cx<double>* par
   if (s.kernel == KGEMM && gemm_tiles < (1LL << 31)) {
     // fewer than two 64 x 64 tiles per multiprocessor: a quarter of the work per CTA (243 x 243 x
     // 243 with a batch of 3 in complex64, 48 tiles: 74 -> 31 us).  Drawing the line at four or eight
-    // takes 330 crossings at q = 3 in complex64 from 238 to 239 or 230 us on one knot, but from 362 to
+    // takes 330 crossings at q = 3 in complex64 (device time, three choices of the over / under bits)
+    // from 238 to 239 or 230 us on one knot, but from 362 to
     // 388 or 378 and from 276 to 289 on others: the smaller tiles read shared memory twice as often
     const bool small = gemm_tiles < 2LL * g_sms;
     const long long grid = small ? ((s.M + 31) / 32) * ((s.N + 31) / 32) * s.Bsz : gemm_tiles;

@@ -220,7 +220,6 @@ struct WaveProgram {
 constexpr int kWaveCtaWarps = 16;          // warps per CTA of the level kernel at most
 constexpr int kWaveMaxCtas = 8;            // CTAs of its cluster at most
 constexpr int kWaveCtaWarps32 = 16, kWaveCtaWarps64 = 8;   // warps of work per CTA it aims at
-constexpr int kWavePasses = 1;             // passes over a level at most; wider levels fill the GPU
 constexpr int kWaveK = 5;                  // terms whose operands a lane loads together
 constexpr int64_t kWaveOuts = 1LL << 18;   // outputs of a step inside a level at most
 constexpr int32_t kWaveExact = 3;          // Plan::wave of the exact residues (after the precisions')

@@ -1,15 +1,15 @@
 // Executor launch shapes, written by paper_1807_02119_gb300/autotune.py from
 // measurements on NVIDIA GB300 (2026-12-04 05:57 UTC); the library's defaults (pk_tuning_default).
-// Batch executor, 4096 knots at q = 3, split, one launch (median ms):
-//   threads  128  ktab   512     4.445
-//   threads  128  ktab  1024     4.501
-//   threads  128  ktab  2048     4.910
-//   threads  256  ktab   512     4.269
-//   threads  256  ktab  1024     4.312
-//   threads  256  ktab  2048     4.308
-//   threads  512  ktab   512     5.555
-//   threads  512  ktab  1024     5.578
-//   threads  512  ktab  2048     5.640
+// Batch executor, 4096 knots at q = 3, split, one launch (median ms; 2026-12-05, level records):
+//   threads  128  ktab   512     4.165
+//   threads  128  ktab  1024     4.228
+//   threads  128  ktab  2048     3.786
+//   threads  256  ktab   512     2.345
+//   threads  256  ktab  1024     2.359
+//   threads  256  ktab  2048     2.203
+//   threads  512  ktab   512     2.071
+//   threads  512  ktab  1024     1.919
+//   threads  512  ktab  2048     1.925
 // Level launches, single evaluations (us per call; 48 evaluations as one group last):
 //                                  q3 c128  q5 split  q3 c64  sliced split  grad q5 split  group
 //   outs <=  1024  work <=   65536    1346       877     441         37125            798   7839

@@ -10,9 +10,10 @@
 
 namespace pk {
 
-// Measured on GB300, whole evaluations: 330 crossings at q = 3 in complex64 1.17 -> 0.35 ms
-// and 167 crossings at q = 5 in split 1.71 -> 0.47 ms (with gemm_short.cuh) against one small step
-// after another in one CTA; the reverse pass of 99 crossings at q = 5 in split 2.11 -> 0.37 ms.  A level
+// Measured on GB300, whole calls of perf/cases.py against one small step after another in one CTA:
+// 330 crossings at q = 3 in complex64 1.17 -> 0.35 ms (0.27 to 0.35 by the over / under bits) and
+// 167 crossings at q = 5 in split 1.97 -> 0.47 ms (with gemm_short.cuh); the reverse pass of 99
+// crossings at q = 5 in split 2.09 -> 0.37 ms.  A level
 // of the cluster kernel takes 1.5 to 2 us: 0.16 us for an operand's round trip to L2, 0.3 us
 // for the cluster barrier, the rest one warp's 200 to 300 dependent instructions (FP64
 // multiply-adds: 63 cycles each).  A level launched alone takes 0.9 us more.

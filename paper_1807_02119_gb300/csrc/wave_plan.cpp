@@ -341,7 +341,7 @@ void wave_stages(const std::vector<Step>& steps, const pk_tuning& tune, int32_t 
     // runs at 2 multiply-adds per cycle and multiprocessor, 16 cycles per warp instruction, so
     // its levels spread over more multiprocessors, and leave the cluster, sooner.
     const int64_t per_cta = fp64 ? kWaveCtaWarps64 : kWaveCtaWarps32;
-    const int64_t fused_max = kWaveMaxCtas * per_cta * kWavePasses;
+    const int64_t fused_max = kWaveMaxCtas * per_cta;
     std::vector<WaveStage>& out = w.stages[fp64];
     out.clear();
     w.n_fused[fp64] = w.n_fused_steps[fp64] = 0;
