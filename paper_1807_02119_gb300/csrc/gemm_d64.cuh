@@ -65,7 +65,8 @@ constexpr int kBad = 1 << 28;                // exponent of a row with a non-fin
 constexpr int kSure = 8;
 constexpr int kListed = 2048, kListWarp = 24;   // small outputs a CTA leaves to its end, at most; of a warp's 128
 // An entry's marks: it reaches 2^-mark(j) of its row's largest entry (a column's: the marks in turn
-// from the last); a pair with a common mark has a product above 2^-(kSure + 2) of P.
+// from the last); a pair with a common mark has a product above 2^-(kSure + 2) of P.  A last mark
+// says that it is not 0 (below 2^-1042: as 0); without a pair of these the output is 0.
 constexpr int kMarks = 3;
 __device__ __forceinline__ constexpr int mark(int j) { return kSure / (kMarks - 1) * j; }
 static_assert(kS * kN <= 256 && kSmem <= 220 * 1024 && kFlush * kS * 2 * kKc < 1024, "tile geometry");
@@ -206,6 +207,7 @@ __device__ __forceinline__ void digits64_block(const Step& s, const Cx<double>* 
 #pragma unroll
         for (int j = 0; j < kMarks; ++j)
           if (top >= least[j]) m |= 1u << (8 * j + u);
+        if (top) m |= 1u << (8 * kMarks + u);
       }
       ((unsigned*)(scratch + (IS_A ? L.xa_off : L.xb_off)))[((bb * tiles + tile) * L.chunks + c) * kT + part * RB + r] = m;
     }
@@ -533,7 +535,7 @@ __global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const __grid_consta
       }
       // the tile, while the next one's products run
       Cx<double>* C = arena + s.off_c;
-      unsigned again = 0;   // outputs that are small against P
+      unsigned again = 0, bare = 0;   // outputs that are small against P; those without digits
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const long long cc = any ? ccp[j] : -1;
@@ -549,11 +551,13 @@ __global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const __grid_consta
           const int et = (int)(top >> 52);   // 0: zero, or below the normal range
           sure = sure || (et > 0 && et - 1023 >= x + 68 - kSure);
           vmax = max(vmax, top);
+        } else {
+          bare |= 1u << j;
         }
         if (!sure) again |= 1u << j;
         st(C + crow + cc, Cx<double>{__longlong_as_double((long long)re), __longlong_as_double((long long)im)});
       }
-      if (__any_sync(0xffffffffu, again)) {   // those with two entries that share a mark are kept
+      if (__any_sync(0xffffffffu, again)) {   // those with two entries that share a mark are kept, and zeros
         const unsigned* xa = (const unsigned*)(scratch + L.xa_off) + row * nchunks * kMc + quarter * 32 + lane;
         const uint4* xb = (const uint4*)(scratch + L.xb_off) + (bb * L.tiles_n + tn) * nchunks * (kNc / 4) + cq;
         uint4 hit = make_uint4(0, 0, 0, 0);
@@ -566,7 +570,8 @@ __global__ void __launch_bounds__(d64::kThreads, 1) k_gemm64(const __grid_consta
           hit.z |= a & b.z;
           hit.w |= a & b.w;
         }
-        again &= (hit.x == 0) | (hit.y == 0) << 1 | (hit.z == 0) << 2 | (hit.w == 0) << 3;
+        const auto open = [](unsigned h) { return h >> (8 * kMarks) && !(h << (32 - 8 * kMarks)) ? 1u : 0u; };
+        again &= open(hit.x) | open(hit.y) << 1 | open(hit.z) << 2 | open(hit.w) << 3 | bare;
         const int most = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(again));
         if (most > 0) {
           // few: left to the end of the CTA's tiles, where their chains of loads run side by side

@@ -56,6 +56,16 @@ def test_evaluate(ctx, q, L, seed, J):
     assert rel_err(sc(z), sc(zn)) <= bound(s["K"] for s in p.steps())
 
 
+@pytest.mark.parametrize("q,L,seed", [(5, 33, 21), (3, 40, 1)])
+def test_zeros(ctx, q, L, seed):
+    """Weights of 0 (colourings): outputs without a term are 0, not formed again."""
+    k = pk.Knot.from_grid_walk(ctx, L, seed, True, 60, 400)
+    w = [(d, 0j if i % 3 == 0 else o) if i % 5 else (0j, o) for i, (d, o) in enumerate(graded(k.info()["n_c"], 3, 1))]
+    p, pn = pk.Plan(ctx, k, q, weights=w), pk.Plan(ctx, k, q, weights=w, flags=pk.FLAG_NO_TC)
+    z, zn = pk.evaluate(p, "c128")[0], pk.evaluate(pn, "c128")[0]
+    assert zn.mantissa and rel_err(sc(z), sc(zn)) <= bound(s["K"] for s in p.steps())
+
+
 @pytest.mark.parametrize("J", [0, 20, 60])
 def test_recorded_launches_follow_new_weights(ctx, J):
     """A plan with the standard weights of q = 3, launched once, then given graded ones: Z, and
